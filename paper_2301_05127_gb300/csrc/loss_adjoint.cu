@@ -409,6 +409,11 @@ loss_status_t run_gradient(loss_ctx* h, Shot& s, const double* d_obs, int32_t ch
     ho = obs.data();
   }
   std::vector<double> gk[3];
+  struct Flag {  // (also reset when a call fails)
+    bool& f;
+    ~Flag() { f = false; }
+  } flag{h->in_gradient};
+  h->in_gradient = true;
   if (s.esize == 8) LOSS_TRY(gradient_t<double>(h, s, ho, C, n_steps, misfit, gk));
   else LOSS_TRY(gradient_t<float>(h, s, ho, C, n_steps, misfit, gk));
   // chain rule (FP64, dense): kappa = rho vp^2 | lambda = rho (vp^2 - 2 vs^2), mu = rho vs^2; b = 1 / rho

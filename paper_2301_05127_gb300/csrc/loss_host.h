@@ -43,6 +43,10 @@ struct Shot {
   void* tmp[8] = {};     // derivative temporaries (acoustic: tmp[0] = d_z v3)
   double* W[3] = {};     // PMBC weights per axis slot, scaled by h/3
   double* Wd[3] = {};     // junction-correction weights of the FP32 truncated-convolution kernels (on first use)
+  // axis tables of the barrier-free engines (conv_axis, on first use): double r^d, d < 64, ConvTap
+  // taps[ntaps], int js[p + 2]
+  void* conv_tab[3] = {};
+  int conv_Q[3] = {0, 0, 0}, conv_ntaps[3] = {0, 0, 0};
   void* nu_tab[3] = {};   // non-uniform axis slot (loss_set_coordinates): PMBC weights and elimination tables
   std::vector<double> coords[3];  // the knots loss_set_coordinates gave an axis slot (empty: equally spaced)
   bool has_model = false;
@@ -78,6 +82,8 @@ struct Shot {
   bool staggered = false;  // velocities hold v at t_step + dt/2 instead of t_step
   // model as given to loss_set_model (dense, FP64), for the chain rule of the misfit gradient
   std::vector<double> h_vp, h_vs, h_rho;
+  double* dmodel = nullptr;  // vp, rho, vs (elastic) on the device, from the first gradient on
+  bool dmodel_valid = false;
   // adjoint workspace (loss_gradient): adjoint fields, adjoint PML memory variables (same slots as psi/phi or
   // pmem), velocity residual arrays, FP64 gradients of (lambda or kappa, mu, b)
   void* lam[LOSS_NUM_FIELDS] = {};
@@ -97,9 +103,9 @@ struct BatchState {
   int* tile0 = nullptr;   // [2][n_shots + 1]: first tile of each shot, X then Z
   void* jobs = nullptr;   // GatherJob[pre jobs + post jobs]
   StepClock* clk = nullptr;
-  size_t cap_bytes[6] = {};  // allocated bytes of xtab, ztab, tile0, jobs, xptab, tztab
+  size_t cap_bytes[7] = {};  // allocated bytes of xtab, ztab, tile0, jobs, xptab, tztab, astab
   int clk_cap = 0;
-  std::vector<unsigned char> host[6];  // last uploaded contents of the same tables
+  std::vector<unsigned char> host[7];  // last uploaded contents of the same tables
   int xthreads = 0, zthreads = 0, xlogc = 0, zlogc = 0;
   size_t xsmem = 0, zsmem = 0;
   int xtiles = 0, ztiles = 0;
@@ -119,6 +125,11 @@ struct BatchState {
   bool conv = false;
   void* xptab = nullptr;  // XpShot[n_shots]
   void* tztab = nullptr;  // TzShot[2 n_shots]
+  // FP64 form on the barrier-free engines: job and block tables of the launches of a step
+  bool stream = false;
+  void* astab = nullptr;
+  AcBatchKind ask[8];
+  int64_t astab_version = 0;
   XpSmem xl{};
   int xpthreads = 0, xpgrid = 0, tztiles = 0;
   int tzthreads[2] = {0, 0}, tzlogc[2] = {4, 4}, tzgrid[2] = {0, 0};
@@ -160,6 +171,9 @@ struct loss_ctx {
   size_t stage_bytes = 0;
   int graph_steps = 0;   // > 0: steps are replayed from a captured CUDA graph of this many steps
   bool capturing = false;
+  // forward runs of loss_gradient: FP32 steps keep the tile, row and line kernels.  The gradient is an FP64 result, and
+  // these kernels' rounding is part of the gradients users compare and store.
+  bool in_gradient = false;
   lossk::BatchState batch;
   // launch accounting (loss_profile / loss_profile_read)
   int64_t launches[LOSS_NUM_KERNELS] = {};
@@ -220,10 +234,15 @@ struct LaunchScope {
 };
 
 // loss_step.cu
+// Axis slot k of a shot on the barrier-free engines (loss_stream.cuh): uploads its tables on first use; *ok = false
+// when the axis does not qualify.
+loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok);
+ColMap col_map(const loss_ctx* h, const Shot& s, int k, int64_t py, int64_t pz);  // strided lines, slot 0 or 1
+RowMap row_map(const loss_ctx* h, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec);  // rows along x
 loss_status_t step_shot(loss_ctx* h, Shot& s);
 loss_status_t unstagger(loss_ctx* h, Shot& s);
 loss_status_t stagger_shot(loss_ctx* h, Shot& s);
-bool batch_eligible(const loss_ctx* h);
+bool batch_eligible(loss_ctx* h);
 bool conv_z_used(const loss_ctx* h);  // some shot's FP32 step runs the convolution z tiles
 loss_status_t step_batched(loss_ctx* h, int64_t n_steps);
 void batch_release(loss_ctx* h);
@@ -274,10 +293,25 @@ size_t tile_smem_z(const TileGeom& t, int mode, int logc);
 template <bool KAHAN>
 cudaError_t launch_xt(const AcXArgs<float>& a, const TileGeom& t, cudaStream_t st);
 size_t xt_smem(const TileGeom& t);
+// loss_kernels_acstream.cu: 2-D acoustic step on the barrier-free engines
+template <typename T, bool KAHAN>
+cudaError_t launch_ac_rows(const AcXArgs<T>& a, const ConvAxis& g, const RowMap& rm, cudaStream_t st);
+cudaError_t launch_ac_cols(const AcZArgs<double>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st);
+void ac_batch_tables(const std::vector<AcStreamShot>& shots, std::vector<unsigned char>& bytes, AcBatchKind (&k)[8]);
+cudaError_t launch_ac_batch(const void* base, const AcBatchKind& k, int kind, cudaStream_t st);
+// Blocks of a k_row launch (4 warps each, kblocks resident per SM).
+inline int row_blocks(const RowMap& rm, int kblocks) {
+  const int need = (rm.groups * rm.nwin + 3) / 4, most = rm.sms * kblocks;
+  return need < most ? need : most;
+}
 // loss_kernels_elastic.cu: elastic y / z tile passes (FP32)
 size_t elt_smem(const ElTile& g, int logc);
 template <bool KAHAN>
 cudaError_t launch_elt(const ElArgs<float>& a, const ElTile& g, int pass, int logc, cudaStream_t st);
+// loss_kernels_stream.cu: elastic passes on the barrier-free engines
+template <typename T, bool KAHAN>
+cudaError_t launch_el_stream(const ElArgs<T>& a, const ConvAxis& g, const ColMap& cm, const RowMap& rm, int pass,
+                             cudaStream_t st);
 size_t xp_smem(const TileGeom& t, bool kahan);
 int xp_rows_per_unit(int n, int threads);
 XpSmem xp_batch_layout(const std::vector<TileGeom>& ts, const std::vector<int>& rs, bool kahan);
@@ -291,6 +325,11 @@ cudaError_t launch_tz_batch(const TzShot* tab, const int* tile0, int nshots, int
                             int logc, size_t smem, int grid, cudaStream_t st);
 template <bool KAHAN>
 cudaError_t tz_batch_per_sm(int mode, int threads, int logc, size_t smem, int* per_sm);
+constexpr int kMisfitBlocks = 512;
+template <typename T>
+cudaError_t launch_residual(const T* tr, const double* obs, double* res, double* part, int64_t n, cudaStream_t st);
+cudaError_t launch_chain(const double* g0, const double* g1, const double* g2, const double* model, int elastic,
+                         int64_t n, int64_t nx, int64_t px, double* out, int num_sms, cudaStream_t st);
 template <typename T>
 cudaError_t launch_adj(const AdjArgs<T>& a, int logc, bool sflav, int threads, cudaStream_t st);
 template <typename T>

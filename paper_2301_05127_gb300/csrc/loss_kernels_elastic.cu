@@ -16,6 +16,7 @@
 
 #include "../../include/loss.h"
 #include "loss_block.cuh"
+#include "loss_elastic.cuh"
 #include "loss_fir.cuh"
 #include "loss_line.cuh"
 #include "loss_tile.cuh"
@@ -26,38 +27,6 @@ namespace lossk {
 enum { EL_BX = 0, EL_BY = 1, EL_BZ = 2, EL_AX = 3, EL_AY = 4 };
 
 size_t smem_bytes(const LineGeom& g, int nbuf, int nstage, size_t esize);  // loss_kernels_acoustic.cu
-
-// tau times the (stretched) derivative g along this pass's axis at line position pos.
-template <typename T>
-__device__ __forceinline__ T eff(int pml, const PmlAxis<T>& pa, T* mem, int64_t gi, int pos, T g, T tau, T tau_lo) {
-  return (pml && pa.in(pos)) ? -pa.step(mem, gi, pos, g) : mulc(g, tau, tau_lo);
-}
-
-// Velocity-sub-step term: returns tau * (stretched derivative); in a layer with receiver corrections on, also
-// stores b (X(tau/2) - X(tau)/2), the amount by which the first half of the step differs from half of it.
-template <typename T>
-__device__ __forceinline__ T effA(const ElArgs<T>& a, int term, int64_t gi, int pos, T g, T tau) {
-  if (!(a.pml && a.pA.in(pos))) return mulc(g, tau, a.acoef_lo);
-  T xh = T(0);
-  const bool rec = a.dlt[term] != nullptr;
-  if (rec) xh = -a.pA.half(a.memA[term], gi, pos, g);
-  const T xf = -a.pA.step(a.memA[term], gi, pos, g);
-  if (rec) a.dlt[term][gi] = (a.b ? a.b[gi] : a.b0) * (xh - T(0.5) * xf);
-  return xf;
-}
-
-// u += delta in registers (compensated with c when KAHAN); the caller loads and stores.
-template <typename T, bool KAHAN>
-__device__ __forceinline__ void upd_r(T& u, T& c, T delta) {
-  if constexpr (KAHAN) {
-    float cc = c;
-    kahan_add(u, cc, delta);
-    c = cc;
-  } else {
-    u += delta;
-  }
-}
-
 
 template <typename T, int LOGC, bool SFLAV, int PASS, bool KAHAN>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? 512 : 1024) k_el(ElArgs<T> a) {
@@ -250,7 +219,8 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 512 : 1024) k_el(ElArgs<T> a)
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// y and z passes of the FP32 step on one-patch tiles, in the truncated-convolution form of loss_fir.cuh (the 2-D z
+// y and z passes of the FP32 step on one-patch tiles (axes the barrier-free engines do not take, and the forward runs of
+// the misfit gradient), in the truncated-convolution form of loss_fir.cuh (the 2-D z
 // tiles' arithmetic): a block takes 32 neighbouring x columns by one patch of the pass axis plus a halo of
 // H = max(n_nb, K) positions on each side, for one index of the remaining axis.  It stages the pass's three source
 // fields (128-byte row segments), forms the FP64 junction corrections of the patch's two junctions for each field,

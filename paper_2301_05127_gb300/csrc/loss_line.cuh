@@ -91,7 +91,8 @@ struct Tab<double> {
 // removes.
 template <typename T>
 __device__ __forceinline__ T mulc(T x, T c, T c_lo) {
-  return fma(c_lo, x, c * x);
+  if constexpr (sizeof(T) == 8) return c * x;  // c_lo = 0: one FP64 operation less
+  else return fma(c_lo, x, c * x);
 }
 
 // FP32 -> FP64 widening on the integer units (IEEE 754: binary32 exponent bias 127, binary64 bias 1023, the 23

@@ -4,6 +4,7 @@
 // to the integer time level (v_n = v_{n+1/2} + dt/2 b grad sigma_n) whenever velocities are read.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -17,6 +18,8 @@ namespace lossk {
     loss_status_t st_ = (expr);     \
     if (st_ != LOSS_OK) return st_; \
   } while (0)
+
+constexpr double kConvRHost = -0.26794919243112270647;  // sqrt(3) - 2
 
 static double ricker(double t, double f0, double t0) {
   const double a = (M_PI * f0 * (t - t0)) * (M_PI * f0 * (t - t0));
@@ -209,8 +212,60 @@ static bool xp_ok(const loss_ctx* h, const Shot& s, const TileGeom& t) {
          xp_smem(t, s.kahan) + 2048 <= (size_t)h->smem_optin;
 }
 
+// Arguments with the engines' derivative scale 3 a / h (they return e / a).
+template <class A>
+static void conv_scale(A& a, const Shot& s, int k) {
+  using T = decltype(a.s3h);
+  const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k];
+  a.s3h = (T)sc;
+  a.s3h_lo = lo_part<T>(sc);
+}
+// A 2-D shot's arrays are within the engines' 32-bit byte offsets and row counts.
+static bool conv_size_ok(const Shot& s) {
+  return (uint64_t)s.total * s.esize <= UINT32_MAX && s.len[0] * ((s.n[2] + 191) / 192) < INT32_MAX / 2;
+}
+
+// The FP64 step of a 2-D acoustic shot on the barrier-free engines (the convolution family, axes that qualify).  The
+// line kernels' limits on the length of lines stay the limits of the step.
+static loss_status_t acs_ok(loss_ctx* h, Shot& s, bool* ok) {
+  *ok = false;
+  if (!h->tiled || s.esize != 8 || s.dim != 2 || s.d.physics != LOSS_ACOUSTIC || !conv_size_ok(s)) return LOSS_OK;
+  for (int k : {0, 2}) {
+    ConvAxis g;
+    LOSS_TRY(conv_axis(h, s, k, &g, ok));
+    if (!*ok) return LOSS_OK;
+    LineGeom lg;
+    int logc, threads;
+    LOSS_TRY(line_geom(h, s, k, s.sz, s.sy, &lg, &logc, &threads, k == 2 ? 3 : 2, k == 2 ? 4 : 0, 0, 0, 0));
+  }
+  return LOSS_OK;
+}
+
+// Rows on the engines: sub-step B (do_B) and the x part of A.
+template <typename T, bool K>
+static loss_status_t acs_rows(loss_ctx* h, Shot& s, int do_B, double acoef, double amp) {
+  ConvAxis g;
+  bool ok;
+  LOSS_TRY(conv_axis(h, s, 2, &g, &ok));
+  AcXArgs<T> a = ac_x_args<T>(h, s, LineGeom{}, do_B, acoef, amp);
+  conv_scale(a, s, 2);
+  LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
+  return cuda_check(h, launch_ac_rows<T, K>(a, g, row_map(h, s, 1, g, s.sy, s.sz, true), h->stream), "acoustic x kernel");
+}
+// Z1 (mode 1) or Z2 (mode 2) of the FP64 step on the engines.
+static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
+  ConvAxis g;
+  bool ok;
+  LOSS_TRY(conv_axis(h, s, 0, &g, &ok));
+  AcZArgs<double> a = ac_z_args<double>(h, s, LineGeom{}, acoef, 0);
+  conv_scale(a, s, 0);
+  LaunchScope ls(h, mode == 1 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2);
+  return cuda_check(h, launch_ac_cols(a, g, col_map(h, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
+}
+
 // x part of the FP32 step (sub-step B and the x part of A, or the latter alone): the pipelined row kernel when a
-// row fits its shared-memory stages, else the (row, patch) item kernels, two launches.
+// row fits its shared-memory stages; else the row engine; else (and in the forward runs of a gradient, and for the
+// family that asks for them) the (row, patch) item kernels, two launches.
 template <bool K>
 static loss_status_t xpart(loss_ctx* h, Shot& s, int do_B, double acoef, double amp) {
   int threads;
@@ -218,6 +273,13 @@ static loss_status_t xpart(loss_ctx* h, Shot& s, int do_B, double acoef, double 
   LOSS_TRY(ensure_delta_weights(h, s, 2));
   t.Wd = s.Wd[2];
   t.ncross = (int)s.len[0];
+  if (!xp_ok(h, s, t) && h->tiled != LOSS_KERNELS_CONVOLUTION_ITEMS && !h->in_gradient && conv_size_ok(s) &&
+      xt_smem(t) <= (size_t)h->smem_optin) {
+    ConvAxis g;
+    bool ok;
+    LOSS_TRY(conv_axis(h, s, 2, &g, &ok));
+    if (ok) return acs_rows<float, K>(h, s, do_B, acoef, amp);
+  }
   const AcXArgs<float> a = ac_x_args<float>(h, s, LineGeom{}, do_B, acoef, amp);
   LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
   if (xp_ok(h, s, t)) {
@@ -289,6 +351,13 @@ static loss_status_t acoustic2d_start(loss_ctx* h, Shot& s) {
     LOSS_TRY(tz<K>(h, s, 1, 0.5 * dt));
     return tz<K>(h, s, 2, 0.0);
   }
+  bool stream;
+  LOSS_TRY(acs_ok(h, s, &stream));
+  if (stream) {
+    LOSS_TRY((acs_rows<T, K>(h, s, 0, 0.5 * dt, 0.0)));
+    LOSS_TRY(acs_cols(h, s, 1, 0.5 * dt));
+    return acs_cols(h, s, 2, 0.0);
+  }
   LOSS_TRY((ac_x<T, K>(h, s, 0, 0.5 * dt, 0.0)));
   return ac_z<T, K>(h, s, 0.5 * dt, 1);
 }
@@ -318,7 +387,10 @@ static loss_status_t acoustic2d_step(loss_ctx* h, Shot& s) {
   }
   LOSS_TRY(gather_fields<T>(h, s, true, 0));  // v at t_{n+1/2}
   const bool conv = sizeof(T) == 4 && tiled_ok(h, s);
+  bool stream;
+  LOSS_TRY(acs_ok(h, s, &stream));
   if (conv) LOSS_TRY(xpart<K>(h, s, 1, dt, pressure_amp(s, s.step)));
+  else if (stream) LOSS_TRY((acs_rows<T, K>(h, s, 1, dt, pressure_amp(s, s.step))));
   else LOSS_TRY((ac_x<T, K>(h, s, 1, dt, pressure_amp(s, s.step))));
   bool side = false;
   if (s.n_rcv) {
@@ -329,6 +401,9 @@ static loss_status_t acoustic2d_step(loss_ctx* h, Shot& s) {
   if (conv) {
     LOSS_TRY(tz<K>(h, s, 1, dt));
     LOSS_TRY(tz<K>(h, s, 2, 0.0));
+  } else if (stream) {
+    LOSS_TRY(acs_cols(h, s, 1, dt));
+    LOSS_TRY(acs_cols(h, s, 2, 0.0));
   } else {
     LOSS_TRY((ac_z<T, K>(h, s, dt, 1)));
   }
@@ -348,6 +423,14 @@ static loss_status_t acoustic2d_unstagger(loss_ctx* h, Shot& s) {
     s.staggered = false;
     return LOSS_OK;
   }
+  bool stream;
+  LOSS_TRY(acs_ok(h, s, &stream));
+  if (stream) {
+    LOSS_TRY((acs_rows<T, K>(h, s, 0, -0.5 * dt, 0.0)));
+    LOSS_TRY(acs_cols(h, s, 1, -0.5 * dt));
+    s.staggered = false;
+    return LOSS_OK;
+  }
   LOSS_TRY((ac_x<T, K>(h, s, 0, -0.5 * dt, 0.0)));
   LOSS_TRY((ac_z<T, K>(h, s, -0.5 * dt, 0)));
   s.staggered = false;
@@ -356,7 +439,8 @@ static loss_status_t acoustic2d_unstagger(loss_ctx* h, Shot& s) {
 
 
 // ---------------------------------------------------------------------------------------------------------------
-// 3-D elastic: five line passes per step (loss_kernels_elastic.cu).
+// 3-D elastic: six passes per step on the barrier-free engines (loss_kernels_stream.cu), or five line passes
+// (loss_kernels_elastic.cu).
 enum { EL_BX = 0, EL_BY = 1, EL_BZ = 2, EL_AX = 3, EL_AY = 4 };
 
 // Arguments of an elastic pass along axis slot k that do not depend on its launch shape.
@@ -456,6 +540,140 @@ static loss_status_t elt_pass(loss_ctx* h, Shot& s, int pass, double acoef, doub
   return cuda_check(h, launch_elt<K>(a, g, pass, elt_logc(s, k), h->stream), "elastic tile kernel");
 }
 
+// ---------------------------------------------------------------------------------------------------------------
+// Axes of the barrier-free engines (loss_stream.cuh).
+loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok) {
+  const int n = (int)s.n[k], p = s.p[k], M = n / p;
+  *ok = false;
+  if (n < 40) return LOSS_OK;  // the line ends' closed forms need whole warm-up sums beside them
+  if (!s.conv_tab[k]) {
+    const bool f32 = s.esize == 4;
+    const int K = f32 ? 16 : 32;
+    const int R = std::max(s.d.n_nb, K), wl = 2 * R + 1;
+    const std::vector<double> D = fir_delta_weights(n, p, s.d.n_nb, K);
+    const double a = fir_const(M).a;
+    // weights that are rounding noise of the difference (or reach less than the last digit) are left out
+    const double tiny = f32 ? 0x1p-44 : 0x1p-52;
+    std::vector<int> js(p + 2, 0);
+    std::vector<ConvTap> taps;
+    double dmax = 0.0;
+    for (int j = 0; j <= p; ++j) {
+      js[j] = (int)taps.size();
+      double sum = 0.0;
+      for (int m = -R; m <= R; ++m) {
+        const double w = D[(size_t)j * wl + R + m];
+        if (std::fabs(w) <= tiny) continue;
+        taps.push_back(ConvTap{w / a, m, 0});
+        sum += std::fabs(w) / a;
+      }
+      dmax = std::max(dmax, sum);
+    }
+    js[p + 1] = (int)taps.size();
+    // reach of a correction: |r|^Q dmax below the working precision
+    const double eps = f32 ? 0x1p-40 : 0x1p-58;
+    int Q = 0;
+    for (double q = dmax; q > eps && Q < 64; q *= -kConvRHost) ++Q;
+    const size_t o1 = 64 * sizeof(double), o2 = o1 + taps.size() * sizeof(ConvTap);
+    std::vector<unsigned char> blob(o2 + js.size() * sizeof(int));
+    double pw[64];
+    pw[0] = 1.0;
+    for (int i = 1; i < 64; ++i) pw[i] = pw[i - 1] * kConvRHost;
+    std::memcpy(blob.data(), pw, sizeof(pw));
+    if (!taps.empty()) std::memcpy(blob.data() + o1, taps.data(), taps.size() * sizeof(ConvTap));
+    std::memcpy(blob.data() + o2, js.data(), js.size() * sizeof(int));
+    void* d = nullptr;
+    LOSS_TRY(dev_alloc(h, blob.size(), &d));
+    LOSS_TRY(cuda_check(h, cudaMemcpyAsync(d, blob.data(), blob.size(), cudaMemcpyHostToDevice, h->stream),
+                        "copy junction taps"));
+    LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
+    s.conv_tab[k] = d;
+    s.conv_Q[k] = Q;
+    s.conv_ntaps[k] = (int)taps.size();
+  }
+  g->n = n, g->p = p, g->M = M, g->Q = s.conv_Q[k], g->ntaps = s.conv_ntaps[k];
+  g->pw = (const double*)s.conv_tab[k];
+  g->taps = (const ConvTap*)(g->pw + 64);
+  g->js = (const int*)(g->taps + g->ntaps);
+  *ok = M >= g->Q + 8 && g->Q < 64;
+  return LOSS_OK;
+}
+
+// Strided lines of an array with row pitch py and plane pitch pz.  A line is cut into segments when there are too few
+// lines to fill the GPU (about 16 warps per SM); a segment re-reads K positions before it and 8 (W + 1) after it, so
+// it keeps at least 40 positions.
+ColMap col_map(const loss_ctx* h, const Shot& s, int k, int64_t py, int64_t pz) {
+  ColMap m{};
+  m.inner = s.len[2];
+  m.lines = s.dense / s.len[k];
+  m.groups = (m.lines + 31) / 32;
+  m.so = k == 1 ? pz : py;
+  m.stride = k == 1 ? py : pz;
+  const int64_t want = 16LL * h->num_sms;
+  const int np = (int)s.n[k] + 1;
+  const int nseg = (int)std::min<int64_t>(std::max<int64_t>(want / m.groups, 1), std::max(np / 40, 1));
+  m.seglen = ((np + nseg - 1) / nseg + 7) & ~7;
+  m.nseg = (np + m.seglen - 1) / m.seglen;
+  return m;
+}
+
+RowMap row_map(const loss_ctx* h, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec) {
+  RowMap m{};
+  const int es = (int)s.esize, W = es == 4 ? 2 : 4;
+  m.rows = (int)(s.len[0] * s.len[1]);
+  m.ny = (int)s.len[1];
+  m.sy = py;
+  m.sz = pz;
+  m.nch = g.n % 8 == 0 ? g.n / 8 : g.n / 8 + 1;
+  m.gw = 8;
+  while (m.gw < 32 && m.gw < m.nch) m.gw *= 2;
+  m.nwin = m.nch <= 32 ? 1 : 1 + (m.nch - 32 + 31 - 2 * W) / (32 - 2 * W);
+  m.groups = (m.rows + 32 / m.gw - 1) / (32 / m.gw);
+  m.vec = vec ? 1 : 0;
+  const int nj = std::min(g.p + 1, (8 * m.gw + 1 + 2 * g.Q) / g.M + 2);
+  m.wbytes = (nf * (32 / m.gw) * nj * es + 15) & ~15;
+  m.sms = h->num_sms;
+  return m;
+}
+
+// The elastic step on those engines: the convolution family (loss_set_kernels) when every axis qualifies.  The line
+// kernels' limit on the length of a row stays the limit of the step.
+template <typename T>
+static loss_status_t els_ok(loss_ctx* h, Shot& s, bool* ok) {
+  *ok = false;
+  if (!h->tiled || s.dim != 3 || (s.esize == 4 && h->in_gradient)) return LOSS_OK;
+  if ((uint64_t)s.total * s.esize > UINT32_MAX) return LOSS_OK;  // the engines use 32-bit byte offsets
+  for (int k = 0; k < 3; ++k) {
+    ConvAxis g;
+    LOSS_TRY(conv_axis(h, s, k, &g, ok));
+    if (!*ok) return LOSS_OK;
+    LineGeom lg;
+    int logc, threads;
+    if (k == 2 && s.len[0] * s.len[1] * ((g.n + 223) / 224) > INT32_MAX / 2) return *ok = false, LOSS_OK;
+    if (k == 2 || s.esize == 8) LOSS_TRY(line_geom(h, s, k, s.sz, s.sy, &lg, &logc, &threads, 6, 0, 0, 0, 0));
+  }
+  return LOSS_OK;
+}
+
+template <typename T, bool K>
+static loss_status_t els_pass(loss_ctx* h, Shot& s, int pass, double acoef, double amp) {
+  const int k = (pass == ES_BX || pass == ES_AX) ? 2 : ((pass == ES_BY || pass == ES_AY) ? 1 : 0);
+  const bool B = pass == ES_BX || pass == ES_BY || pass == ES_BZ;
+  const int src = B ? 0 : (pass == ES_AZ ? 1 : (pass == ES_AX ? 2 : 3));
+  ElArgs<T> a = el_args<T>(h, s, k, src, B ? 1 : 0, B ? 0 : 1, acoef, amp);
+  const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k];  // the engines return e / a
+  a.s3h = (T)sc;
+  a.s3h_lo = lo_part<T>(sc);
+  ConvAxis g;
+  bool ok;
+  LOSS_TRY(conv_axis(h, s, k, &g, &ok));
+  ColMap cm{};
+  RowMap rm{};
+  if (k == 2) rm = row_map(h, s, 3, g, s.sy, s.sz, true);
+  else cm = col_map(h, s, k, s.sy, s.sz);
+  LaunchScope ls(h, k == 2 ? LOSS_KERNEL_ELASTIC_X : (k == 1 ? LOSS_KERNEL_ELASTIC_Y : LOSS_KERNEL_ELASTIC_Z));
+  return cuda_check(h, launch_el_stream<T, K>(a, g, cm, rm, pass, h->stream), "elastic kernel");
+}
+
 template <typename T, bool K>
 static loss_status_t el_pass(loss_ctx* h, Shot& s, int pass, int do_B, int do_A, double acoef, double amp) {
   // internal axis slot of the pass: x = 2, y = 1, z = 0
@@ -491,6 +709,13 @@ template <typename T, bool K>
 static loss_status_t elastic_A(loss_ctx* h, Shot& s, double tau, double force_t) {
   double famp = 0.0;
   if (s.src_on && (s.src_kinds & kForceMask)) famp = tau * s.src_norm * ricker(force_t, s.src_f0, s.src_t0);
+  bool conv;
+  LOSS_TRY(els_ok<T>(h, s, &conv));
+  if (conv) {
+    LOSS_TRY((els_pass<T, K>(h, s, ES_AZ, tau, 0.0)));
+    LOSS_TRY((els_pass<T, K>(h, s, ES_AX, tau, 0.0)));
+    return els_pass<T, K>(h, s, ES_AY, tau, famp);
+  }
   if (sizeof(T) == 4 && elt_ok(h, s)) {
     LOSS_TRY((elt_pass<K>(h, s, ET_AZ, tau, 0.0)));
     LOSS_TRY((el_pass<T, K>(h, s, EL_AX, 0, 1, tau, 0.0)));
@@ -516,7 +741,12 @@ static loss_status_t elastic3d_step(loss_ctx* h, Shot& s) {
     amp = dt * s.src_norm * ricker(tn + 0.5 * dt, s.src_f0, s.src_t0);
   double famp = 0.0;
   if (s.src_on && (s.src_kinds & kForceMask)) famp = dt * s.src_norm * ricker(tn + dt, s.src_f0, s.src_t0);
-  if (sizeof(T) == 4 && elt_ok(h, s)) {
+  bool conv;
+  LOSS_TRY(els_ok<T>(h, s, &conv));
+  if (conv) {
+    for (int pass : {ES_BX, ES_BY, ES_BZ, ES_AZ, ES_AX, ES_AY})
+      LOSS_TRY((els_pass<T, K>(h, s, pass, dt, pass == ES_BZ ? amp : (pass == ES_AY ? famp : 0.0))));
+  } else if (sizeof(T) == 4 && elt_ok(h, s)) {
     LOSS_TRY((el_pass<T, K>(h, s, EL_BX, 1, 0, dt, 0.0)));
     LOSS_TRY((elt_pass<K>(h, s, ET_BY, dt, 0.0)));
     LOSS_TRY((elt_pass<K>(h, s, ET_BZ, dt, amp)));
@@ -553,7 +783,7 @@ static loss_status_t elastic3d_unstagger(loss_ctx* h, Shot& s) {
 
 static bool conv_batch_ok(const loss_ctx* h);
 
-bool batch_eligible(const loss_ctx* h) {
+bool batch_eligible(loss_ctx* h) {
   if (h->shots.empty()) return false;
   if (!(h->graph_steps > 0 || (h->batched && h->shots.size() > 1))) return false;
   const Shot& s0 = h->shots[0];
@@ -566,6 +796,16 @@ bool batch_eligible(const loss_ctx* h) {
   if (s0.esize == 4 && !conv_batch_ok(h))
     for (const Shot& s : h->shots)
       if (s.n[2] > 2048) return false;
+  // FP64: the batch takes the engines or the line kernels for all shots; handles that mix the two go per shot
+  if (s0.esize == 8) {
+    int n = 0;
+    for (Shot& s : h->shots) {
+      bool ok = false;
+      acs_ok(h, s, &ok);
+      n += ok ? 1 : 0;
+    }
+    if (n != 0 && n != (int)h->shots.size()) return false;
+  }
   return true;
 }
 
@@ -701,6 +941,22 @@ static loss_status_t batch_launch_step(loss_ctx* h) {
       LaunchScope ls(h, LOSS_KERNEL_CLOCK);
       return cuda_check(h, launch_tick(B.clk, S, h->stream), "clock tick");
     }
+  }
+  if (B.stream) {
+    const int kid[8] = {LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_X,
+                        LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_Z, LOSS_KERNEL_ACOUSTIC_Z, LOSS_KERNEL_ACOUSTIC_Z2};
+    for (int k = 0; k < 8; ++k) {
+      if (B.ask[k].blocks == 0) continue;
+      LaunchScope ls(h, kid[k]);
+      LOSS_TRY(cuda_check(h, launch_ac_batch(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
+    }
+    if (B.npost) {
+      LaunchScope ls(h, LOSS_KERNEL_GATHER);
+      LOSS_TRY(cuda_check(h, launch_gather_batch<T>(jobs + B.npre, B.npost, B.post_max, h->stream),
+                          "batched receiver gather"));
+    }
+    LaunchScope ls(h, LOSS_KERNEL_CLOCK);
+    return cuda_check(h, launch_tick(B.clk, S, h->stream), "clock tick");
   }
   {
     LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
@@ -885,18 +1141,51 @@ static loss_status_t conv_tables(loss_ctx* h) {
   return LOSS_OK;
 }
 
+// Tables of the batched FP64 step on the engines.
+static loss_status_t acs_tables(loss_ctx* h) {
+  BatchState& B = h->batch;
+  std::vector<AcStreamShot> v;
+  for (size_t i = 0; i < h->shots.size(); ++i) {
+    Shot& s = h->shots[i];
+    AcStreamShot q{};
+    bool ok;
+    LOSS_TRY(conv_axis(h, s, 2, &q.gx, &ok));
+    LOSS_TRY(conv_axis(h, s, 0, &q.gz, &ok));
+    q.rm = row_map(h, s, 1, q.gx, s.sy, s.sz, true);
+    q.cm = col_map(h, s, 0, s.sy, s.sz);
+    q.x = ac_x_args<double>(h, s, LineGeom{}, 1, s.d.dt, 0.0);
+    q.x.src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
+    q.x.src.amp_tab = s.amp_tab;
+    q.x.src.clk = B.clk + i;
+    conv_scale(q.x, s, 2);
+    q.z = ac_z_args<double>(h, s, LineGeom{}, s.d.dt, 0);
+    conv_scale(q.z, s, 0);
+    v.push_back(q);
+  }
+  std::vector<unsigned char> bytes;
+  ac_batch_tables(v, bytes, B.ask);
+  if (bytes != B.host[6]) ++B.astab_version;  // the launch shapes may differ with the contents: capture again
+  return upload_table(h, 6, bytes, &B.astab);
+}
+
 template <typename T, bool K>
 static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   BatchState& B = h->batch;
   const int S = (int)h->shots.size();
   B.conv = false;
   if constexpr (sizeof(T) == 4) B.conv = conv_batch_ok(h);
+  B.stream = sizeof(T) == 8;  // every FP64 shot on the engines (batch_eligible leaves mixed handles per shot)
+  for (Shot& s : h->shots) {
+    bool ok = false;
+    if (B.stream) LOSS_TRY(acs_ok(h, s, &ok));
+    B.stream = B.stream && ok;
+  }
   // per-shot preparation: receiver corrections, staggered start (that of the per-shot schedule of the same
   // kernels), source amplitudes
   for (Shot& s : h->shots) {
     LOSS_TRY(ensure_rdelta(h, s));
     if (!s.staggered) {
-      if (B.conv) {
+      if (B.conv || B.stream) {
         LOSS_TRY((acoustic2d_start<T, K>(h, s)));
       } else {
         LOSS_TRY((ac_x<T, K>(h, s, 0, 0.5 * s.d.dt, 0.0)));
@@ -908,7 +1197,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   }
   // launch shapes and descriptors
   std::vector<LineGeom> gx, gz;
-  if (!B.conv) {
+  if (!B.conv && !B.stream) {
     LOSS_TRY(batch_geoms(h, 2, LOSS_KERNEL_ACOUSTIC_X, 3, 4, gx, &B.xlogc, &B.xthreads, &B.xsmem));
     LOSS_TRY(batch_geoms(h, 0, LOSS_KERNEL_ACOUSTIC_Z, 2, 0, gz, &B.zlogc, &B.zthreads, &B.zsmem));
   }
@@ -927,7 +1216,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   int64_t pre_max = 0, post_max = 0;
   for (int i = 0; i < S; ++i) {
     Shot& s = h->shots[i];
-    if (!B.conv) {
+    if (!B.conv && !B.stream) {
       xa[i] = ac_x_args<T>(h, s, gx[i], 1, s.d.dt, 0.0);
       xa[i].src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
       xa[i].src.amp_tab = s.amp_tab;
@@ -972,6 +1261,8 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   jobs.insert(jobs.end(), post.begin(), post.end());
   if (B.conv) {
     if constexpr (sizeof(T) == 4) LOSS_TRY(conv_tables<K>(h));
+  } else if (B.stream) {
+    LOSS_TRY(acs_tables(h));
   } else {
     LOSS_TRY(upload_table(h, 0, as_bytes(xa), &B.xtab));
     LOSS_TRY(upload_table(h, 1, as_bytes(za), &B.ztab));
@@ -990,7 +1281,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
                         "upload clocks"));
     LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
   }
-  if (!B.conv) {
+  if (!B.conv && !B.stream) {
     LOSS_TRY(cuda_check(h, batch_grid_ac_x<T, K>(B.xlogc, B.xthreads, B.xsmem, B.xtiles, h->num_sms, &B.xgrid),
                         "batched x kernel shape"));
     LOSS_TRY(cuda_check(h, batch_grid_ac_z<T, K>(B.zlogc, B.zthreads, B.zsmem, B.ztiles, h->num_sms, &B.zgrid),
@@ -1008,7 +1299,8 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
                                       (int64_t)(intptr_t)B.xptab, (int64_t)(intptr_t)B.tztab, B.xpgrid, B.xpthreads,
                                       B.xl.total, B.tzthreads[0], B.tzthreads[1], B.tzlogc[0], B.tzlogc[1],
                                       B.tztiles, B.tzgrid[0], B.tzgrid[1],
-                                      (int64_t)B.tzsmem[0], (int64_t)B.tzsmem[1], (int64_t)h->wait_polls};
+                                      (int64_t)B.tzsmem[0], (int64_t)B.tzsmem[1], (int64_t)h->wait_polls,
+                                      B.stream ? 1 : 0, (int64_t)(intptr_t)B.astab, B.astab_version};
     if (!B.gexec || sig != B.gsig) {
       LOSS_TRY((capture_graph<T, K>(h, k)));
       B.gsig = sig;

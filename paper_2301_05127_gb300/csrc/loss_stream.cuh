@@ -1,0 +1,577 @@
+// Barrier-free engines of the truncated-convolution form (loss_fir.cuh) of the LOSS derivative, FP32 and FP64.
+//
+// Both evaluate  e_i = (R_i - L_i) + sum_j D_j r^|i - jM|  (the scaled derivative over a; the caller multiplies by
+// 3 a / h) with warps that never wait for one another:
+//   - k_col: lines along a strided axis.  One thread per line, 32 neighbouring lines per warp; a thread marches along
+//     its line in chunks of 8 positions.  Its samples pass through a ring of chunks in shared memory that the thread
+//     fills with cp.async and reads alone, so every sample is read from global memory once and no barrier is needed.
+//   - k_row: lines along the contiguous axis.  A warp (or 8 or 16 lanes of it, for short rows) takes up to 32 chunks of
+//     8 positions of a row, one chunk per lane, staged in the warp's own shared memory; the warm-up sums of a
+//     chunk come from its neighbour lanes by shuffles.
+//
+// Recursions start from sums over W whole neighbour chunks (16 terms in FP32, 32 in FP64: |r|^16 = 7e-10, |r|^32 =
+// 5e-19), or, beyond a line's end, from the closed form of the odd reflection f_{-k} = 2 f_0 - f_k:
+// L_0 = 2 f_0 / (1 - r) - R_0 and R_n = 2 f_n / (1 - r) - L_n.
+//
+// Junction corrections.  D_j = sum_m w_jm f_{jM + m} in FP64.  Away from the line ends the PMBC weights equal the
+// convolution's own weights term by term up to min(n_nb, K) (both are the Toeplitz inverse), so all but the outer
+// taps of a row vanish up to the rounding of their difference; the host keeps the taps that do not (ConvAxis::taps,
+// 8 instead of 41 per junction at n_nb = 20, K = 16).  A correction reaches Q positions, where |r|^Q |D| is
+// below the working precision (host rule conv_axis in loss_step.cu); longer patches make the second term of the
+// patch-end correction, r^M D, vanish by the same rule.
+#pragma once
+
+#include <cstdint>
+#include <type_traits>
+#include <cuda_runtime.h>
+
+#include "loss_fir.cuh"
+#include "loss_line.cuh"
+#include "loss_types.h"
+
+namespace lossk {
+
+// Powers of r = sqrt(3) - 2 and 2 / (1 - r) in the working precision.
+constexpr double kConvR = -0.26794919243112270647255365849413;
+constexpr double conv_pow(int k) { return k == 0 ? 1.0 : kConvR * conv_pow(k - 1); }
+template <typename T>
+struct Conv {
+  static constexpr int W = sizeof(T) == 4 ? 2 : 4;  // neighbour chunks of a warm-up sum
+  static constexpr int K = 8 * W;
+};
+
+// Weights of a junction's correction at distance d: rs[64 + d] = r^|d| for |d| <= Q, 0 beyond, d = -64 .. 79, in
+// shared memory (no barrier).
+constexpr int kReach = 144;
+template <typename T>
+__device__ __forceinline__ void fill_reach(T* rs, const ConvAxis& g) {
+  for (int i = threadIdx.x; i < kReach; i += blockDim.x) {
+    const int d = abs(i - 64);
+    rs[i] = d <= g.Q ? (T)__ldg(g.pw + min(d, 63)) : T(0);
+  }
+}
+
+// The axis's taps in shared memory when they fit (no barrier).
+constexpr int kTapsSmem = 128;
+__device__ __forceinline__ const ConvTap* stage_taps(const ConvAxis& g, ConvTap* tsm) {
+  if (g.ntaps > kTapsSmem) return g.taps;
+  for (int i = threadIdx.x; i < g.ntaps; i += blockDim.x) tsm[i] = g.taps[i];
+  return tsm;
+}
+
+// Element at a byte offset below 4 GB from a (uniform) base: one 32-bit offset serves every array of a pass.
+template <typename T>
+__device__ __forceinline__ T& at_off(T* p, uint32_t o) {
+  using C = std::conditional_t<std::is_const_v<T>, const char, char>;
+  return *reinterpret_cast<T*>(reinterpret_cast<C*>(p) + o);
+}
+
+// Junction corrections D[f] of junction j of NF lines with their samples at byte offset o + (jM + m) * sb of src[f]; taps:
+// the axis's taps (a shared-memory copy or g.taps); four taps' samples in flight at a time.
+template <typename T, int NF>
+__device__ __forceinline__ void conv_junction(const ConvAxis& g, const ConvTap* taps, int j, const T* const (&src)[NF],
+                                              uint32_t o, uint32_t sb, T (&D)[NF]) {
+  int t = __ldg(g.js + j);
+  const int t1 = __ldg(g.js + j + 1);
+  double s[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) s[f] = 0.0;
+  for (; t < t1; t += 4) {
+    double w[4];
+    T v[4][NF];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const ConvTap tap = taps[min(t + k, t1 - 1)];
+      w[k] = t + k < t1 ? tap.w : 0.0;
+      const uint32_t ot = o + (uint32_t)(j * g.M + tap.m) * sb;
+#pragma unroll
+      for (int f = 0; f < NF; ++f) v[k][f] = at_off(src[f], ot);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (t + k < t1)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) s[f] = fma(w[k], to_f64(v[k][f]), s[f]);
+  }
+#pragma unroll
+  for (int f = 0; f < NF; ++f) D[f] = (T)s[f];
+}
+
+// Block-wide copy of a launch descriptor into shared memory (no barrier).
+template <class J>
+__device__ __forceinline__ void copy_job(J* dst, const J* __restrict__ src) {
+  static_assert(sizeof(J) % 8 == 0, "descriptor size");
+  for (int i = threadIdx.x; i < (int)(sizeof(J) / 8); i += blockDim.x)
+    reinterpret_cast<uint64_t*>(dst)[i] = reinterpret_cast<const uint64_t*>(src)[i];
+}
+
+// ---------------------------------------------------------------------------------------------------------------
+// Strided lines.  Line q (0 .. lines - 1) starts at (q / inner) * so + q % inner and steps by `stride`; it is cut into
+// segments of seglen positions (a multiple of 8, nseg of them), each marched by one thread.
+//
+// OP: static constexpr int NF (fields differentiated), B (positions whose pointwise operands are held in registers),
+//   const T* src(int f); struct Regs; void load(Regs&, int pos, uint32_t o);
+//   void apply(Regs&, const T (&e)[NF], int pos, uint32_t o, int outer, int x)
+// o: byte offset of the position in every array.  Operands are loaded B positions ahead of their use, across chunks.
+template <typename T, class OP>
+__device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, const OP& op, int bid,
+                                          unsigned char* sm) {
+  constexpr int NF = OP::NF, W = Conv<T>::W, NR = W + 2;
+  constexpr T r = (T)kConvR, r7 = (T)conv_pow(7), r8 = (T)conv_pow(8), r16 = (T)conv_pow(16);
+  constexpr T i1r = (T)(2.0 / (1.0 - kConvR));
+  __shared__ T rs[kReach];
+  __shared__ ConvTap tsm[kTapsSmem];
+  fill_reach(rs, g);
+  const ConvTap* taps = stage_taps(g, tsm);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t item = (int64_t)bid * 4 + warp;
+  if (item >= cm.groups * cm.nseg) return;
+  const int seg = (int)(item / cm.groups);
+  const int64_t q0 = (item - (int64_t)seg * cm.groups) * 32 + lane;
+  const bool valid = q0 < cm.lines;
+  const int64_t q = valid ? q0 : cm.lines - 1;  // surplus lanes repeat the last line and store nothing
+  const int outer = (int)(q / cm.inner), x = (int)(q - (int64_t)outer * cm.inner);
+  const uint32_t base = (uint32_t)(((int64_t)outer * cm.so + x) * (int64_t)sizeof(T));
+  const uint32_t sb = (uint32_t)(cm.stride * (int64_t)sizeof(T));
+  const int n = g.n;
+  const int s0 = seg * cm.seglen, s1 = min(s0 + cm.seglen, n + 1);
+  const int nc = (s1 - s0 + 7) >> 3;      // chunks of the segment
+  const int ce = (n - s0) >> 3;           // chunk that holds position n
+  const int le = n - s0 - 8 * ce;         // its place there
+  T* ring = reinterpret_cast<T*>(sm) + (size_t)warp * NR * 8 * NF * 32 + lane;
+  auto slot = [&](int c) { return ring + (size_t)(c % NR) * (8 * NF * 32); };
+  auto issue = [&](int c) {
+    T* d = slot(c);
+    const int p = s0 + 8 * c;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (p + j <= n)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) cp_async<sizeof(T)>(d + (j * NF + f) * 32, &at_off(op.src(f), base + (uint32_t)(p + j) * sb));
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int c = 0; c <= W; ++c) issue(c);
+  typename OP::Regs pr[OP::B];
+#pragma unroll
+  for (int b = 0; b < OP::B; ++b)
+    if (s0 + b < s1) op.load(pr[b], s0 + b, base + (uint32_t)(s0 + b) * sb);
+  // left sums of the segment's first position
+  T L[NF];
+  if (s0 > 0) {
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      T a = T(0);
+#pragma unroll 8
+      for (int k = Conv<T>::K; k >= 1; --k) a = at_off(op.src(f), base + (uint32_t)(s0 - k) * sb) + r * a;
+      L[f] = a;
+    }
+  }
+  T pb[NF][W];     // sums r^j f_j of the next W chunks
+  T Rn[NF];        // R_n, from the moment chunk ce is in the ring
+  T Da[NF], Db[NF];  // corrections of junctions jn - 2 and jn - 1
+  int jn = s0 <= g.Q ? 0 : (s0 - g.Q + g.M - 1) / g.M;
+  int ja = -1, jb = -1;
+  bool tailed = false;
+#pragma unroll
+  for (int f = 0; f < NF; ++f) Rn[f] = Da[f] = Db[f] = T(0);
+  auto sums = [&](int c, int k) {
+    const T* d = slot(c);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      T a = T(0);
+      if (c < ce) {
+#pragma unroll
+        for (int j = 7; j >= 0; --j) a = d[(j * NF + f) * 32] + r * a;
+      }
+      pb[f][k] = a;
+    }
+  };
+  cp_async_wait<0>();
+#pragma unroll
+  for (int c = 1; c < W; ++c) sums(c, c);  // shifted down by the first iteration
+  for (int c = 0; c < nc; ++c) {
+    issue(c + W + 1);
+    cp_async_wait<1>();
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int k = 0; k + 1 < W; ++k) pb[f][k] = pb[f][k + 1];
+    sums(c + W, W - 1);
+    const T* d = slot(c);
+    const int p0 = s0 + 8 * c;
+    if (c == 0 && s0 == 0) {  // odd reflection at the line's start (n >= 40: chunks 0 .. W are whole)
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        T a = pb[f][0] + r8 * pb[f][1];
+        if (W == 4) a += r16 * (pb[f][W - 2] + r8 * pb[f][W - 1]);
+        T b = T(0);
+#pragma unroll
+        for (int j = 7; j >= 1; --j) b = d[(j * NF + f) * 32] + r * b;
+        L[f] = i1r * d[f * 32] - (b + r7 * a);
+      }
+    }
+    if (!tailed && c + W >= ce) {  // R_n, and the sum of chunk ce with its reflected continuation
+      tailed = true;
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        T s = L[f];
+        for (int i = 8 * c; i < n - s0; ++i) s = slot(i >> 3)[((i & 7) * NF + f) * 32] + r * s;
+        const T* de = slot(ce);
+        const T R = i1r * de[(le * NF + f) * 32] - s;
+        Rn[f] = R;
+        s = R;
+        for (int j = le; j >= 0; --j) s = de[(j * NF + f) * 32] + r * s;
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+          if (c + 1 + k == ce) pb[f][k] = s;
+      }
+    }
+    const int len = min(8, s1 - p0);
+    T e[NF][8];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      T v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = d[(j * NF + f) * 32];
+      T s = L[f];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        e[f][j] = s;
+        s = v[j] + r * s;
+      }
+      L[f] = s;
+      T t = pb[f][0] + r8 * pb[f][1];
+      if (W == 4) t += r16 * (pb[f][W - 2] + r8 * pb[f][W - 1]);
+      if (c == ce) t = Rn[f];
+#pragma unroll
+      for (int j = 7; j >= 0; --j)
+        if (c != ce || j <= le) {
+          e[f][j] = t - e[f][j];
+          t = v[j] + r * t;
+        }
+    }
+    // junction corrections: those within Q of the chunk (at most two, M >= Q + 8)
+    while (g.ntaps && jn <= g.p && jn * g.M <= p0 + 7 + g.Q) {
+      ja = jb;
+      jb = jn;
+      const T* fs[NF];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        Da[f] = Db[f];
+        fs[f] = op.src(f);
+      }
+      conv_junction<T, NF>(g, taps, jn, fs, base, sb, Db);
+      ++jn;
+    }
+    const int oa = p0 - ja * g.M, ob = p0 - jb * g.M;
+    if (ja >= 0 && oa <= g.Q) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) e[f][j] += Da[f] * rs[64 + oa + j];
+    }
+    if (jb >= 0 && ob <= g.Q) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) e[f][j] += Db[f] * rs[64 + ob + j];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j >= len) break;
+      T ej[NF];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) ej[f] = e[f][j];
+      const uint32_t o = base + (uint32_t)(p0 + j) * sb;
+      if (valid) op.apply(pr[j % OP::B], ej, p0 + j, o, outer, x);
+      if (p0 + j + OP::B < s1) op.load(pr[j % OP::B], p0 + j + OP::B, o + OP::B * sb);
+    }
+  }
+  cp_async_wait<0>();
+}
+
+template <typename T, class OP>
+__global__ void __launch_bounds__(128, OP::kBlocks) k_col(ConvAxis g, ColMap cm, OP op) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  col_block<T>(g, cm, op, blockIdx.x, sm);
+}
+
+// All shots in one launch: block b does the work of block blk[b].y of shot blk[b].x's own launch.
+template <typename T, class OP>
+struct ColJob {
+  ConvAxis g;
+  ColMap cm;
+  OP op;
+};
+template <typename T, class OP>
+__global__ void __launch_bounds__(128, OP::kBlocks)
+    k_col_batch(const ColJob<T, OP>* __restrict__ jobs, const int2* __restrict__ blk) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ __align__(16) unsigned char raw[sizeof(ColJob<T, OP>)];
+  const int2 w = blk[blockIdx.x];
+  ColJob<T, OP>& j = *reinterpret_cast<ColJob<T, OP>*>(raw);
+  copy_job(&j, jobs + w.x);
+  __syncthreads();
+  col_block<T>(j.g, j.cm, j.op, w.y, sm);
+}
+
+// Dynamic shared memory of a k_col block.
+template <typename T>
+constexpr size_t col_smem(int nf) { return (size_t)4 * (Conv<T>::W + 2) * 8 * nf * 32 * sizeof(T); }
+
+// ---------------------------------------------------------------------------------------------------------------
+// Contiguous rows.  Row q (0 .. rows - 1) starts at (q / ny) * sz + (q % ny) * sy.  A row has nch chunks of 8 positions,
+// the last of 1 to 9 (position n joins the chunk before it when n is a multiple of 8).  Rows of at most 32 chunks are
+// one window of gw = 8, 16 or 32 lanes (32 / gw rows per warp); longer rows are cut into nwin windows of 32 chunks
+// that overlap by 2 W chunks, of which each owns all but the W at its inner ends.
+//
+// A lane loads its chunk straight into registers (two 16-byte loads in FP32, 32 bytes apart from its neighbours': the
+// second finds the first's sectors in L1), so nothing is staged; samples cross lanes only in the warm-up sums.
+
+// Eight consecutive elements (vec: p is 16-byte aligned).
+template <typename T>
+__device__ __forceinline__ void ld8(const T* __restrict__ p, bool vec, int len, T* v) {
+  if (vec) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int j = 0; j < 8; j += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p + j);
+        v[j] = t.x, v[j + 1] = t.y, v[j + 2] = t.z, v[j + 3] = t.w;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        const double2 t = *reinterpret_cast<const double2*>(p + j);
+        v[j] = t.x, v[j + 1] = t.y;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = j < len ? p[j] : T(0);
+  }
+}
+// The first min(len, 8) of eight consecutive elements, and the ninth when len = 9.
+template <typename T>
+__device__ __forceinline__ void st9(T* __restrict__ p, bool vec, int len, const T* v) {
+  if (vec && len >= 8) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int j = 0; j < 8; j += 4)
+        *reinterpret_cast<float4*>(p + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) *reinterpret_cast<double2*>(p + j) = make_double2(v[j], v[j + 1]);
+    }
+    if (len > 8) p[8] = v[8];
+  } else {
+#pragma unroll
+    for (int j = 0; j < 9; ++j)
+      if (j < len) p[j] = v[j];
+  }
+}
+template <typename T>
+__device__ __forceinline__ void ld9(const T* __restrict__ p, bool vec, int len, T (&v)[9]) {
+  ld8(p, vec, len, v);
+  v[8] = len > 8 ? p[8] : T(0);
+}
+
+// v[i] by selects on the bits (a plain conditional chain is turned into an array in local memory).
+__device__ __forceinline__ float pick9(const float (&v)[9], int i) {
+  unsigned b = 0;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) b |= j == i ? __float_as_uint(v[j]) : 0u;
+  return __uint_as_float(b);
+}
+__device__ __forceinline__ double pick9(const double (&v)[9], int i) {
+  unsigned long long b = 0;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) b |= j == i ? (unsigned long long)__double_as_longlong(v[j]) : 0ull;
+  return __longlong_as_double((long long)b);
+}
+
+// Samples f of a chunk (0 beyond len) -> e without its junction corrections, in place.  Called by all lanes of the
+// warp; c: chunk of the row, gl: lane of the gw-lane group, end: the chunk holds position n.
+template <typename T>
+__device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, int gl, int gw, T rlen) {
+  constexpr int W = Conv<T>::W;
+  constexpr T r = (T)kConvR, r7 = (T)conv_pow(7), r8 = (T)conv_pow(8), r16 = (T)conv_pow(16);
+  constexpr T i1r = (T)(2.0 / (1.0 - kConvR));
+  const unsigned full = 0xffffffffu;
+  T e[9];
+  T pa = T(0), pb = f[8], pb1;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) pa = f[j] + r * pa;
+#pragma unroll
+  for (int j = 7; j >= 1; --j) pb = f[j] + r * pb;
+  pb1 = pb;
+  pb = f[0] + r * pb;
+  auto down = [&](T v, int d) {
+    const T u = __shfl_down_sync(full, v, d, gw);
+    return gl + d < gw ? u : T(0);
+  };
+  // left sums: chunk -1 of the row is the reflected continuation, whose whole sum is L_0
+  T t = pb + r8 * down(pb, 1);
+  if (W == 4) t += r16 * down(t, 2);
+  const T R0 = pb1 + r7 * down(t, 1);
+  const T l0 = c == 0 ? i1r * f[0] - R0 : T(0);
+  const T L0 = __shfl_sync(full, l0, 0, gw);  // 0 in windows that do not start the row
+  T u = __shfl_up_sync(full, pa, 1, gw);
+  T s = pa + r8 * (gl == 0 ? L0 : u);
+  if (W == 4) {
+    u = __shfl_up_sync(full, s, 2, gw);
+    s += r16 * (gl == 0 ? T(0) : (gl == 1 ? L0 : u));
+  }
+  u = __shfl_up_sync(full, s, 1, gw);
+  s = gl == 0 ? L0 : u;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    e[j] = s;
+    s = f[j] + r * s;
+  }
+  // right sums: the chunk that holds position n continues with R_n
+  T Rn = T(0);
+  if (end) {
+    Rn = len == 9 ? i1r * f[8] - e[8] : i1r * pick9(f, len - 1) - pick9(e, len - 1);
+    pb += rlen * Rn;
+  }
+  t = pb + r8 * down(pb, 1);
+  if (W == 4) t += r16 * down(t, 2);
+  t = down(t, 1);
+  if (end) t = Rn;
+#pragma unroll
+  for (int j = 8; j >= 0; --j) {
+    const T fj = f[j];
+    f[j] = t - e[j];
+    if (j < len) t = fj + r * t;
+  }
+}
+
+// OP: NF, src(f) and void chunk(T (&e)[NF][9], int p0, int len, int64_t gi, int q): the positions p0 .. p0 + len - 1 of
+// row q (flat index gi of position p0).  TWO (rows of one window, NF = 1): chunk leaves the samples of a second
+// derivative along the same rows, also stored at src2(), in e, and chunk2 takes that derivative.
+template <typename T, class OP>
+__device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, const OP& op, int bid, int nblk,
+                                          unsigned char* sm) {
+  constexpr int NF = OP::NF;
+  __shared__ T rs[kReach];
+  __shared__ ConvTap tsm[kTapsSmem];
+  fill_reach(rs, g);
+  const ConvTap* taps = stage_taps(g, tsm);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int gw = rm.gw, rpw = 32 / gw;
+  T* dsm = reinterpret_cast<T*>(sm + (size_t)warp * rm.wbytes);
+  const int gl = lane & (gw - 1), k = lane / gw;
+  const int items = rm.groups * rm.nwin;
+  for (int item = bid * 4 + warp; item < items; item += nblk * 4) {
+    const int grp = item / rm.nwin, win = item - grp * rm.nwin;
+    const int c0 = win * (32 - 2 * Conv<T>::W);              // first chunk of the window
+    const int c1 = min(rm.nch, c0 + gw);                     // past its last
+    const int o0 = win == 0 ? 0 : c0 + Conv<T>::W;           // own chunks
+    const int o1 = c1 == rm.nch ? rm.nch : c1 - Conv<T>::W;
+    auto rbase = [&](int q) {
+      const int z = q / rm.ny;
+      return z * rm.sz + (q - z * rm.ny) * rm.sy;
+    };
+    const int nrow = min(rpw, rm.rows - grp * rpw);
+    const int q = grp * rpw + min(k, nrow - 1);
+    const int64_t rb = rbase(q);
+    const int c = c0 + gl;
+    const int len = (k < nrow && c < c1) ? (c == rm.nch - 1 ? g.n + 1 - 8 * c : 8) : 0;
+    const bool end = len > 0 && c == rm.nch - 1;
+    const T rlen = end ? (T)__ldg(g.pw + len) : T(0);
+    T e[NF][9];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+#pragma unroll
+      for (int j = 0; j < 9; ++j) e[f][j] = T(0);
+      if (len > 0) ld9(op.src(f) + rb + 8 * c, rm.vec, len, e[f]);
+    }
+    // junctions within Q of the own positions
+    int j0 = 0, nj = 0;
+    if (g.ntaps) {
+      const int lo = 8 * o0, hi = o1 == rm.nch ? g.n : 8 * o1 - 1;
+      j0 = lo <= g.Q ? 0 : (lo - g.Q + g.M - 1) / g.M;
+      nj = min(g.p, (hi + g.Q) / g.M) - j0 + 1;
+    }
+    // e of the NF fields whose samples are in e and at s0 (fields 1 ..: at op.src)
+    auto derive = [&](const T* s0) {
+      if (nj > 0) {  // one lane per (field, row, junction)
+        __syncwarp();
+        for (int i = lane; i < NF * nrow * nj; i += 32) {
+          const int j = i % nj, fk = i / nj, f = fk / nrow;
+          int64_t off = rbase(grp * rpw + fk - f * nrow);
+#pragma unroll
+          for (int s = 1; s < NF; ++s) off += f == s ? op.src(s) - s0 : (int64_t)0;
+          const T* fs[1] = {s0 + off};
+          T D[1];
+          conv_junction<T, 1>(g, taps, j0 + j, fs, 0u, (uint32_t)sizeof(T), D);
+          dsm[i] = D[0];
+        }
+        __syncwarp();
+      }
+      if (end && len < 8)
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (j >= len) e[f][j] = T(0);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) row_solve<T>(e[f], c, len, end, gl, gw, rlen);
+      if (nj > 0 && len > 0) {
+        const int ja = 8 * c / g.M;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const int jj = ja + s - j0, o = 8 * c - (ja + s) * g.M;  // offset of the chunk from the junction
+          if (jj >= 0 && jj < nj && o <= g.Q && -o - 8 <= g.Q) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+              const T D = dsm[(f * nrow + k) * nj + jj];
+#pragma unroll
+              for (int j = 0; j < 9; ++j) e[f][j] += D * rs[64 + o + j];
+            }
+          }
+        }
+      }
+    };
+    derive(op.src(0));
+    const bool own = len > 0 && c >= o0 && c < o1;
+    if (own) op.chunk(e, 8 * c, len, rb + 8 * c, q);
+    if constexpr (OP::TWO) {
+      if (!own)  // lanes beyond the row carry no samples into the second derivative
+#pragma unroll
+        for (int j = 0; j < 9; ++j) e[0][j] = T(0);
+      derive(op.src2());
+      if (own) op.chunk2(e, 8 * c, len, rb + 8 * c, q);
+    }
+  }
+}
+
+template <typename T, class OP>
+__global__ void __launch_bounds__(128, OP::kBlocks) k_row(ConvAxis g, RowMap rm, OP op) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  row_block<T>(g, rm, op, blockIdx.x, gridDim.x, sm);
+}
+
+// All shots in one launch, as k_col_batch; blk[b].z: blocks of the shot.
+template <typename T, class OP>
+struct RowJob {
+  ConvAxis g;
+  RowMap rm;
+  OP op;
+};
+template <typename T, class OP>
+__global__ void __launch_bounds__(128, OP::kBlocks)
+    k_row_batch(const RowJob<T, OP>* __restrict__ jobs, const int4* __restrict__ blk) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ __align__(16) unsigned char raw[sizeof(RowJob<T, OP>)];
+  const int4 w = blk[blockIdx.x];
+  RowJob<T, OP>& j = *reinterpret_cast<RowJob<T, OP>*>(raw);
+  copy_job(&j, jobs + w.x);
+  __syncthreads();
+  row_block<T>(j.g, j.rm, j.op, w.y, w.z, sm);
+}
+
+}  // namespace lossk

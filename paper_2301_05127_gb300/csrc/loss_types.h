@@ -273,6 +273,9 @@ struct TzShot {
 // unit0 .. unit0 + ceil(t.ncross / R) - 1.
 constexpr int kXpMaxGroups = 8;
 
+// Elastic passes on the barrier-free engines (loss_kernels_stream.cu).
+enum { ES_BX = 0, ES_BY = 1, ES_BZ = 2, ES_AZ = 3, ES_AX = 4, ES_AY = 5 };
+
 // Elastic y / z tile passes (FP32 truncated-convolution form).
 enum { ET_BY = 0, ET_BZ = 1, ET_AZ = 2, ET_AY = 3 };
 struct ElTile {
@@ -281,6 +284,46 @@ struct ElTile {
   int nouter;       // its extent
   int ncg;          // groups of 32 x columns
   int nx;           // x columns
+};
+// Axis of the barrier-free engines (loss_stream.cuh): n intervals in p patches of M; the taps of junction j are
+// taps[js[j]] .. taps[js[j + 1] - 1] (weights over a, offsets m from the junction), ntaps in all; a junction's correction
+// reaches Q positions; pw: r^d, d = 0 .. 63.
+struct ConvTap {
+  double w;
+  int m;
+  int pad;
+};
+struct ConvAxis {
+  int n, p, M, Q, ntaps;
+  const int* js;
+  const ConvTap* taps;
+  const double* pw;
+};
+// Strided lines of an array: line q starts at (q / inner) * so + q % inner and steps by stride; groups of 32 lines,
+// nseg segments of seglen positions per line.
+struct ColMap {
+  int64_t lines, groups, inner, so, stride;
+  int nseg, seglen;
+};
+// Contiguous rows of an array: row q starts at (q / ny) * sz + (q % ny) * sy; nch chunks per row, gw lanes per row
+// window, nwin windows per row, groups of 32 / gw rows; vec: rows start on 16-byte boundaries and are readable to the
+// next multiple of 8 positions; wbytes: shared memory of a warp; sms: multiprocessors.
+struct RowMap {
+  int64_t sz, sy;
+  int rows, groups, ny, nch, gw, nwin, vec, wbytes, sms;
+};
+// One shot of a batched FP64 acoustic step on these engines, and one launch of it: its job and block tables at byte
+// offsets of the uploaded tables.
+struct AcStreamShot {
+  ConvAxis gx, gz;
+  RowMap rm;
+  ColMap cm;
+  AcXArgs<double> x;
+  AcZArgs<double> z;
+};
+struct AcBatchKind {
+  int blocks = 0;
+  size_t jobs = 0, blk = 0, smem = 0;
 };
 struct XpShot {
   AcXArgs<float> a;
