@@ -237,8 +237,8 @@ static loss_status_t adjoint_step(loss_ctx* h, Shot& s, const Snap& sn, const Sn
 }
 
 template <typename T>
-static loss_status_t gradient_t(loss_ctx* h, Shot& s, const double* d_obs_host, int64_t C, int64_t n_steps,
-                                double* misfit, std::vector<double> grads_out[3]) {
+static loss_status_t gradient_t(loss_ctx* h, Shot& s, const double* d_obs, int64_t C, int64_t n_steps,
+                                double* misfit) {
   const size_t fb = (size_t)s.total * s.esize;
   const size_t gb = (size_t)s.total * sizeof(double);
   const bool el = s.d.physics == LOSS_ELASTIC;
@@ -298,20 +298,9 @@ static loss_status_t gradient_t(loss_ctx* h, Shot& s, const double* d_obs_host, 
     LOSS_TRY(step_shot(h, s));
   }
   LOSS_TRY(copy_arrays(h, full, (char*)ck + (size_t)K * ck_bytes, fb, true));
-  // residual and misfit
+  // residual and misfit, on the device (partial sums in a fixed order, so that equal runs give equal bits)
   const int64_t nr = s.n_rcv;
-  std::vector<char> tr((size_t)n_steps * nr * s.esize);
-  LOSS_TRY(cuda_check(h, cudaMemcpyAsync(tr.data(), s.traces, tr.size(), cudaMemcpyDeviceToHost, h->stream),
-                      "copy traces"));
-  LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
-  std::vector<double> res((size_t)n_steps * nr);
-  double J = 0.0;
-  for (size_t i = 0; i < res.size(); ++i) {
-    const double v = s.esize == 8 ? ((const double*)tr.data())[i] : (double)((const float*)tr.data())[i];
-    res[i] = v - d_obs_host[i];
-    J += 0.5 * res[i] * res[i];
-  }
-  *misfit = J;
+  const int64_t nres = n_steps * nr;
   double* dres = nullptr;
   void* djobs = nullptr;
   struct Free2 {
@@ -323,9 +312,11 @@ static loss_status_t gradient_t(loss_ctx* h, Shot& s, const double* d_obs_host, 
       dev_free(h, *b);
     }
   } fr2{h, &dres, &djobs};
-  LOSS_TRY(dev_alloc(h, res.size() * sizeof(double), (void**)&dres));
-  LOSS_TRY(cuda_check(h, cudaMemcpyAsync(dres, res.data(), res.size() * sizeof(double), cudaMemcpyHostToDevice,
-                                         h->stream), "copy residual"));
+  LOSS_TRY(dev_alloc(h, (size_t)(nres + kMisfitBlocks + 1) * sizeof(double), (void**)&dres));
+  double* part_sums = dres + nres;
+  LOSS_TRY(cuda_check(h, launch_residual<T>((const T*)s.traces, d_obs, dres, part_sums, nres, h->stream), "residual"));
+  LOSS_TRY(cuda_check(h, cudaMemcpyAsync(misfit, part_sums + kMisfitBlocks, sizeof(double), cudaMemcpyDeviceToHost,
+                                         h->stream), "copy misfit"));
   std::vector<InjectJob<T>> jobs;
   int64_t max_cnt = 0;
   for (int f = 0; f < LOSS_NUM_FIELDS; ++f) {
@@ -373,15 +364,6 @@ static loss_status_t gradient_t(loss_ctx* h, Shot& s, const double* d_obs_host, 
   s.step = n_steps;
   s.staggered = true;
   s.rcv_steps = rsteps_saved;
-  // gradients of the model coefficients, dense, FP64
-  const int nk = 3;
-  for (int i = 0; i < nk; ++i) {
-    grads_out[i].assign((size_t)s.dense, 0.0);
-    const size_t w = (size_t)s.len[2] * sizeof(double);
-    LOSS_TRY(cuda_check(h, cudaMemcpy2DAsync(grads_out[i].data(), w, s.grad[i], (size_t)s.px * sizeof(double), w,
-                                             (size_t)(s.len[0] * s.len[1]), cudaMemcpyDeviceToHost, h->stream),
-                        "copy gradient"));
-  }
   LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
   return LOSS_OK;
 }
@@ -401,42 +383,50 @@ loss_status_t run_gradient(loss_ctx* h, Shot& s, const double* d_obs, int32_t ch
   if (mem != LOSS_MEM_HOST && mem != LOSS_MEM_DEVICE) return err(h, LOSS_E_ARG, "bad mem");
   const int64_t C = checkpoint_every > 0 ? checkpoint_every : (int64_t)std::ceil(std::sqrt((double)n_steps));
   const size_t nobs = (size_t)n_steps * s.n_rcv;
-  std::vector<double> obs;
-  const double* ho = d_obs;
-  if (mem == LOSS_MEM_DEVICE) {
-    obs.resize(nobs);
-    LOSS_TRY(cuda_check(h, cudaMemcpy(obs.data(), d_obs, nobs * sizeof(double), cudaMemcpyDeviceToHost), "copy d_obs"));
-    ho = obs.data();
+  const bool el = s.d.physics == LOSS_ELASTIC;
+  const size_t N = (size_t)s.dense;
+  struct Tmp {
+    loss_ctx* h;
+    void* p[2] = {nullptr, nullptr};
+    ~Tmp() {
+      for (void* q : p) dev_free(h, q);
+    }
+  } tmp{h};
+  LOSS_TRY(dev_alloc(h, nobs * sizeof(double), &tmp.p[0]));
+  LOSS_TRY(dev_alloc(h, 3 * N * sizeof(double), &tmp.p[1]));
+  double* obs = (double*)tmp.p[0];
+  double* out = (double*)tmp.p[1];
+  // caller buffers are read and written in the order of the legacy default stream, whatever the handle's stream is (a
+  // device-to-device cudaMemcpy does not wait for its end by itself)
+  LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
+  LOSS_TRY(cuda_check(h, cudaMemcpy(obs, d_obs, nobs * sizeof(double),
+                                    mem == LOSS_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
+                      "copy d_obs"));
+  LOSS_TRY(cuda_check(h, cudaStreamSynchronize(cudaStreamLegacy), "sync"));
+  // the model as loss_set_model got it, in FP64 on the device from the first gradient on (refreshed after a new model)
+  if (!s.dmodel) LOSS_TRY(dev_alloc(h, (el ? 3 : 2) * N * sizeof(double), (void**)&s.dmodel));
+  if (!s.dmodel_valid) {
+    const std::vector<double>* src[3] = {&s.h_vp, &s.h_rho, &s.h_vs};
+    for (int i = 0; i < (el ? 3 : 2); ++i)
+      LOSS_TRY(cuda_check(h, cudaMemcpy(s.dmodel + i * N, src[i]->data(), N * sizeof(double), cudaMemcpyHostToDevice),
+                          "copy model"));
+    s.dmodel_valid = true;
   }
-  std::vector<double> gk[3];
   struct Flag {  // (also reset when a call fails)
     bool& f;
     ~Flag() { f = false; }
   } flag{h->in_gradient};
   h->in_gradient = true;
-  if (s.esize == 8) LOSS_TRY(gradient_t<double>(h, s, ho, C, n_steps, misfit, gk));
-  else LOSS_TRY(gradient_t<float>(h, s, ho, C, n_steps, misfit, gk));
-  // chain rule (FP64, dense): kappa = rho vp^2 | lambda = rho (vp^2 - 2 vs^2), mu = rho vs^2; b = 1 / rho
-  const size_t N = (size_t)s.dense;
-  std::vector<double> ovp(N), ovs(s.d.physics == LOSS_ELASTIC ? N : 0), orho(N);
-  for (size_t i = 0; i < N; ++i) {
-    const double vp = s.h_vp[i], rho = s.h_rho[i];
-    if (s.d.physics == LOSS_ELASTIC) {
-      const double vs = s.h_vs[i];
-      ovp[i] = gk[0][i] * 2.0 * rho * vp;
-      ovs[i] = gk[0][i] * (-4.0 * rho * vs) + gk[1][i] * 2.0 * rho * vs;
-      orho[i] = gk[0][i] * (vp * vp - 2.0 * vs * vs) + gk[1][i] * vs * vs - gk[2][i] / (rho * rho);
-    } else {
-      ovp[i] = gk[0][i] * 2.0 * rho * vp;
-      orho[i] = gk[0][i] * vp * vp - gk[2][i] / (rho * rho);
-    }
-  }
-  const cudaMemcpyKind kind = mem == LOSS_MEM_HOST ? cudaMemcpyHostToHost : cudaMemcpyHostToDevice;
-  LOSS_TRY(cuda_check(h, cudaMemcpy(g_vp, ovp.data(), N * sizeof(double), kind), "copy g_vp"));
-  LOSS_TRY(cuda_check(h, cudaMemcpy(g_rho, orho.data(), N * sizeof(double), kind), "copy g_rho"));
-  if (s.d.physics == LOSS_ELASTIC)
-    LOSS_TRY(cuda_check(h, cudaMemcpy(g_vs, ovs.data(), N * sizeof(double), kind), "copy g_vs"));
-  return LOSS_OK;
+  if (s.esize == 8) LOSS_TRY(gradient_t<double>(h, s, obs, C, n_steps, misfit));
+  else LOSS_TRY(gradient_t<float>(h, s, obs, C, n_steps, misfit));
+  LOSS_TRY(cuda_check(h, launch_chain(s.grad[0], s.grad[1], s.grad[2], s.dmodel, el ? 1 : 0, (int64_t)N, s.len[2], s.px,
+                                      out, h->num_sms, h->stream), "chain rule"));
+  LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
+  const cudaMemcpyKind kind = mem == LOSS_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+  LOSS_TRY(cuda_check(h, cudaMemcpy(g_vp, out, N * sizeof(double), kind), "copy g_vp"));
+  LOSS_TRY(cuda_check(h, cudaMemcpy(g_rho, out + N, N * sizeof(double), kind), "copy g_rho"));
+  if (el) LOSS_TRY(cuda_check(h, cudaMemcpy(g_vs, out + 2 * N, N * sizeof(double), kind), "copy g_vs"));
+  return cuda_check(h, cudaStreamSynchronize(cudaStreamLegacy), "sync");
 }
 
 // Stand-alone D^T along internal slot k of dense arrays (DEVICE pointers).

@@ -866,6 +866,7 @@ loss_status_t loss_set_model(loss_handle_t h, int32_t shot, const double* vp, co
       md[1][i] = 1.0 / r;              // b
     }
   }
+  s->dmodel_valid = false;
   s->h_vp.assign(pvp, pvp + N);
   s->h_rho.assign(prho, prho + N);
   if (el) s->h_vs.assign(pvs, pvs + N);
