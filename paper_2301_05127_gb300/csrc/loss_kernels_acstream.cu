@@ -23,11 +23,12 @@
 namespace lossk {
 
 // Pointers that a launch does not use (no layer, constant density) are readable ones; b_on: the density is an array.
-template <typename T, bool KAHAN, bool REC, bool DOB, bool DOA>
+// TAB: the source amplitude of the step comes from the shot's device table and clock (batched launches).
+template <typename T, bool KAHAN, bool REC, bool DOB, bool DOA, bool TAB>
 struct AcRowOp {
   static constexpr int NF = 1;
   static constexpr bool TWO = DOB && DOA;
-  static constexpr int kBlocks = 4;
+  static constexpr int kBlocks = sizeof(T) == 8 ? 3 : 4;
   AcXArgs<T> a;
   int b_on, pad;
   __device__ __forceinline__ const T* src(int) const { return DOB ? a.v1 : a.sigma; }
@@ -46,7 +47,8 @@ struct AcRowOp {
     m = m1;
     return x;
   }
-  // sub-step B of a chunk; leaves the new sigma in e
+  // sub-step B of a chunk; leaves the new sigma in e.  (The ninth position exists in a row's last chunk at most: every
+  // loop leaves before it otherwise.)
   __device__ __forceinline__ void stress(T (&e)[9], int p0, int len, int64_t gi, int q) const {
     const bool lay = a.pml && (a.xB.in(p0) || a.xB.in(p0 + len - 1));
     const bool zlay = a.pml && a.zB.in(q);
@@ -60,44 +62,69 @@ struct AcRowOp {
     if (zlay) {
       const int n1 = a.zB.n + 1;
 #pragma unroll
-      for (int j = 0; j < 9; ++j) gz[j] = flow(a.zB.tab, n1, q, gz[j], mz[j]);
+      for (int j = 0; j < 9; ++j) {
+        if (j == 8 && len < 9) break;
+        gz[j] = -flow(a.zB.tab, n1, q, gz[j], mz[j]);
+      }
       st9(a.phiz + gi, true, len, mz);
     } else {
 #pragma unroll
-      for (int j = 0; j < 9; ++j) gz[j] = -mulc(gz[j], a.dt, a.dt_lo);
+      for (int j = 0; j < 9; ++j) {
+        if (j == 8 && len < 9) break;
+        gz[j] = mulc(gz[j], a.dt, a.dt_lo);
+      }
     }
     if (lay) {
       const int n1 = a.xB.n + 1;
 #pragma unroll
       for (int j = 0; j < 9; ++j) {
-        const T g = mulc(e[j], a.s3h, a.s3h_lo);
-        e[j] = (j < len && a.xB.in(p0 + j)) ? flow(a.xB.tab, n1, p0 + j, g, mx[j]) : -mulc(g, a.dt, a.dt_lo);
+        if (j == 8 && len < 9) break;
+        if (j < len && a.xB.in(p0 + j)) e[j] = -flow(a.xB.tab, n1, min(p0 + j, a.xB.n), mulc(e[j], a.s3h, a.s3h_lo), mx[j]);
+        else e[j] = mulc(e[j], a.sdt, a.sdt_lo);
       }
       st9(a.phix + gi, true, len, mx);
+#pragma unroll
+      for (int j = 0; j < 9; ++j) {
+        if (j == 8 && len < 9) break;
+        e[j] += gz[j];
+      }
     } else {
 #pragma unroll
-      for (int j = 0; j < 9; ++j) e[j] = -mulc(mulc(e[j], a.s3h, a.s3h_lo), a.dt, a.dt_lo);
+      for (int j = 0; j < 9; ++j) {
+        if (j == 8 && len < 9) break;
+        if constexpr (sizeof(T) == 8) e[j] = fma(e[j], a.sdt, gz[j]);
+        else e[j] = mulc(e[j], a.sdt, a.sdt_lo) + gz[j];
+      }
     }
-#pragma unroll
-    for (int j = 0; j < 9; ++j) e[j] = kp[j] * (e[j] + gz[j]);
+    // e = minus the divergence's increment: sigma += -kappa e (+ source)
     if (a.src.on && (unsigned)(q - a.src.zs + 12) < 25u) {
-      const double amp = a.src.amp_tab ? a.src.amp_tab[a.src.clk->step] : a.src.amp;
+      double amp = a.src.amp;
+      if constexpr (TAB) amp = a.src.amp_tab[a.src.clk->step];
       if (amp != 0.0)
 #pragma unroll
         for (int j = 0; j < 9; ++j) {
           const int dx = p0 + j - a.src.xs + 12;
-          if (j < len && (unsigned)dx < 25u) e[j] += (T)(amp * a.src.g[q - a.src.zs + 12] * a.src.g[dx]);
+          if (j < len && (unsigned)dx < 25u) {
+            const T sv = (T)(amp * a.src.g[min((unsigned)(q - a.src.zs + 12), 24u)] * a.src.g[min((unsigned)dx, 24u)]);
+            if constexpr (KAHAN) {
+              e[j] = -kp[j] * e[j] + sv;
+              kp[j] = T(-1);
+            } else {
+              sg[j] += sv;
+            }
+          }
         }
     }
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
+      if (j == 8 && len < 9) break;
       if constexpr (KAHAN) {
         float v = sg[j], c = cs[j];
-        kahan_add(v, c, e[j]);
+        kahan_add(v, c, -kp[j] * e[j]);
         e[j] = v;
         cs[j] = c;
       } else {
-        e[j] = sg[j] + e[j];
+        e[j] = fma(-kp[j], e[j], sg[j]);
       }
     }
     st9(a.sigma + gi, true, len, e);
@@ -116,39 +143,42 @@ struct AcRowOp {
     if constexpr (KAHAN) ld9(a.cv1 + gi, true, len, c);
     if (b_on) ld9(a.b + gi, true, len, bb);
     if (lay) ld9(a.psix + gi, true, len, m);
-    if (lay) {
-      const int n1 = a.xA.n + 1;
-#pragma unroll
-      for (int j = 0; j < 9; ++j) {
-        const T g = mulc(e[j], a.s3h, a.s3h_lo);
-        if (j < len && a.xA.in(p0 + j)) {
-          const int i = p0 + j;
-          const T m0 = m[j];
-          e[j] = flow(a.xA.tab, n1, i, g, m[j]);
-          if constexpr (REC) {
-            T mh = m0;
-            const T ih = flow(a.xA.tabh, n1, i, g, mh);
-            a.dlt[gi + j] = (b_on ? bb[j] : a.b0) * (ih - T(0.5) * e[j]);
-          }
-        } else {
-          e[j] = -mulc(g, a.acoef, a.acoef_lo);
-        }
-      }
-      st9(a.psix + gi, true, len, m);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 9; ++j) e[j] = -mulc(mulc(e[j], a.s3h, a.s3h_lo), a.acoef, a.acoef_lo);
-    }
+    const T sa = -(a.s3h * a.acoef), sa_lo = -(a.s3h * a.acoef_lo + a.s3h_lo * a.acoef);  // with an array of b
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
-      const T delta = b_on ? bb[j] * e[j] : mulc(e[j], a.b0, a.b0_lo);
-      if constexpr (KAHAN) {
-        float vv = v[j], cc = c[j];
-        kahan_add(vv, cc, delta);
-        v[j] = vv;
-        c[j] = cc;
+      if (j == 8 && len < 9) break;
+      if (lay && j < len && a.xA.in(p0 + j)) {
+        const int n1 = a.xA.n + 1, i = min(p0 + j, a.xA.n);
+        const T g = mulc(e[j], a.s3h, a.s3h_lo), m0 = m[j];
+        e[j] = flow(a.xA.tab, n1, i, g, m[j]);
+        if constexpr (REC) {
+          T mh = m0;
+          const T ih = flow(a.xA.tabh, n1, i, g, mh);
+          a.dlt[gi + j] = (b_on ? bb[j] : a.b0) * (ih - T(0.5) * e[j]);
+        }
+        e[j] = b_on ? bb[j] * e[j] : mulc(e[j], a.b0, a.b0_lo);
+      } else if (b_on) {
+        e[j] = bb[j] * mulc(e[j], sa, sa_lo);
+      } else if constexpr (sizeof(T) == 8) {
+        v[j] = fma(e[j], a.sc, v[j]);
+        e[j] = T(0);
       } else {
-        v[j] += delta;
+        e[j] = mulc(e[j], a.sc, a.sc_lo);
+      }
+    }
+    if (lay) st9(a.psix + gi, true, len, m);
+    if (sizeof(T) == 4 || b_on || lay) {
+#pragma unroll
+      for (int j = 0; j < 9; ++j) {
+        if (j == 8 && len < 9) break;
+        if constexpr (KAHAN) {
+          float vv = v[j], cc = c[j];
+          kahan_add(vv, cc, e[j]);
+          v[j] = vv;
+          c[j] = cc;
+        } else {
+          v[j] += e[j];
+        }
       }
     }
     st9(a.v1 + gi, true, len, v);
@@ -175,27 +205,27 @@ struct AcColOp {
     }
   }
   __device__ __forceinline__ void apply(Regs& r, const T (&e)[1], int pos, uint32_t o, int, int) const {
-    const T g = mulc(e[0], a.s3h, a.s3h_lo);
     if constexpr (MODE == 2) {
-      at_off(a.tmp, o) = g;
-    } else {
-      T inc;
-      if (a.pml && a.zA.in(pos)) {
-        const int n1 = a.zA.n + 1;
-        const T* t = a.zA.tab;
-        const T m1 = t[pos] * r.m - t[n1 + pos] * g;
-        inc = t[2 * n1 + pos] * (m1 - r.m) - t[3 * n1 + pos] * g;
-        if constexpr (REC) {
-          const T* th = a.zA.tabh;
-          const T mh = th[pos] * r.m - th[n1 + pos] * g;
-          const T ih = th[2 * n1 + pos] * (mh - r.m) - th[3 * n1 + pos] * g;
-          at_off(a.dlt, o) = (b_on ? r.b : a.b0) * (ih - T(0.5) * inc);
-        }
-        at_off(a.psiz, o) = m1;
-      } else {
-        inc = -mulc(g, a.acoef, a.acoef_lo);
+      at_off(a.tmp, o) = mulc(e[0], a.s3h, a.s3h_lo);
+    } else if (a.pml && a.zA.in(pos)) {
+      const T g = mulc(e[0], a.s3h, a.s3h_lo);
+      const int n1 = a.zA.n + 1;
+      const T* t = a.zA.tab;
+      const T m1 = t[pos] * r.m - t[n1 + pos] * g;
+      const T inc = t[2 * n1 + pos] * (m1 - r.m) - t[3 * n1 + pos] * g;
+      const T bb = b_on ? r.b : a.b0;
+      if constexpr (REC) {
+        const T* th = a.zA.tabh;
+        const T mh = th[pos] * r.m - th[n1 + pos] * g;
+        const T ih = th[2 * n1 + pos] * (mh - r.m) - th[3 * n1 + pos] * g;
+        at_off(a.dlt, o) = bb * (ih - T(0.5) * inc);
       }
-      at_off(a.v3, o) = r.v + (b_on ? r.b * inc : mulc(inc, a.b0, a.b0_lo));
+      at_off(a.psiz, o) = m1;
+      at_off(a.v3, o) = r.v + bb * inc;
+    } else if (b_on) {
+      at_off(a.v3, o) = fma(r.b * -(a.s3h * a.acoef), e[0], r.v);
+    } else {
+      at_off(a.v3, o) = fma(e[0], a.sc, r.v);
     }
   }
 };
@@ -248,15 +278,15 @@ cudaError_t launch_ac_rows(const AcXArgs<T>& a, const ConvAxis& g, const RowMap&
   AcXArgs<T> f = a;
   fill_unused(f);
   if (a.do_B && rm.nwin == 1) {
-    if (rec) return go_row<T>(g, rm, AcRowOp<T, KAHAN, true, true, true>{f, b_on, 0}, st);
-    return go_row<T>(g, rm, AcRowOp<T, KAHAN, false, true, true>{f, b_on, 0}, st);
+    if (rec) return go_row<T>(g, rm, AcRowOp<T, KAHAN, true, true, true, false>{f, b_on, 0}, st);
+    return go_row<T>(g, rm, AcRowOp<T, KAHAN, false, true, true, false>{f, b_on, 0}, st);
   }
   if (a.do_B) {
-    const cudaError_t e = go_row<T>(g, rm, AcRowOp<T, KAHAN, false, true, false>{f, b_on, 0}, st);
+    const cudaError_t e = go_row<T>(g, rm, AcRowOp<T, KAHAN, false, true, false, false>{f, b_on, 0}, st);
     if (e != cudaSuccess) return e;
   }
-  if (rec) return go_row<T>(g, rm, AcRowOp<T, KAHAN, true, false, true>{f, b_on, 0}, st);
-  return go_row<T>(g, rm, AcRowOp<T, KAHAN, false, false, true>{f, b_on, 0}, st);
+  if (rec) return go_row<T>(g, rm, AcRowOp<T, KAHAN, true, false, true, false>{f, b_on, 0}, st);
+  return go_row<T>(g, rm, AcRowOp<T, KAHAN, false, false, true, false>{f, b_on, 0}, st);
 }
 // mode 1: Z1, mode 2: Z2 (FP64).
 cudaError_t launch_ac_cols(const AcZArgs<double>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st) {
@@ -280,11 +310,11 @@ template <class F>
 static void with_kind(int kind, F&& f) {
   using D = double;
   switch (kind) {
-    case 0: return f(RowJob<D, AcRowOp<D, false, false, true, true>>{});
-    case 1: return f(RowJob<D, AcRowOp<D, false, true, true, true>>{});
-    case 2: return f(RowJob<D, AcRowOp<D, false, false, true, false>>{});
-    case 3: return f(RowJob<D, AcRowOp<D, false, false, false, true>>{});
-    case 4: return f(RowJob<D, AcRowOp<D, false, true, false, true>>{});
+    case 0: return f(RowJob<D, AcRowOp<D, false, false, true, true, true>>{});
+    case 1: return f(RowJob<D, AcRowOp<D, false, true, true, true, true>>{});
+    case 2: return f(RowJob<D, AcRowOp<D, false, false, true, false, true>>{});
+    case 3: return f(RowJob<D, AcRowOp<D, false, false, false, true, true>>{});
+    case 4: return f(RowJob<D, AcRowOp<D, false, true, false, true, true>>{});
     case 5: return f(ColJob<D, AcColOp<D, 1, false>>{});
     case 6: return f(ColJob<D, AcColOp<D, 1, true>>{});
     default: return f(ColJob<D, AcColOp<D, 2, false>>{});

@@ -32,6 +32,10 @@ struct ElColOp {
     T m[3];  // the memory variables of the three terms (layers only)
   };
   __device__ __forceinline__ const T* src(int f) const { return a.src[f]; }
+  __device__ __forceinline__ T source_at(int dz, int dy, int dx) const {
+    return (T)(a.srcp.amp * a.srcp.g[min((unsigned)dz, 24u)] * a.srcp.g[min((unsigned)dy, 24u)] *
+               a.srcp.g[min((unsigned)dx, 24u)]);
+  }
   static __device__ __forceinline__ constexpr int stress(int i) {  // the six stresses in the order of the updates below
     return i == 0 ? LOSS_FIELD_S11 : (i == 1 ? LOSS_FIELD_S22 : (i == 2 ? LOSS_FIELD_S12 : (i == 3 ? LOSS_FIELD_S13 :
            (i == 4 ? LOSS_FIELD_S23 : LOSS_FIELD_S33))));
@@ -67,9 +71,9 @@ struct ElColOp {
   __device__ __forceinline__ void apply(Regs& r, const T (&e)[3], int pos, uint32_t o, int outer, int x) const {
     T* const* t = a.tmp;
     T g[3];
-#pragma unroll
-    for (int f = 0; f < 3; ++f) g[f] = mulc(e[f], a.s3h, a.s3h_lo);
     if (a.pml && a.pB.in(pos)) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) g[f] = mulc(e[f], a.s3h, a.s3h_lo);
       // the exact sub-flow (PmlAxis::step) on the memory values loaded ahead
       const PmlAxis<T>& pa = kStress ? a.pB : a.pA;
       const int n1 = pa.n + 1;
@@ -96,7 +100,7 @@ struct ElColOp {
       }
     } else {
 #pragma unroll
-      for (int f = 0; f < 3; ++f) g[f] = kStress ? mulc(g[f], a.dt, a.dt_lo) : mulc(g[f], a.acoef, a.acoef_lo);
+      for (int f = 0; f < 3; ++f) g[f] = mulc(e[f], a.st, a.st_lo);
     }
     if constexpr (PASS == ES_BY) {
       at_off(t[1], o) = r.t[0] + g[0];
@@ -116,7 +120,7 @@ struct ElColOp {
       if (a.srcp.on) {
         const int dz = pos - a.srcp.zs + 12, dy = outer - a.srcp.ys + 12, dx = x - a.srcp.xs + 12;
         if ((unsigned)dz < 25u && (unsigned)dy < 25u && (unsigned)dx < 25u) {
-          const T sv = (T)(a.srcp.amp * a.srcp.g[dz] * a.srcp.g[dy] * a.srcp.g[dx]);
+          const T sv = source_at(dz, dy, dx);
           if (a.src_explosive) s11 += sv, s22 += sv, s33 += sv;
           if (a.src_shear) s13 += sv;
         }
@@ -133,7 +137,7 @@ struct ElColOp {
       if (a.srcp.on) {
         const int dz = outer - a.srcp.zs + 12, dy = pos - a.srcp.ys + 12, dx = x - a.srcp.xs + 12;
         if ((unsigned)dz < 25u && (unsigned)dy < 25u && (unsigned)dx < 25u)
-          force = (T)(a.srcp.amp * a.srcp.g[dz] * a.srcp.g[dy] * a.srcp.g[dx]);
+          force = source_at(dz, dy, dx);
       }
       auto mb = [&](T v) { return b_on ? r.m0 * v : mulc(v, a.b0, a.b0_lo); };
 #pragma unroll
@@ -171,25 +175,22 @@ struct ElRowOp {
 #pragma unroll
       for (int f = 0; f < 3; ++f) ld9(mem[f] + gi, true, len, m[f]);
     }
-#pragma unroll
-    for (int f = 0; f < 3; ++f)
-#pragma unroll
-      for (int j = 0; j < 9; ++j) e[f][j] = mulc(e[f][j], a.s3h, a.s3h_lo);
     if (lay) {  // X[f,x] or Y[f,x] inside the layers: the exact sub-flow with its memory variable (PmlAxis::step)
       const int n1 = pa.n + 1;
 #pragma unroll
       for (int j = 0; j < 9; ++j) {
-        const int i = p0 + j;
+        const int i = min(p0 + j, pa.n);
         if (j < len && pa.in(i)) {
           const T T0 = pa.tab[i], T1 = pa.tab[n1 + i], T2 = pa.tab[2 * n1 + i], T3 = pa.tab[3 * n1 + i];
           T x[3];
 #pragma unroll
           for (int f = 0; f < 3; ++f) {
-            const T m1 = T0 * m[f][j] - T1 * e[f][j];
-            x[f] = -(T2 * (m1 - m[f][j]) - T3 * e[f][j]);
+            const T g = mulc(e[f][j], a.s3h, a.s3h_lo);
+            const T m1 = T0 * m[f][j] - T1 * g;
+            x[f] = -(T2 * (m1 - m[f][j]) - T3 * g);
             if constexpr (REC) {
-              const T h1 = pa.tabh[i] * m[f][j] - pa.tabh[n1 + i] * e[f][j];
-              const T xh = -(pa.tabh[2 * n1 + i] * (h1 - m[f][j]) - pa.tabh[3 * n1 + i] * e[f][j]);
+              const T h1 = pa.tabh[i] * m[f][j] - pa.tabh[n1 + i] * g;
+              const T xh = -(pa.tabh[2 * n1 + i] * (h1 - m[f][j]) - pa.tabh[3 * n1 + i] * g);
               a.dlt[f][gi + j] = (b_on ? a.b[gi + j] : a.b0) * (xh - T(0.5) * x[f]);
             }
             m[f][j] = m1;
@@ -197,8 +198,7 @@ struct ElRowOp {
           }
         } else {
 #pragma unroll
-          for (int f = 0; f < 3; ++f)
-            e[f][j] = PASS == ES_BX ? mulc(e[f][j], a.dt, a.dt_lo) : mulc(e[f][j], a.acoef, a.acoef_lo);
+          for (int f = 0; f < 3; ++f) e[f][j] = mulc(e[f][j], a.st, a.st_lo);
         }
       }
 #pragma unroll
@@ -207,8 +207,10 @@ struct ElRowOp {
 #pragma unroll
       for (int f = 0; f < 3; ++f)
 #pragma unroll
-        for (int j = 0; j < 9; ++j)
-          e[f][j] = PASS == ES_BX ? mulc(e[f][j], a.dt, a.dt_lo) : mulc(e[f][j], a.acoef, a.acoef_lo);
+        for (int j = 0; j < 9; ++j) {
+          if (j == 8 && len < 9) break;
+          e[f][j] = mulc(e[f][j], a.st, a.st_lo);
+        }
     }
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
@@ -216,7 +218,10 @@ struct ElRowOp {
         st9(t[f] + gi, true, len, e[f]);
       } else {
 #pragma unroll
-        for (int j = 0; j < 9; ++j) u[f][j] += e[f][j];
+        for (int j = 0; j < 9; ++j) {
+          if (j == 8 && len < 9) break;
+          u[f][j] += e[f][j];
+        }
         st9(t[5 + f] + gi, true, len, u[f]);
       }
     }

@@ -214,11 +214,17 @@ static bool xp_ok(const loss_ctx* h, const Shot& s, const TileGeom& t) {
 
 // Arguments with the engines' derivative scale 3 a / h (they return e / a).
 template <class A>
-static void conv_scale(A& a, const Shot& s, int k) {
+static void conv_scale(A& a, const Shot& s, int k, double acoef) {
   using T = decltype(a.s3h);
   const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k];
   a.s3h = (T)sc;
   a.s3h_lo = lo_part<T>(sc);
+  a.sc = (T)(-acoef * s.b0 * sc);
+  a.sc_lo = lo_part<T>(-acoef * s.b0 * sc);
+  if constexpr (std::is_same_v<A, AcXArgs<T>>) {
+    a.sdt = (T)(sc * s.d.dt);
+    a.sdt_lo = lo_part<T>(sc * s.d.dt);
+  }
 }
 // A 2-D shot's arrays are within the engines' 32-bit byte offsets and row counts.
 static bool conv_size_ok(const Shot& s) {
@@ -248,7 +254,7 @@ static loss_status_t acs_rows(loss_ctx* h, Shot& s, int do_B, double acoef, doub
   bool ok;
   LOSS_TRY(conv_axis(h, s, 2, &g, &ok));
   AcXArgs<T> a = ac_x_args<T>(h, s, LineGeom{}, do_B, acoef, amp);
-  conv_scale(a, s, 2);
+  conv_scale(a, s, 2, acoef);
   LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
   return cuda_check(h, launch_ac_rows<T, K>(a, g, row_map(h, s, 1, g, s.sy, s.sz, true), h->stream), "acoustic x kernel");
 }
@@ -258,7 +264,7 @@ static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
   bool ok;
   LOSS_TRY(conv_axis(h, s, 0, &g, &ok));
   AcZArgs<double> a = ac_z_args<double>(h, s, LineGeom{}, acoef, 0);
-  conv_scale(a, s, 0);
+  conv_scale(a, s, 0, acoef);
   LaunchScope ls(h, mode == 1 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2);
   return cuda_check(h, launch_ac_cols(a, g, col_map(h, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
 }
@@ -663,6 +669,9 @@ static loss_status_t els_pass(loss_ctx* h, Shot& s, int pass, double acoef, doub
   const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k];  // the engines return e / a
   a.s3h = (T)sc;
   a.s3h_lo = lo_part<T>(sc);
+  const double tau = B ? s.d.dt : acoef;
+  a.st = (T)(sc * tau);
+  a.st_lo = lo_part<T>(sc * tau);
   ConvAxis g;
   bool ok;
   LOSS_TRY(conv_axis(h, s, k, &g, &ok));
@@ -1157,9 +1166,9 @@ static loss_status_t acs_tables(loss_ctx* h) {
     q.x.src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
     q.x.src.amp_tab = s.amp_tab;
     q.x.src.clk = B.clk + i;
-    conv_scale(q.x, s, 2);
+    conv_scale(q.x, s, 2, s.d.dt);
     q.z = ac_z_args<double>(h, s, LineGeom{}, s.d.dt, 0);
-    conv_scale(q.z, s, 0);
+    conv_scale(q.z, s, 0, s.d.dt);
     v.push_back(q);
   }
   std::vector<unsigned char> bytes;

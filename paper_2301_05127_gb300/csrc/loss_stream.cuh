@@ -19,6 +19,9 @@
 // 8 instead of 41 per junction at n_nb = 20, K = 16).  A correction reaches Q positions, where |r|^Q |D| is
 // below the working precision (host rule conv_axis in loss_step.cu); longer patches make the second term of the
 // patch-end correction, r^M D, vanish by the same rule.
+//
+// Every address formed here is a readable one, whatever the predicate it stands under: offsets are clamped to their line
+// or row, and pointers that a launch lacks are replaced on the host or excluded by a template parameter.
 #pragma once
 
 #include <cstdint>
@@ -155,8 +158,7 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
   for (int c = 0; c <= W; ++c) issue(c);
   typename OP::Regs pr[OP::B];
 #pragma unroll
-  for (int b = 0; b < OP::B; ++b)
-    if (s0 + b < s1) op.load(pr[b], s0 + b, base + (uint32_t)(s0 + b) * sb);
+  for (int b = 0; b < OP::B; ++b) op.load(pr[b], min(s0 + b, n), base + (uint32_t)min(s0 + b, n) * sb);
   // left sums of the segment's first position
   T L[NF];
   if (s0 > 0) {
@@ -164,7 +166,7 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
     for (int f = 0; f < NF; ++f) {
       T a = T(0);
 #pragma unroll 8
-      for (int k = Conv<T>::K; k >= 1; --k) a = at_off(op.src(f), base + (uint32_t)(s0 - k) * sb) + r * a;
+      for (int k = Conv<T>::K; k >= 1; --k) a = at_off(op.src(f), base + (uint32_t)max(s0 - k, 0) * sb) + r * a;
       L[f] = a;
     }
   }
@@ -228,31 +230,9 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
           if (c + 1 + k == ce) pb[f][k] = s;
       }
     }
-    const int len = min(8, s1 - p0);
-    T e[NF][8];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      T v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = d[(j * NF + f) * 32];
-      T s = L[f];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        e[f][j] = s;
-        s = v[j] + r * s;
-      }
-      L[f] = s;
-      T t = pb[f][0] + r8 * pb[f][1];
-      if (W == 4) t += r16 * (pb[f][W - 2] + r8 * pb[f][W - 1]);
-      if (c == ce) t = Rn[f];
-#pragma unroll
-      for (int j = 7; j >= 0; --j)
-        if (c != ce || j <= le) {
-          e[f][j] = t - e[f][j];
-          t = v[j] + r * t;
-        }
-    }
-    // junction corrections: those within Q of the chunk (at most two, M >= Q + 8)
+    // Junctions within Q of the chunk (at most two, M >= Q + 8).  D r^|i - q| is added through the sums: L_i - D r^(i - q)
+    // at positions from q on (the recursion carries it along) and R_i + D r^(q - i) before q, so a junction costs an
+    // operation per chunk; only a chunk with a junction inside adds it point by point.
     while (g.ntaps && jn <= g.p && jn * g.M <= p0 + 7 + g.Q) {
       ja = jb;
       jb = jn;
@@ -263,20 +243,56 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
         fs[f] = op.src(f);
       }
       conv_junction<T, NF>(g, taps, jn, fs, base, sb, Db);
+      const int o = p0 - jn * g.M;  // before the segment's first position
+      if (o > 0)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) L[f] -= Db[f] * rs[64 + o];
       ++jn;
     }
-    const int oa = p0 - ja * g.M, ob = p0 - jb * g.M;
-    if (ja >= 0 && oa <= g.Q) {
+    const int oa = ja >= 0 ? p0 - ja * g.M : 1, ob = jb >= 0 ? p0 - jb * g.M : 1;
+    const int len = min(8, s1 - p0);
+    T e[NF][8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
+    for (int f = 0; f < NF; ++f) {
+      T v[8];
 #pragma unroll
-        for (int f = 0; f < NF; ++f) e[f][j] += Da[f] * rs[64 + oa + j];
+      for (int j = 0; j < 8; ++j) v[j] = d[(j * NF + f) * 32];
+      if (oa == 0) L[f] -= Da[f];
+      if (ob == 0) L[f] -= Db[f];
+      T s = L[f];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        e[f][j] = s;
+        s = v[j] + r * s;
+      }
+      L[f] = s;
+      T t = pb[f][0] + r8 * pb[f][1];
+      if (W == 4) t += r16 * (pb[f][W - 2] + r8 * pb[f][W - 1]);
+      if (c == ce) t = Rn[f];
+      if (oa < -7) t += Da[f] * rs[64 - oa - 7];
+      if (ob < -7) t += Db[f] * rs[64 - ob - 7];
+#pragma unroll
+      for (int j = 7; j >= 0; --j)
+        if (c != ce || j <= le) {
+          e[f][j] = t - e[f][j];
+          t = v[j] + r * t;
+        }
     }
-    if (jb >= 0 && ob <= g.Q) {
+    if (oa < 0 && oa >= -7) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
+      for (int f = 0; f < NF; ++f) {
 #pragma unroll
-        for (int f = 0; f < NF; ++f) e[f][j] += Db[f] * rs[64 + ob + j];
+        for (int j = 0; j < 8; ++j) e[f][j] += Da[f] * rs[64 + oa + j];
+        L[f] -= Da[f] * rs[64 + oa + 8];
+      }
+    }
+    if (ob < 0 && ob >= -7) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) e[f][j] += Db[f] * rs[64 + ob + j];
+        L[f] -= Db[f] * rs[64 + ob + 8];
+      }
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -286,7 +302,8 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
       for (int f = 0; f < NF; ++f) ej[f] = e[f][j];
       const uint32_t o = base + (uint32_t)(p0 + j) * sb;
       if (valid) op.apply(pr[j % OP::B], ej, p0 + j, o, outer, x);
-      if (p0 + j + OP::B < s1) op.load(pr[j % OP::B], p0 + j + OP::B, o + OP::B * sb);
+      const int pn = min(p0 + j + OP::B, n);
+      if (p0 + j + OP::B < s1) op.load(pr[j % OP::B], pn, base + (uint32_t)pn * sb);
     }
   }
   cp_async_wait<0>();
@@ -349,7 +366,10 @@ __device__ __forceinline__ void ld8(const T* __restrict__ p, bool vec, int len, 
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = j < len ? p[j] : T(0);
+    for (int j = 0; j < 8; ++j) {
+      const T u = p[min(j, max(len - 1, 0))];
+      v[j] = j < len ? u : T(0);
+    }
   }
 }
 // The first min(len, 8) of eight consecutive elements, and the ninth when len = 9.
@@ -374,37 +394,28 @@ __device__ __forceinline__ void st9(T* __restrict__ p, bool vec, int len, const 
 template <typename T>
 __device__ __forceinline__ void ld9(const T* __restrict__ p, bool vec, int len, T (&v)[9]) {
   ld8(p, vec, len, v);
-  v[8] = len > 8 ? p[8] : T(0);
+  const T* p8 = p + (len > 8 ? 8 : 0);
+  v[8] = T(0);
+  if (len > 8) v[8] = *p8;
 }
 
-// v[i] by selects on the bits (a plain conditional chain is turned into an array in local memory).
-__device__ __forceinline__ float pick9(const float (&v)[9], int i) {
-  unsigned b = 0;
-#pragma unroll
-  for (int j = 0; j < 9; ++j) b |= j == i ? __float_as_uint(v[j]) : 0u;
-  return __uint_as_float(b);
-}
-__device__ __forceinline__ double pick9(const double (&v)[9], int i) {
-  unsigned long long b = 0;
-#pragma unroll
-  for (int j = 0; j < 9; ++j) b |= j == i ? (unsigned long long)__double_as_longlong(v[j]) : 0ull;
-  return __longlong_as_double((long long)b);
-}
-
-// Samples f of a chunk (0 beyond len) -> e without its junction corrections, in place.  Called by all lanes of the
-// warp; c: chunk of the row, gl: lane of the gw-lane group, end: the chunk holds position n.
+// Samples f of a chunk (0 beyond len) -> e, in place, but for the corrections of junctions inside the chunk.  Called by
+// all lanes of the warp; c: chunk of the row, gl: lane of the gw-lane group, end: the chunk holds position n, rlen =
+// r^len; dL, dR: corrections of the junctions before and after the chunk, at its first and its last position.
 template <typename T>
-__device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, int gl, int gw, T rlen) {
+__device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, int gl, int gw, T rlen, T dL, T dR) {
   constexpr int W = Conv<T>::W;
   constexpr T r = (T)kConvR, r7 = (T)conv_pow(7), r8 = (T)conv_pow(8), r16 = (T)conv_pow(16);
   constexpr T i1r = (T)(2.0 / (1.0 - kConvR));
   const unsigned full = 0xffffffffu;
   T e[9];
-  T pa = T(0), pb = f[8], pb1;
+  T pa = f[0], pb, pb1;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) pa = f[j] + r * pa;
+  for (int j = 1; j < 8; ++j) pa = f[j] + r * pa;
+  if (len > 8) pb = f[7] + r * f[8];  // the ninth position of a row's last chunk
+  else pb = f[7];
 #pragma unroll
-  for (int j = 7; j >= 1; --j) pb = f[j] + r * pb;
+  for (int j = 6; j >= 1; --j) pb = f[j] + r * pb;
   pb1 = pb;
   pb = f[0] + r * pb;
   auto down = [&](T v, int d) {
@@ -425,23 +436,38 @@ __device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, i
   }
   u = __shfl_up_sync(full, s, 1, gw);
   s = gl == 0 ? L0 : u;
+  // (the corrections enter after the sums that neighbour chunks take, and R_n is formed without them)
+  T Rn = T(0);
+  if (end) {
+    T q = s, Ln = s, fn = f[0];
 #pragma unroll
-  for (int j = 0; j < 9; ++j) {
+    for (int j = 0; j < 8; ++j) {
+      q = f[j] + r * q;
+      if (j + 1 < len) Ln = q, fn = f[j + 1];
+    }
+    Rn = i1r * fn - Ln;
+    pb += rlen * Rn;
+  }
+  s -= dL;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
     e[j] = s;
     s = f[j] + r * s;
   }
+  e[8] = s;
   // right sums: the chunk that holds position n continues with R_n
-  T Rn = T(0);
-  if (end) {
-    Rn = len == 9 ? i1r * f[8] - e[8] : i1r * pick9(f, len - 1) - pick9(e, len - 1);
-    pb += rlen * Rn;
-  }
   t = pb + r8 * down(pb, 1);
   if (W == 4) t += r16 * down(t, 2);
   t = down(t, 1);
   if (end) t = Rn;
+  t += dR;
+  if (len > 8) {
+    const T f8 = f[8];
+    f[8] = t - e[8];
+    t = f8 + r * t;
+  }
 #pragma unroll
-  for (int j = 8; j >= 0; --j) {
+  for (int j = 7; j >= 0; --j) {
     const T fj = f[j];
     f[j] = t - e[j];
     if (j < len) t = fj + r * t;
@@ -481,13 +507,14 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
     const int c = c0 + gl;
     const int len = (k < nrow && c < c1) ? (c == rm.nch - 1 ? g.n + 1 - 8 * c : 8) : 0;
     const bool end = len > 0 && c == rm.nch - 1;
+    const int64_t gi = rb + 8 * min(c, rm.nch - 1);  // of the chunk, or for lanes beyond the row of its last one
     const T rlen = end ? (T)__ldg(g.pw + len) : T(0);
     T e[NF][9];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
 #pragma unroll
       for (int j = 0; j < 9; ++j) e[f][j] = T(0);
-      if (len > 0) ld9(op.src(f) + rb + 8 * c, rm.vec, len, e[f]);
+      if (len > 0) ld9(op.src(f) + gi, rm.vec, len, e[f]);
     }
     // junctions within Q of the own positions
     int j0 = 0, nj = 0;
@@ -518,33 +545,34 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
 #pragma unroll
           for (int j = 0; j < 8; ++j)
             if (j >= len) e[f][j] = T(0);
+      // the junctions before (or at the start of) the chunk and after it; at most one of each is within Q
+      const int ja = 8 * c / g.M, o0j = 8 * c - ja * g.M, o1j = o0j - g.M;  // the chunk's offsets from ja and ja + 1
+      const int ia = ja - j0, ib = ia + 1;
+      const bool hasa = len > 0 && ia >= 0 && ia < nj && o0j <= g.Q;
+      const bool hasb = len > 0 && ib >= 0 && ib < nj && -o1j - 8 <= g.Q;
+      const bool inb = hasb && -o1j < len;  // junction ja + 1 inside the chunk
 #pragma unroll
-      for (int f = 0; f < NF; ++f) row_solve<T>(e[f], c, len, end, gl, gw, rlen);
-      if (nj > 0 && len > 0) {
-        const int ja = 8 * c / g.M;
+      for (int f = 0; f < NF; ++f) {
+        T dL = T(0), dR = T(0);
+        if (hasa) dL = dsm[(f * nrow + k) * nj + ia] * rs[64 + o0j];
+        if (hasb && !inb) dR = dsm[(f * nrow + k) * nj + ib] * rs[64 - o1j - (len - 1)];
+        row_solve<T>(e[f], c, len, end, gl, gw, rlen, dL, dR);
+        if (inb) {
+          const T D = dsm[(f * nrow + k) * nj + ib];
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const int jj = ja + s - j0, o = 8 * c - (ja + s) * g.M;  // offset of the chunk from the junction
-          if (jj >= 0 && jj < nj && o <= g.Q && -o - 8 <= g.Q) {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              const T D = dsm[(f * nrow + k) * nj + jj];
-#pragma unroll
-              for (int j = 0; j < 9; ++j) e[f][j] += D * rs[64 + o + j];
-            }
-          }
+          for (int j = 0; j < 9; ++j) e[f][j] += D * rs[64 + o1j + j];
         }
       }
     };
     derive(op.src(0));
     const bool own = len > 0 && c >= o0 && c < o1;
-    if (own) op.chunk(e, 8 * c, len, rb + 8 * c, q);
+    if (own) op.chunk(e, 8 * c, len, gi, q);
     if constexpr (OP::TWO) {
       if (!own)  // lanes beyond the row carry no samples into the second derivative
 #pragma unroll
         for (int j = 0; j < 9; ++j) e[0][j] = T(0);
       derive(op.src2());
-      if (own) op.chunk2(e, 8 * c, len, rb + 8 * c, q);
+      if (own) op.chunk2(e, 8 * c, len, gi, q);
     }
   }
 }

@@ -151,6 +151,7 @@ struct AcXArgs {
   T s3h;             // 3 / h_x
   T dt_lo, acoef_lo, s3h_lo, b0_lo;  // rounding errors of dt, acoef, s3h, b0 (mulc; 0 in FP64)
   T sc, sc_lo;       // -acoef * b0 * s3h and its rounding error (the velocity update with constant density)
+  T sdt, sdt_lo;     // s3h * dt and its rounding error (row engine)
   T minf;
   int do_B;
   SourceArgs src;
@@ -202,6 +203,7 @@ struct ElArgs {
   T lam0, mu0, b0;
   T dt, acoef, s3h, minf;
   T dt_lo, acoef_lo, s3h_lo, lam0_lo, mu0_lo, b0_lo;  // rounding errors (mulc; 0 in FP64)
+  T st, st_lo;   // s3h times the pass's step length (dt or acoef) and its rounding error (column and row engines)
   int do_B, do_A;
   int pml;
   PmlAxis<T> pB, pA;
