@@ -18,6 +18,7 @@
 #include <string>
 #include <vector>
 
+#include "loss_fir.cuh"
 #include "loss_host.h"
 
 namespace lossk {
@@ -438,6 +439,21 @@ static loss_status_t derivative_adjoint_t(loss_ctx* h, Shot& s, int k, const T* 
   int logc, threads;
   LOSS_TRY(line_geom(h, s, k, sz, sy, &geo, &logc, &threads, 4, 0, h->lines_per_block[LOSS_KERNEL_ADJOINT],
                      adj_logc<T>(h), adj_threads<T>(h)));
+  const int kid = LOSS_KERNEL_ADJOINT;
+  if (h->lines_per_block[kid] <= 0 && h->tile_threads[kid] <= 0 && h->chunk_log2[kid] <= 0) {
+    ConvAxis ca;
+    bool ok;
+    LOSS_TRY(conv_axis(h, s, k, &ca, &ok));
+    if (ok && conv_operator_ok(s, k, s.conv[k])) {
+      ColMap cm{};
+      RowMap rm{};
+      if (k == 2) rm = row_map(h->num_sms, s, 1, ca, sy, sz, false);
+      else cm = col_map(h->num_sms, s, k, sy, sz);
+      LaunchScope ls(h, kid);
+      return cuda_check(h, launch_trans_stream<T>(ca, cm, rm, k == 2, false, g, out,
+                                                  (T)(fir_const(ca.M).a * 3.0 / s.h[k]), h->stream), "adjoint kernel");
+    }
+  }
   AdjArgs<T> a{};
   a.g = geo;
   a.tb = Tables{s.W[k], h->t32, h->t64};

@@ -400,6 +400,10 @@ static loss_status_t setup_shot(loss_ctx* h, Shot& s) {
     LOSS_TRY(cuda_check(h, cudaMemcpyAsync(s.W[k], W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice,
                                            h->stream), "copy W"));
     LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
+    // now, so that the operators may be captured on a caller's stream
+    ConvAxis g;
+    bool ok;
+    LOSS_TRY(conv_axis(h, s, k, &g, &ok));
   }
   return LOSS_OK;
 }
@@ -1346,6 +1350,18 @@ static loss_status_t run_derivative_t(loss_ctx* h, Shot& s, int k, const T* f, T
   int logc, threads;
   LOSS_TRY(line_geom(h, s, k, sz, sy, &g, &logc, &threads, d2 ? 3 : 2, 0, h->lines_per_block[LOSS_KERNEL_DERIVATIVE],
                      h->chunk_log2[LOSS_KERNEL_DERIVATIVE], h->tile_threads[LOSS_KERNEL_DERIVATIVE]));
+  // A launch shape asked for (loss_set_launch, loss_set_tile) is one of the line kernel's, and only that kernel reads
+  // a whole line before it writes one.
+  const int kid = LOSS_KERNEL_DERIVATIVE;
+  if (d1 && !phi && !overlaps(s, f, d1) && !overlaps(s, f, d2) && h->lines_per_block[kid] <= 0 && h->tile_threads[kid] <= 0 && h->chunk_log2[kid] <= 0) {
+    ConvAxis ca;
+    bool ok;
+    LOSS_TRY(conv_axis(h, s, k, &ca, &ok));
+    if (ok && conv_operator_ok(s, k, s.conv[k])) {
+      LaunchScope ls(h, LOSS_KERNEL_DERIVATIVE);
+      return deriv_stream<T>(h, s, k, ca, h->num_sms, f, d1, d2);
+    }
+  }
   DerivArgs<T> a{};
   a.g = g;
   a.tb = tables_for<T>(h, s, k);

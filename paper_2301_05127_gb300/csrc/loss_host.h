@@ -24,6 +24,14 @@ inline int force_components(uint32_t kinds) {
          ((kinds & LOSS_SRC_FORCE_Z) ? 4 : 0);
 }
 
+// Host side of an axis's tables (conv_host): the bytes to upload, laid out as double r^d (d < 64), ConvTap taps[ntaps],
+// double wd[p + 1][2 R + 1], int js[p + 2]; ok: the engines take the axis.
+struct ConvHost {
+  int Q = 0, ntaps = 0, R = 0;
+  bool ok = false;
+  size_t bytes = 0;
+};
+
 // One independent grid (shot).  Internal axis slots: 0 = z, 1 = y, 2 = x; 2-D grids have a y extent of 1.
 // Device arrays use a padded layout: x pitch px (multiple of 32 elements), y stride sy = px, z stride sz.
 struct Shot {
@@ -43,10 +51,9 @@ struct Shot {
   void* tmp[8] = {};     // derivative temporaries (acoustic: tmp[0] = d_z v3)
   double* W[3] = {};     // PMBC weights per axis slot, scaled by h/3
   double* Wd[3] = {};     // junction-correction weights of the FP32 truncated-convolution kernels (on first use)
-  // axis tables of the barrier-free engines (conv_axis, on first use): double r^d, d < 64, ConvTap
-  // taps[ntaps], int js[p + 2]
+  // axis tables of the barrier-free engines (conv_axis, on first use)
   void* conv_tab[3] = {};
-  int conv_Q[3] = {0, 0, 0}, conv_ntaps[3] = {0, 0, 0};
+  ConvHost conv[3];
   void* nu_tab[3] = {};   // non-uniform axis slot (loss_set_coordinates): PMBC weights and elimination tables
   std::vector<double> coords[3];  // the knots loss_set_coordinates gave an axis slot (empty: equally spaced)
   bool has_model = false;
@@ -237,8 +244,10 @@ struct LaunchScope {
 // Axis slot k of a shot on the barrier-free engines (loss_stream.cuh): uploads its tables on first use; *ok = false
 // when the axis does not qualify.
 loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok);
-ColMap col_map(const loss_ctx* h, const Shot& s, int k, int64_t py, int64_t pz);  // strided lines, slot 0 or 1
-RowMap row_map(const loss_ctx* h, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec);  // rows along x
+std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c);
+ConvAxis conv_axis_at(const Shot& s, int k, const ConvHost& c, const void* tab);  // the tables at a device address
+ColMap col_map(int num_sms, const Shot& s, int k, int64_t py, int64_t pz);  // strided lines, slot 0 or 1
+RowMap row_map(int num_sms, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec);  // rows along x
 loss_status_t step_shot(loss_ctx* h, Shot& s);
 loss_status_t unstagger(loss_ctx* h, Shot& s);
 loss_status_t stagger_shot(loss_ctx* h, Shot& s);
@@ -293,6 +302,25 @@ size_t tile_smem_z(const TileGeom& t, int mode, int logc);
 template <bool KAHAN>
 cudaError_t launch_xt(const AcXArgs<float>& a, const TileGeom& t, cudaStream_t st);
 size_t xt_smem(const TileGeom& t);
+// loss_kernels_deriv.cu: derivative operators on the barrier-free engines (s1 = 3 a / h, s2 = 6 / (2 sqrt(3) h^2); d2 may
+// be null), and out (+)= scale * transpose
+template <typename T>
+cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, const T* f, T* d1, T* d2,
+                                T s1, T s2, cudaStream_t st);
+template <typename T>
+cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, bool acc, const T* in,
+                                T* out, T scale, cudaStream_t st);
+// Whether the operators of axis slot k run on the engines, for tables of c.bytes bytes: those fit the static array of
+// loss_derivative_noalloc (which launches the same kernels), and the dense array fits the engines' 32-bit offsets.
+constexpr size_t kNoAllocScratchBytes = 64 * 1024;
+bool conv_operator_ok(const Shot& s, int k, const ConvHost& c);
+// Whether two dense arrays share bytes (null: no array).
+inline bool overlaps(const Shot& s, const void* a, const void* b) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b, n = (uintptr_t)(s.dense * s.esize);
+  return b && x < y + n && y < x + n;
+}
+template <typename T>
+loss_status_t deriv_stream(loss_ctx* h, const Shot& s, int k, const ConvAxis& g, int num_sms, const T* f, T* d1, T* d2);
 // loss_kernels_acstream.cu: 2-D acoustic step on the barrier-free engines
 template <typename T, bool KAHAN>
 cudaError_t launch_ac_rows(const AcXArgs<T>& a, const ConvAxis& g, const RowMap& rm, cudaStream_t st);

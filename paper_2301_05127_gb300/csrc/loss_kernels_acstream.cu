@@ -27,6 +27,7 @@ namespace lossk {
 template <typename T, bool KAHAN, bool REC, bool DOB, bool DOA, bool TAB>
 struct AcRowOp {
   static constexpr int NF = 1;
+  static constexpr bool SECOND = false;
   static constexpr bool TWO = DOB && DOA;
   static constexpr int kBlocks = sizeof(T) == 8 ? 3 : 4;
   AcXArgs<T> a;
@@ -189,6 +190,7 @@ struct AcRowOp {
 template <typename T, int MODE, bool REC>
 struct AcColOp {
   static constexpr int NF = 1;
+  static constexpr bool SECOND = false;
   static constexpr int kBlocks = 4;
   static constexpr int B = MODE == 1 ? 4 : 1;
   AcZArgs<T> a;

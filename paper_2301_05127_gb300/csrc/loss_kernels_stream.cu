@@ -22,6 +22,7 @@ namespace lossk {
 template <typename T, int PASS, bool KAHAN, bool REC>
 struct ElColOp {
   static constexpr int NF = 3;
+  static constexpr bool SECOND = false;
   static constexpr int kBlocks = sizeof(T) == 4 ? 4 : 1;
   static constexpr int B = PASS == ES_AZ || PASS == ES_BY ? 4 : 2;
   ElArgs<T> a;
@@ -155,6 +156,7 @@ struct ElColOp {
 template <typename T, int PASS, bool REC>
 struct ElRowOp {
   static constexpr int NF = 3;
+  static constexpr bool SECOND = false;
   static constexpr bool TWO = false;
   static constexpr int kBlocks = sizeof(T) == 4 ? (REC ? 3 : 4) : 2;
   ElArgs<T> a;

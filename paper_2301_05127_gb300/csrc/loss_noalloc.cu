@@ -18,8 +18,8 @@
 
 namespace lossk {
 
-// 64 KiB: PMBC weights ((p + 1) * (2 n_nb + 1) doubles) followed by the two Thomas tables.
-constexpr size_t kNoAllocScratchBytes = 64 * 1024;
+// kNoAllocScratchBytes = 64 KiB: the tables of the barrier-free engines, or PMBC weights ((p + 1) * (2 n_nb + 1) doubles)
+// followed by the two Thomas tables.
 constexpr size_t kNoAllocTableBytes = kTableLen * (sizeof(double) + sizeof(float));
 constexpr size_t kNoAllocMaxWeights = (kNoAllocScratchBytes - kNoAllocTableBytes) / sizeof(double);
 
@@ -48,6 +48,17 @@ template <typename T>
 static loss_status_t noalloc_run(loss_ctx* h, Shot& s, int k, const T* f, T* d1, unsigned char* scratch) {
   const std::vector<double> W = pmbc_weights_scaled((int)s.n[k], s.p[k], s.d.n_nb);
   if (W.size() > kNoAllocMaxWeights) return LOSS_E_UNSUPPORTED;
+  LineGeom g;
+  int logc, threads;
+  loss_status_t st = line_geom(h, s, k, s.len[2] * s.len[1], s.len[2], &g, &logc, &threads, 2, 0, 0, 0);
+  if (st != LOSS_OK) return st;
+  ConvHost ch;
+  const std::vector<unsigned char> blob = conv_host(s, k, &ch);
+  if (conv_operator_ok(s, k, ch) && !overlaps(s, f, d1)) {  // the kernels that loss_derivative takes for this axis
+    if (cudaMemcpyAsync(scratch, blob.data(), blob.size(), cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
+      return LOSS_E_CUDA;
+    return deriv_stream<T>(h, s, k, conv_axis_at(s, k, ch, scratch), h->num_sms, f, d1, nullptr);
+  }
   std::vector<double> t64;
   std::vector<float> t32;
   thomas_tables(t64, t32);
@@ -59,11 +70,6 @@ static loss_status_t noalloc_run(loss_ctx* h, Shot& s, int k, const T* f, T* d1,
       cudaMemcpyAsync(d_t32, t32.data(), kTableLen * sizeof(float), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
       cudaMemcpyAsync(d_W, W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
     return LOSS_E_CUDA;
-  const int64_t sy = s.len[2], sz = s.len[2] * s.len[1];
-  LineGeom g;
-  int logc, threads;
-  loss_status_t st = line_geom(h, s, k, sz, sy, &g, &logc, &threads, 2, 0, 0, 0);
-  if (st != LOSS_OK) return st;
   DerivArgs<T> a{};
   a.g = g;
   a.tb = Tables{d_W, d_t32, d_t64};
@@ -94,15 +100,17 @@ extern "C" loss_status_t loss_derivative_noalloc(const loss_grid_desc_t* desc, i
   loss_status_t st = validate(geo, &why);
   if (st != LOSS_OK) return st;
   if (axis < 0 || axis >= desc->dim) return LOSS_E_ARG;
-  int dev = 0, smem = 0;
+  int dev = 0, smem = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return LOSS_E_CUDA;
   if (cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return LOSS_E_CUDA;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LOSS_E_CUDA;
   void* scratch = nullptr;
   if (scratch_address(dev, &scratch) != cudaSuccess) return LOSS_E_CUDA;
   loss_ctx ctx;  // host-side launch parameters only; nothing is allocated on the device
   ctx.stream = (cudaStream_t)cuda_stream;
   ctx.device = dev;
   ctx.smem_optin = smem;
+  ctx.num_sms = sms;
   Shot s;
   s.d = geo;
   shot_geometry(s);

@@ -256,7 +256,7 @@ static loss_status_t acs_rows(loss_ctx* h, Shot& s, int do_B, double acoef, doub
   AcXArgs<T> a = ac_x_args<T>(h, s, LineGeom{}, do_B, acoef, amp);
   conv_scale(a, s, 2, acoef);
   LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
-  return cuda_check(h, launch_ac_rows<T, K>(a, g, row_map(h, s, 1, g, s.sy, s.sz, true), h->stream), "acoustic x kernel");
+  return cuda_check(h, launch_ac_rows<T, K>(a, g, row_map(h->num_sms, s, 1, g, s.sy, s.sz, true), h->stream), "acoustic x kernel");
 }
 // Z1 (mode 1) or Z2 (mode 2) of the FP64 step on the engines.
 static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
@@ -266,7 +266,7 @@ static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
   AcZArgs<double> a = ac_z_args<double>(h, s, LineGeom{}, acoef, 0);
   conv_scale(a, s, 0, acoef);
   LaunchScope ls(h, mode == 1 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2);
-  return cuda_check(h, launch_ac_cols(a, g, col_map(h, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
+  return cuda_check(h, launch_ac_cols(a, g, col_map(h->num_sms, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
 }
 
 // x part of the FP32 step (sub-step B and the x part of A, or the latter alone): the pipelined row kernel when a
@@ -548,73 +548,94 @@ static loss_status_t elt_pass(loss_ctx* h, Shot& s, int pass, double acoef, doub
 
 // ---------------------------------------------------------------------------------------------------------------
 // Axes of the barrier-free engines (loss_stream.cuh).
-loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok) {
+std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
   const int n = (int)s.n[k], p = s.p[k], M = n / p;
-  *ok = false;
-  if (n < 40) return LOSS_OK;  // the line ends' closed forms need whole warm-up sums beside them
-  if (!s.conv_tab[k]) {
-    const bool f32 = s.esize == 4;
-    const int K = f32 ? 16 : 32;
-    const int R = std::max(s.d.n_nb, K), wl = 2 * R + 1;
-    const std::vector<double> D = fir_delta_weights(n, p, s.d.n_nb, K);
-    const double a = fir_const(M).a;
-    // weights that are rounding noise of the difference (or reach less than the last digit) are left out
-    const double tiny = f32 ? 0x1p-44 : 0x1p-52;
-    std::vector<int> js(p + 2, 0);
-    std::vector<ConvTap> taps;
-    double dmax = 0.0;
-    for (int j = 0; j <= p; ++j) {
-      js[j] = (int)taps.size();
-      double sum = 0.0;
-      for (int m = -R; m <= R; ++m) {
-        const double w = D[(size_t)j * wl + R + m];
-        if (std::fabs(w) <= tiny) continue;
-        taps.push_back(ConvTap{w / a, m, 0});
-        sum += std::fabs(w) / a;
-      }
-      dmax = std::max(dmax, sum);
+  *c = ConvHost{};
+  if (n < 40) return {};  // the line ends' closed forms need whole warm-up sums beside them
+  const bool f32 = s.esize == 4;
+  const int K = f32 ? 16 : 32;
+  const int R0 = std::max(s.d.n_nb, K), wl = 2 * R0 + 1;
+  const std::vector<double> D = fir_delta_weights(n, p, s.d.n_nb, K);
+  const double a = fir_const(M).a;
+  // weights that are rounding noise of the difference (or reach less than the last digit) are left out
+  const double tiny = f32 ? 0x1p-44 : 0x1p-52;
+  std::vector<int> js(p + 2, 0);
+  std::vector<ConvTap> taps;
+  double dmax = 0.0;
+  for (int j = 0; j <= p; ++j) {
+    js[j] = (int)taps.size();
+    double sum = 0.0;
+    for (int m = -R0; m <= R0; ++m) {
+      const double w = D[(size_t)j * wl + R0 + m];
+      if (std::fabs(w) <= tiny) continue;
+      taps.push_back(ConvTap{w / a, m, 0});
+      c->R = std::max(c->R, std::abs(m));
+      sum += std::fabs(w) / a;
     }
-    js[p + 1] = (int)taps.size();
-    // reach of a correction: |r|^Q dmax below the working precision
-    const double eps = f32 ? 0x1p-40 : 0x1p-58;
-    int Q = 0;
-    for (double q = dmax; q > eps && Q < 64; q *= -kConvRHost) ++Q;
-    const size_t o1 = 64 * sizeof(double), o2 = o1 + taps.size() * sizeof(ConvTap);
-    std::vector<unsigned char> blob(o2 + js.size() * sizeof(int));
-    double pw[64];
-    pw[0] = 1.0;
-    for (int i = 1; i < 64; ++i) pw[i] = pw[i - 1] * kConvRHost;
-    std::memcpy(blob.data(), pw, sizeof(pw));
-    if (!taps.empty()) std::memcpy(blob.data() + o1, taps.data(), taps.size() * sizeof(ConvTap));
-    std::memcpy(blob.data() + o2, js.data(), js.size() * sizeof(int));
+    dmax = std::max(dmax, sum);
+  }
+  js[p + 1] = (int)taps.size();
+  // reach of a correction: |r|^Q dmax below the working precision
+  const double eps = f32 ? 0x1p-40 : 0x1p-58;
+  for (double q = dmax; q > eps && c->Q < 64; q *= -kConvRHost) ++c->Q;
+  c->ntaps = (int)taps.size();
+  c->ok = M >= c->Q + 8 && c->Q <= 48;
+  const int wr = 2 * c->R + 1;
+  std::vector<double> wd((size_t)(p + 1) * wr, 0.0);
+  for (int j = 0; j <= p; ++j)
+    for (int t = js[j]; t < js[j + 1]; ++t) wd[(size_t)j * wr + c->R + taps[t].m] = taps[t].w;
+  double pw[64];
+  pw[0] = 1.0;
+  for (int i = 1; i < 64; ++i) pw[i] = pw[i - 1] * kConvRHost;
+  std::vector<unsigned char> blob;
+  auto put = [&](const void* q, size_t nb) {
+    const unsigned char* b = (const unsigned char*)q;
+    blob.insert(blob.end(), b, b + nb);
+  };
+  put(pw, sizeof(pw));
+  put(taps.data(), taps.size() * sizeof(ConvTap));
+  put(wd.data(), wd.size() * sizeof(double));
+  put(js.data(), js.size() * sizeof(int));
+  c->bytes = blob.size();
+  return blob;
+}
+ConvAxis conv_axis_at(const Shot& s, int k, const ConvHost& c, const void* tab) {
+  ConvAxis g{};
+  g.n = (int)s.n[k], g.p = s.p[k], g.M = g.n / g.p, g.Q = c.Q, g.ntaps = c.ntaps, g.R = c.R;
+  g.pw = (const double*)tab;
+  g.taps = (const ConvTap*)(g.pw + 64);
+  g.wd = (const double*)(g.taps + g.ntaps);
+  g.js = (const int*)(g.wd + (size_t)(g.p + 1) * (2 * g.R + 1));
+  return g;
+}
+loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok) {
+  *ok = false;
+  if (s.n[k] < 40) return LOSS_OK;
+  if (!s.conv_tab[k]) {
+    const std::vector<unsigned char> blob = conv_host(s, k, &s.conv[k]);
     void* d = nullptr;
     LOSS_TRY(dev_alloc(h, blob.size(), &d));
     LOSS_TRY(cuda_check(h, cudaMemcpyAsync(d, blob.data(), blob.size(), cudaMemcpyHostToDevice, h->stream),
                         "copy junction taps"));
     LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
     s.conv_tab[k] = d;
-    s.conv_Q[k] = Q;
-    s.conv_ntaps[k] = (int)taps.size();
   }
-  g->n = n, g->p = p, g->M = M, g->Q = s.conv_Q[k], g->ntaps = s.conv_ntaps[k];
-  g->pw = (const double*)s.conv_tab[k];
-  g->taps = (const ConvTap*)(g->pw + 64);
-  g->js = (const int*)(g->taps + g->ntaps);
-  *ok = M >= g->Q + 8 && g->Q < 64;
+  *g = conv_axis_at(s, k, s.conv[k], s.conv_tab[k]);
+  *ok = s.conv[k].ok;
   return LOSS_OK;
 }
 
 // Strided lines of an array with row pitch py and plane pitch pz.  A line is cut into segments when there are too few
 // lines to fill the GPU (about 16 warps per SM); a segment re-reads K positions before it and 8 (W + 1) after it, so
 // it keeps at least 40 positions.
-ColMap col_map(const loss_ctx* h, const Shot& s, int k, int64_t py, int64_t pz) {
+ColMap col_map(int num_sms, const Shot& s, int k, int64_t py, int64_t pz) {
   ColMap m{};
   m.inner = s.len[2];
   m.lines = s.dense / s.len[k];
   m.groups = (m.lines + 31) / 32;
   m.so = k == 1 ? pz : py;
   m.stride = k == 1 ? py : pz;
-  const int64_t want = 16LL * h->num_sms;
+  const int64_t want = 16LL * num_sms;
   const int np = (int)s.n[k] + 1;
   const int nseg = (int)std::min<int64_t>(std::max<int64_t>(want / m.groups, 1), std::max(np / 40, 1));
   m.seglen = ((np + nseg - 1) / nseg + 7) & ~7;
@@ -622,7 +643,7 @@ ColMap col_map(const loss_ctx* h, const Shot& s, int k, int64_t py, int64_t pz) 
   return m;
 }
 
-RowMap row_map(const loss_ctx* h, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec) {
+RowMap row_map(int num_sms, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec) {
   RowMap m{};
   const int es = (int)s.esize, W = es == 4 ? 2 : 4;
   m.rows = (int)(s.len[0] * s.len[1]);
@@ -635,11 +656,32 @@ RowMap row_map(const loss_ctx* h, const Shot& s, int nf, const ConvAxis& g, int6
   m.nwin = m.nch <= 32 ? 1 : 1 + (m.nch - 32 + 31 - 2 * W) / (32 - 2 * W);
   m.groups = (m.rows + 32 / m.gw - 1) / (32 / m.gw);
   m.vec = vec ? 1 : 0;
-  const int nj = std::min(g.p + 1, (8 * m.gw + 1 + 2 * g.Q) / g.M + 2);
+  const int nj = std::min(g.p + 1, (8 * m.gw + 1 + 2 * std::max(g.Q, g.R)) / g.M + 2);
   m.wbytes = (nf * (32 / m.gw) * nj * es + 15) & ~15;
-  m.sms = h->num_sms;
+  m.sms = num_sms;
   return m;
 }
+
+bool conv_operator_ok(const Shot& s, int k, const ConvHost& c) {
+  return c.ok && c.bytes <= kNoAllocScratchBytes && (uint64_t)s.dense * s.esize <= UINT32_MAX &&
+         s.len[0] * s.len[1] * ((s.n[2] + 191) / 192) < INT32_MAX / 2 && 4 * (s.n[k] / s.p[k]) > 8 + 2 * c.R;
+}
+// d1 (and d2) along slot k of dense arrays.
+template <typename T>
+loss_status_t deriv_stream(loss_ctx* h, const Shot& s, int k, const ConvAxis& g, int num_sms, const T* f, T* d1, T* d2) {
+  const int64_t py = s.len[2], pz = s.len[2] * s.len[1];
+  const double hk = s.h[k];
+  ColMap cm{};
+  RowMap rm{};
+  if (k == 2) rm = row_map(num_sms, s, 1, g, py, pz, false);
+  else cm = col_map(num_sms, s, k, py, pz);
+  return cuda_check(h, launch_deriv_stream<T>(g, cm, rm, k == 2, f, d1, d2, (T)(fir_const(g.M).a * 3.0 / hk),
+                                              (T)(6.0 / (2.0 * 1.7320508075688772 * hk * hk)), h->stream),
+                    "derivative kernel");
+}
+template loss_status_t deriv_stream<float>(loss_ctx*, const Shot&, int, const ConvAxis&, int, const float*, float*, float*);
+template loss_status_t deriv_stream<double>(loss_ctx*, const Shot&, int, const ConvAxis&, int, const double*, double*,
+                                            double*);
 
 // The elastic step on those engines: the convolution family (loss_set_kernels) when every axis qualifies.  The line
 // kernels' limit on the length of a row stays the limit of the step.
@@ -677,8 +719,8 @@ static loss_status_t els_pass(loss_ctx* h, Shot& s, int pass, double acoef, doub
   LOSS_TRY(conv_axis(h, s, k, &g, &ok));
   ColMap cm{};
   RowMap rm{};
-  if (k == 2) rm = row_map(h, s, 3, g, s.sy, s.sz, true);
-  else cm = col_map(h, s, k, s.sy, s.sz);
+  if (k == 2) rm = row_map(h->num_sms, s, 3, g, s.sy, s.sz, true);
+  else cm = col_map(h->num_sms, s, k, s.sy, s.sz);
   LaunchScope ls(h, k == 2 ? LOSS_KERNEL_ELASTIC_X : (k == 1 ? LOSS_KERNEL_ELASTIC_Y : LOSS_KERNEL_ELASTIC_Z));
   return cuda_check(h, launch_el_stream<T, K>(a, g, cm, rm, pass, h->stream), "elastic kernel");
 }
@@ -1160,8 +1202,8 @@ static loss_status_t acs_tables(loss_ctx* h) {
     bool ok;
     LOSS_TRY(conv_axis(h, s, 2, &q.gx, &ok));
     LOSS_TRY(conv_axis(h, s, 0, &q.gz, &ok));
-    q.rm = row_map(h, s, 1, q.gx, s.sy, s.sz, true);
-    q.cm = col_map(h, s, 0, s.sy, s.sz);
+    q.rm = row_map(h->num_sms, s, 1, q.gx, s.sy, s.sz, true);
+    q.cm = col_map(h->num_sms, s, 0, s.sy, s.sz);
     q.x = ac_x_args<double>(h, s, LineGeom{}, 1, s.d.dt, 0.0);
     q.x.src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
     q.x.src.amp_tab = s.amp_tab;

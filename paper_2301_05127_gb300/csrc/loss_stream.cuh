@@ -108,6 +108,20 @@ __device__ __forceinline__ void copy_job(J* dst, const J* __restrict__ src) {
     reinterpret_cast<uint64_t*>(dst)[i] = reinterpret_cast<const uint64_t*>(src)[i];
 }
 
+// Correction of the second derivative by a junction at offset o of the chunk: slopes that differ by D r^|i - q| shift the
+// scaled second derivative f_i + r (R_i + L_i) by -6 a D sgn(i - q) r^|i - q| (at the junction itself the two patches' values
+// average to 0; a line end has one patch).
+template <typename T, int N>
+__device__ __forceinline__ void add_second(T (&v)[N], T D, int o, int j, const ConvAxis& g, const T* rs) {
+  const T w = (T)(6.0 * kConvR) * D;  // a = -r
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int d = o + i;
+    const T sg = d > 0 ? T(1) : (d < 0 ? T(-1) : (j == 0 ? T(1) : (j == g.p ? T(-1) : T(0))));
+    v[i] += w * sg * rs[64 + d];
+  }
+}
+
 // ---------------------------------------------------------------------------------------------------------------
 // Strided lines.  Line q (0 .. lines - 1) starts at (q / inner) * so + q % inner and steps by `stride`; it is cut into
 // segments of seglen positions (a multiple of 8, nseg of them), each marched by one thread.
@@ -119,7 +133,7 @@ __device__ __forceinline__ void copy_job(J* dst, const J* __restrict__ src) {
 template <typename T, class OP>
 __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, const OP& op, int bid,
                                           unsigned char* sm) {
-  constexpr int NF = OP::NF, W = Conv<T>::W, NR = W + 2;
+  constexpr int NF = OP::NF, W = Conv<T>::W, LA = W + (OP::SECOND ? 1 : 0), NR = LA + 2;
   constexpr T r = (T)kConvR, r7 = (T)conv_pow(7), r8 = (T)conv_pow(8), r16 = (T)conv_pow(16);
   constexpr T i1r = (T)(2.0 / (1.0 - kConvR));
   __shared__ T rs[kReach];
@@ -155,7 +169,7 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
     cp_async_commit();
   };
 #pragma unroll
-  for (int c = 0; c <= W; ++c) issue(c);
+  for (int c = 0; c <= LA; ++c) issue(c);
   typename OP::Regs pr[OP::B];
 #pragma unroll
   for (int b = 0; b < OP::B; ++b) op.load(pr[b], min(s0 + b, n), base + (uint32_t)min(s0 + b, n) * sb);
@@ -191,16 +205,56 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
     }
   };
   cp_async_wait<0>();
+  // second differences (field 0): sample i of the segment, and the sums of the next chunks as for the samples
+  T pb2[W], L2 = T(0), Rn2 = T(0);
+  T fprev = T(0);  // the sample before the chunk
+  auto val = [&](int i) { return slot(i >> 3)[(i & 7) * NF * 32]; };
+  auto sums2 = [&](int c, int k) {
+    T a = T(0);
+    if (c < ce) {
+      T fp = val(8 * c + 8), f0 = val(8 * c + 7);
+#pragma unroll
+      for (int j = 7; j >= 0; --j) {
+        const T fm = val(8 * c + j - 1);
+        a = ((fp - f0) - (f0 - fm)) + r * a;
+        fp = f0;
+        f0 = fm;
+      }
+    }
+    pb2[k] = a;
+  };
+  if constexpr (OP::SECOND) {
+    if (s0 > 0) {
+      const T* f = op.src(0);
+      auto at = [&](int i) { return at_off(f, base + (uint32_t)max(i, 0) * sb); };
+      fprev = at(s0 - 1);
+      T fm = at(s0 - Conv<T>::K - 1), f0 = at(s0 - Conv<T>::K);
+#pragma unroll 8
+      for (int k = Conv<T>::K; k >= 1; --k) {
+        const T fp = at(s0 - k + 1);
+        L2 = ((fp - f0) - (f0 - fm)) + r * L2;
+        fm = f0;
+        f0 = fp;
+      }
+    }
+#pragma unroll
+    for (int c = 1; c < W; ++c) sums2(c, c);
+  }
 #pragma unroll
   for (int c = 1; c < W; ++c) sums(c, c);  // shifted down by the first iteration
   for (int c = 0; c < nc; ++c) {
-    issue(c + W + 1);
+    issue(c + LA + 1);
     cp_async_wait<1>();
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
       for (int k = 0; k + 1 < W; ++k) pb[f][k] = pb[f][k + 1];
     sums(c + W, W - 1);
+    if constexpr (OP::SECOND) {
+#pragma unroll
+      for (int k = 0; k + 1 < W; ++k) pb2[k] = pb2[k + 1];
+      sums2(c + W, W - 1);
+    }
     const T* d = slot(c);
     const int p0 = s0 + 8 * c;
     if (c == 0 && s0 == 0) {  // odd reflection at the line's start (n >= 40: chunks 0 .. W are whole)
@@ -212,6 +266,34 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
 #pragma unroll
         for (int j = 7; j >= 1; --j) b = d[(j * NF + f) * 32] + r * b;
         L[f] = i1r * d[f * 32] - (b + r7 * a);
+      }
+    }
+    if constexpr (OP::SECOND) {
+      if (c == 0 && s0 == 0) {
+        T a = pb2[0] + r8 * pb2[1];
+        if (W == 4) a += r16 * (pb2[W - 2] + r8 * pb2[W - 1]);
+        T b = T(0);
+#pragma unroll
+        for (int j = 7; j >= 1; --j) b = ((val(j + 1) - val(j)) - (val(j) - val(j - 1))) + r * b;
+        L2 = -(b + r7 * a);
+      }
+      if (!tailed && c + W >= ce) {
+        T s = L2, fm = fprev, f0 = val(8 * c);
+        for (int i = 8 * c; i < n - s0; ++i) {
+          const T fp = val(i + 1);
+          s = (i + s0 == 0 ? T(0) : (fp - f0) - (f0 - fm)) + r * s;
+          fm = f0;
+          f0 = fp;
+        }
+        Rn2 = -s;
+        s = r * Rn2;  // position n has second difference 0
+        for (int j = le - 1; j >= 0; --j) {
+          const int i = 8 * ce + j;
+          s = ((val(i + 1) - val(i)) - (val(i) - val(max(i - 1, 0)))) + r * s;
+        }
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+          if (c + 1 + k == ce) pb2[k] = s;
       }
     }
     if (!tailed && c + W >= ce) {  // R_n, and the sum of chunk ce with its reflected continuation
@@ -278,6 +360,39 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
           t = v[j] + r * t;
         }
     }
+    if constexpr (OP::SECOND) {
+      T v2[8], fm = fprev, f0 = d[0];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const T fp = j < 7 ? d[(j + 1) * NF * 32] : val(8 * c + 8);
+        const int i = p0 + j;
+        v2[j] = i > 0 && i < n ? (fp - f0) - (f0 - fm) : T(0);
+        fm = f0;
+        f0 = fp;
+      }
+      fprev = fm;
+      T e2[8], s = L2;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        e2[j] = s;
+        s = v2[j] + r * s;
+      }
+      L2 = s;
+      T t = pb2[0] + r8 * pb2[1];
+      if (W == 4) t += r16 * (pb2[W - 2] + r8 * pb2[W - 1]);
+      if (c == ce) t = Rn2;
+#pragma unroll
+      for (int j = 7; j >= 0; --j)
+        if (c != ce || j <= le) {
+          e2[j] = v2[j] + r * (t + e2[j]);
+          t = v2[j] + r * t;
+        }
+      if (ja >= 0 && oa <= g.Q) add_second(e2, Da[0], oa, ja, g, rs);
+      if (jb >= 0 && ob <= g.Q) add_second(e2, Db[0], ob, jb, g, rs);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j < len && valid) op.apply2nd(e2[j], base + (uint32_t)(p0 + j) * sb);
+    }
     if (oa < 0 && oa >= -7) {
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
@@ -336,7 +451,9 @@ __global__ void __launch_bounds__(128, OP::kBlocks)
 
 // Dynamic shared memory of a k_col block.
 template <typename T>
-constexpr size_t col_smem(int nf) { return (size_t)4 * (Conv<T>::W + 2) * 8 * nf * 32 * sizeof(T); }
+constexpr size_t col_smem(int nf, bool second = false) {
+  return (size_t)4 * (Conv<T>::W + 2 + (second ? 1 : 0)) * 8 * nf * 32 * sizeof(T);
+}
 
 // ---------------------------------------------------------------------------------------------------------------
 // Contiguous rows.  Row q (0 .. rows - 1) starts at (q / ny) * sz + (q % ny) * sy.  A row has nch chunks of 8 positions,
@@ -399,14 +516,19 @@ __device__ __forceinline__ void ld9(const T* __restrict__ p, bool vec, int len, 
   if (len > 8) v[8] = *p8;
 }
 
-// Samples f of a chunk (0 beyond len) -> e, in place, but for the corrections of junctions inside the chunk.  Called by
-// all lanes of the warp; c: chunk of the row, gl: lane of the gw-lane group, end: the chunk holds position n, rlen =
-// r^len; dL, dR: corrections of the junctions before and after the chunk, at its first and its last position.
-template <typename T>
+// What a solve forms of the samples f of a chunk (0 beyond len), in place:
+//   kFirst:  R_i - L_i (the first derivative over a, but for junctions inside the chunk);
+//   kSecond: f_i + r (R_i + L_i), the second derivative's convolution of the second differences f;
+//   kTrans:  L_i - R_i over zeros beyond the ends, plus the transpose of the odd reflection: with E_0 = sum r^i f_i it
+//            is a r^(i-1) E_0 at i > 0 (as if L_0 were E_0 / r) and -2 E_0 / (1 - r) at i = 0; at n with the sign reversed.
+// Called by all lanes of the warp; c: chunk of the row, gl: lane of the gw-lane group, end: the chunk holds position n,
+// rlen = r^len; dL, dR: corrections of the junctions before and after the chunk, at its first and its last position.
+enum { kFirst = 0, kSecond = 1, kTrans = 2 };
+template <typename T, int MODE = kFirst>
 __device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, int gl, int gw, T rlen, T dL, T dR) {
   constexpr int W = Conv<T>::W;
   constexpr T r = (T)kConvR, r7 = (T)conv_pow(7), r8 = (T)conv_pow(8), r16 = (T)conv_pow(16);
-  constexpr T i1r = (T)(2.0 / (1.0 - kConvR));
+  constexpr T i1r = (T)(2.0 / (1.0 - kConvR)), ir = (T)(1.0 / kConvR);
   const unsigned full = 0xffffffffu;
   T e[9];
   T pa = f[0], pb, pb1;
@@ -426,7 +548,8 @@ __device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, i
   T t = pb + r8 * down(pb, 1);
   if (W == 4) t += r16 * down(t, 2);
   const T R0 = pb1 + r7 * down(t, 1);
-  const T l0 = c == 0 ? i1r * f[0] - R0 : T(0);
+  const T E0 = t;
+  const T l0 = c == 0 ? (MODE == kTrans ? ir * E0 : i1r * f[0] - R0) : T(0);
   const T L0 = __shfl_sync(full, l0, 0, gw);  // 0 in windows that do not start the row
   T u = __shfl_up_sync(full, pa, 1, gw);
   T s = pa + r8 * (gl == 0 ? L0 : u);
@@ -437,7 +560,7 @@ __device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, i
   u = __shfl_up_sync(full, s, 1, gw);
   s = gl == 0 ? L0 : u;
   // (the corrections enter after the sums that neighbour chunks take, and R_n is formed without them)
-  T Rn = T(0);
+  T Rn = T(0), endv = T(0);
   if (end) {
     T q = s, Ln = s, fn = f[0];
 #pragma unroll
@@ -445,7 +568,13 @@ __device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, i
       q = f[j] + r * q;
       if (j + 1 < len) Ln = q, fn = f[j + 1];
     }
-    Rn = i1r * fn - Ln;
+    if constexpr (MODE == kTrans) {
+      const T En = fn + r * Ln;
+      Rn = ir * En;
+      endv = Ln + i1r * En;
+    } else {
+      Rn = i1r * fn - Ln;
+    }
     pb += rlen * Rn;
   }
   s -= dL;
@@ -461,16 +590,24 @@ __device__ __forceinline__ void row_solve(T (&f)[9], int c, int len, bool end, i
   t = down(t, 1);
   if (end) t = Rn;
   t += dR;
+  auto out = [&](T fj, T lj, T rj) { return MODE == kFirst ? rj - lj : (MODE == kSecond ? fj + r * (rj + lj) : lj - rj); };
   if (len > 8) {
     const T f8 = f[8];
-    f[8] = t - e[8];
+    f[8] = out(f8, e[8], t);
     t = f8 + r * t;
   }
 #pragma unroll
   for (int j = 7; j >= 0; --j) {
     const T fj = f[j];
-    f[j] = t - e[j];
+    f[j] = out(fj, e[j], t);
+    if (MODE == kTrans && j == 0 && c == 0) f[0] = -t - i1r * E0;
     if (j < len) t = fj + r * t;
+  }
+  if constexpr (MODE == kTrans) {
+    if (end)
+#pragma unroll
+      for (int j = 0; j < 9; ++j)
+        if (j == len - 1) f[j] = endv;
   }
 }
 
@@ -564,9 +701,33 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
         }
       }
     };
-    derive(op.src(0));
     const bool own = len > 0 && c >= o0 && c < o1;
+    T q2[9];
+    if constexpr (OP::SECOND) {  // second differences, 0 at the line's ends
+      const T fm = __shfl_up_sync(0xffffffffu, e[0][7], 1, gw), fp = __shfl_down_sync(0xffffffffu, e[0][0], 1, gw);
+#pragma unroll
+      for (int j = 0; j < 9; ++j) {
+        const T m = j == 0 ? fm : e[0][j - 1];
+        const T p = j == 8 ? T(0) : (j == 7 ? (len > 8 ? e[0][8] : fp) : e[0][j + 1]);
+        const bool in = j < len && !(c == 0 && j == 0) && !(end && j == len - 1);
+        q2[j] = in ? (p - e[0][j]) - (e[0][j] - m) : T(0);
+      }
+    }
+    derive(op.src(0));
     if (own) op.chunk(e, 8 * c, len, gi, q);
+    if constexpr (OP::SECOND) {
+      row_solve<T, kSecond>(q2, c, len, end, gl, gw, rlen, T(0), T(0));
+      if (nj > 0 && len > 0) {
+        const int ja = 8 * c / g.M;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const int jj = ja + s - j0, o = 8 * c - (ja + s) * g.M;
+          if (jj >= 0 && jj < nj && o <= g.Q && -o - 8 <= g.Q)
+            add_second(q2, dsm[k * nj + jj], o, ja + s, g, rs);
+        }
+      }
+      if (own) op.chunk2nd(q2, 8 * c, len, gi);
+    }
     if constexpr (OP::TWO) {
       if (!own)  // lanes beyond the row carry no samples into the second derivative
 #pragma unroll

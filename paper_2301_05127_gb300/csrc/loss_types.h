@@ -289,7 +289,7 @@ struct ElTile {
 };
 // Axis of the barrier-free engines (loss_stream.cuh): n intervals in p patches of M; the taps of junction j are
 // taps[js[j]] .. taps[js[j + 1] - 1] (weights over a, offsets m from the junction), ntaps in all; a junction's correction
-// reaches Q positions; pw: r^d, d = 0 .. 63.
+// reaches Q positions; pw: r^d, d = 0 .. 63; wd: the same weights dense, [p + 1][2 R + 1] for the offsets -R .. R.
 struct ConvTap {
   double w;
   int m;
@@ -300,6 +300,8 @@ struct ConvAxis {
   const int* js;
   const ConvTap* taps;
   const double* pw;
+  const double* wd;
+  int R, pad;
 };
 // Strided lines of an array: line q starts at (q / inner) * so + q % inner and steps by stride; groups of 32 lines,
 // nseg segments of seglen positions per line.

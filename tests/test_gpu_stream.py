@@ -143,3 +143,47 @@ def test_batched_fp64_equals_per_shot(pkg, graph, mixed):
     for s in range(len(ws)):
         for a, b in zip(res[0][s], res[1][s]):
             assert np.array_equal(a, b), s
+
+
+# (n, p, n_nb) of two or three axes: segments of 40 positions and more, two row windows, a 9-point last chunk, the
+# shortest line and patch, patches that overlap in three junctions' reach, odd row lengths (unaligned rows)
+OPERATORS = [((40, 41), (1, 1), 8), ((257, 510), (1, 17), 20), ((512, 264), (16, 8), 12), ((44, 40, 63), (1, 2, 1), 9),
+             ((120, 48, 72), (5, 2, 3), 16)]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("geom", range(len(OPERATORS)))
+def test_derivative_operators(pkg, prec, geom):
+    """First and second derivative and the transpose against the oracle (tolerances of the derivative tests), device
+    arrays at an odd element offset; written over their input they give the same."""
+    import torch
+
+    from oracle import spline
+
+    n, p, n_nb = OPERATORS[geom]
+    h = tuple(1.0 + 0.5 * k for k in range(len(n)))
+    t1, t2 = (1e-12, 1e-11) if prec == "fp64" else (2e-5, 2e-4)
+    g = pkg.Grid([pkg.make_desc(len(n), pkg.LOSS_ACOUSTIC, pkg.PRECISIONS[prec], n_nb, n, p, h, 1e-3)])
+    rng = np.random.default_rng(geom)
+    f = (rng.standard_normal(g.shape()) + 5.0 * np.sin(np.linspace(0, 9, g.shape()[-1]))).astype(g.dtype)
+    dev = torch.empty(f.size + 1, dtype=torch.float64 if prec == "fp64" else torch.float32, device="cuda")[1:]
+    dev = dev.view(f.shape)
+    dev.copy_(torch.from_numpy(f))
+    for axis in range(len(n)):
+        r1, r2 = spline.derivative(f.astype(np.float64), axis, n[axis], p[axis], h[axis], n_nb, second=True)
+        d1, d2 = (v.cpu().numpy() for v in g.derivative(0, axis, dev, second=True))
+        only = g.derivative(0, axis, dev).cpu().numpy()
+        assert np.abs(d1 - r1).max() < t1 * np.abs(r1).max(), axis
+        assert np.abs(only - r1).max() < t1 * np.abs(r1).max(), axis
+        assert np.abs(d2 - r2).max() < t2 * np.abs(r2).max(), axis
+        eye = np.eye(n[axis] + 1)
+        D = spline.derivative(eye, 0, n[axis], p[axis], h[axis], n_nb)
+        D = D[0] if isinstance(D, tuple) else D
+        rt = np.moveaxis(np.tensordot(D.T, f.astype(np.float64), axes=(1, axis)), 0, axis)
+        t = g.derivative_adjoint(0, axis, dev).cpu().numpy()
+        assert np.abs(t - rt).max() < t1 * np.abs(rt).max(), axis
+        over = dev.clone()
+        assert pkg.lib().loss_derivative(g.h, 0, axis, over.data_ptr(), over.data_ptr(), None, pkg.LOSS_MEM_DEVICE) == 0
+        g.sync()
+        assert np.abs(over.cpu().numpy() - r1).max() < t1 * np.abs(r1).max(), axis
+    g.close()
