@@ -1116,7 +1116,7 @@ loss_status_t loss_step(loss_handle_t h, int64_t n_steps) {
     LOSS_TRY(step_batched(h, n_steps));
   } else {
     for (int64_t k = 0; k < n_steps; ++k) {
-      for (Shot& s : h->shots) LOSS_TRY(step_shot(h, s));
+      for (Shot& s : h->shots) LOSS_TRY(step_shot(h, s, k > 0, k + 1 < n_steps));
     }
   }
   if (h->watch_every > 0) {
@@ -1351,9 +1351,10 @@ static loss_status_t run_derivative_t(loss_ctx* h, Shot& s, int k, const T* f, T
   LOSS_TRY(line_geom(h, s, k, sz, sy, &g, &logc, &threads, d2 ? 3 : 2, 0, h->lines_per_block[LOSS_KERNEL_DERIVATIVE],
                      h->chunk_log2[LOSS_KERNEL_DERIVATIVE], h->tile_threads[LOSS_KERNEL_DERIVATIVE]));
   // A launch shape asked for (loss_set_launch, loss_set_tile) is one of the line kernel's, and only that kernel reads
-  // a whole line before it writes one.
+  // a whole line before it writes one.  FP64 second derivatives along columns stay there too: the second recurrence
+  // costs more arithmetic than the line kernel's elimination shares (257^3: 837 us on the engine, 801 us there).
   const int kid = LOSS_KERNEL_DERIVATIVE;
-  if (d1 && !phi && !overlaps(s, f, d1) && !overlaps(s, f, d2) && h->lines_per_block[kid] <= 0 && h->tile_threads[kid] <= 0 && h->chunk_log2[kid] <= 0) {
+  if (d1 && !phi && !(d2 && s.esize == 8 && k != 2) && !overlaps(s, f, d1) && !overlaps(s, f, d2) && h->lines_per_block[kid] <= 0 && h->tile_threads[kid] <= 0 && h->chunk_log2[kid] <= 0) {
     ConvAxis ca;
     bool ok;
     LOSS_TRY(conv_axis(h, s, k, &ca, &ok));

@@ -34,6 +34,13 @@ struct ConvHost {
 
 // One independent grid (shot).  Internal axis slots: 0 = z, 1 = y, 2 = x; 2-D grids have a y extent of 1.
 // Device arrays use a padded layout: x pitch px (multiple of 32 elements), y stride sy = px, z stride sz.
+// Tables of the knot solver behind the others of a non-uniform axis: offset in nu_tab, segments of 8, and how many
+// segments back / ahead the recurrences reach.
+struct KnotHost {
+  size_t off = 0;
+  int S = 0, lf = 1, lb = 1;
+};
+
 struct Shot {
   loss_grid_desc_t d{};
   int dim = 0;
@@ -55,6 +62,7 @@ struct Shot {
   void* conv_tab[3] = {};
   ConvHost conv[3];
   void* nu_tab[3] = {};   // non-uniform axis slot (loss_set_coordinates): PMBC weights and elimination tables
+  KnotHost knots[3];      // of k_knots, per axis slot with nu_tab
   std::vector<double> coords[3];  // the knots loss_set_coordinates gave an axis slot (empty: equally spaced)
   bool has_model = false;
   double vmax = 0.0;
@@ -212,7 +220,9 @@ loss_status_t run_nu_derivative(loss_ctx* h, Shot& s, int k, const T* f, T* d1, 
 template <typename T>
 loss_status_t run_nu_derivative_adjoint(loss_ctx* h, Shot& s, int k, const T* g, T* out);
 loss_status_t set_coordinates(loss_ctx* h, Shot& s, int k, const double* x);
-loss_status_t nu_step(loss_ctx* h, Shot& s);  // one Strang step of a shot with non-uniform axes (2-D acoustic)
+// one Strang step of a shot with non-uniform axes (2-D acoustic); head: the previous call may have done the first half A
+// of this step, more: this one may do the next step's (steps of one loss_step)
+loss_status_t nu_step(loss_ctx* h, Shot& s, bool head, bool more);
 inline bool any_nonuniform(const Shot& s) { return s.nu_tab[0] || s.nu_tab[1] || s.nu_tab[2]; }
 // loss_adjoint.cu
 loss_status_t run_derivative_adjoint(loss_ctx* h, Shot& s, int k, const void* g, void* out, int mem);
@@ -248,7 +258,7 @@ std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c);
 ConvAxis conv_axis_at(const Shot& s, int k, const ConvHost& c, const void* tab);  // the tables at a device address
 ColMap col_map(int num_sms, const Shot& s, int k, int64_t py, int64_t pz);  // strided lines, slot 0 or 1
 RowMap row_map(int num_sms, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec);  // rows along x
-loss_status_t step_shot(loss_ctx* h, Shot& s);
+loss_status_t step_shot(loss_ctx* h, Shot& s, bool head = false, bool more = false);  // head, more: as nu_step
 loss_status_t unstagger(loss_ctx* h, Shot& s);
 loss_status_t stagger_shot(loss_ctx* h, Shot& s);
 bool batch_eligible(loss_ctx* h);

@@ -324,7 +324,8 @@ cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMa
     kern<<<grid, 128, smem, st>>>(g, cm, op);
     return cudaGetLastError();
   };
-  if (d2) return go(DerivColOp<T, true>{f, d1, d2, s1, s2}, k_col<T, DerivColOp<T, true>>, col_smem<T>(1, true));
+  if constexpr (sizeof(T) == 4)
+    if (d2) return go(DerivColOp<T, true>{f, d1, d2, s1, s2}, k_col<T, DerivColOp<T, true>>, col_smem<T>(1, true));
   return go(DerivColOp<T, false>{f, d1, d1, s1, s2}, k_col<T, DerivColOp<T, false>>, col_smem<T>(1));
 }
 

@@ -19,7 +19,8 @@
 // factors (the patch matrices differ, so there is no shared factor table).  Samples of the PMBC sums are
 // accumulated in FP64.
 //
-// One thread per (grid line, patch): it forms both junction sums, sweeps forward writing the eliminated right-hand
+// Lines that fit a block (KnotHost, knot_shape) are solved by k_knots (loss_knots.cuh).  Longer ones by k_nu_deriv, one
+// thread per (grid line, patch): it forms both junction sums, sweeps forward writing the eliminated right-hand
 // side into the output line, and sweeps back.  Consecutive threads take consecutive lines of the same patch, so
 // lines along y and z (consecutive x) load and store coalesced; lines along x are walked by each thread alone.
 #include <cuda_runtime.h>
@@ -28,9 +29,11 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "loss_host.h"
+#include "loss_knots.cuh"
 #include "loss_line.cuh"
 
 namespace lossk {
@@ -310,6 +313,39 @@ __global__ void __launch_bounds__(256) k_nu_adj2(NuArgs<T> a, T* __restrict__ ou
   *o = junction ? (T)acc : (T)((double)*o + acc);
 }
 
+// Tables of k_knots (KnotAxis: l, g, ra, rb, then the segments' products) and its reach in segments.
+static std::vector<double> knot_tables(const NuHost& t, int n, int p, bool f32, KnotHost* kh) {
+  const int S = n / 8 + 1, n8 = 8 * S, M = n / p;
+  std::vector<double> v((size_t)4 * n8 + 2 * S, 0.0);
+  for (int i = 0; i <= n; ++i) {
+    if (i % M == 0) continue;
+    // the first knot of a patch is eliminated with phi, which is not scaled
+    v[i] = i % M == 1 || M == 1 ? t.A[i] * t.IU[i] : t.L[i] * t.IU[i] / t.IU[i - 1];
+    v[n8 + i] = t.G[i] * t.IU[i];
+    v[2 * n8 + i] = t.ra[i] * t.IU[i];
+    v[3 * n8 + i] = t.rb[i] * t.IU[i];
+  }
+  double* seg = v.data() + 4 * n8;
+  for (int s = 0; s < S; ++s) {
+    seg[s] = seg[S + s] = 1.0;
+    for (int j = 0; j < 8; ++j) {
+      if (8 * s + j > n) continue;
+      seg[s] *= -v[8 * s + j];
+      seg[S + s] *= -v[n8 + 8 * s + j];
+    }
+  }
+  const double eps = f32 ? 0x1p-34 : 0x1p-64;
+  kh->S = S;
+  kh->lf = kh->lb = 1;
+  for (int s = 0; s < S; ++s) {
+    double w = 1.0;
+    for (int k = 1; s - k >= 0 && std::fabs(w) > eps; ++k) kh->lf = std::max(kh->lf, k), w *= seg[s - k];
+    w = 1.0;
+    for (int k = 1; s + k < S && std::fabs(w) > eps; ++k) kh->lb = std::max(kh->lb, k), w *= seg[S + s + k];
+  }
+  return v;
+}
+
 // Uploads the tables of axis slot k of shot s (built from the knots x, n[k] + 1 of them).
 static loss_status_t nu_upload(loss_ctx* h, Shot& s, int k, const std::vector<double>& x) {
   NuHost t;
@@ -318,7 +354,18 @@ static loss_status_t nu_upload(loss_ctx* h, Shot& s, int k, const std::vector<do
   const size_t np = (size_t)s.n[k] + 1;
   const size_t wbytes = t.W.size() * sizeof(double);
   const size_t tbytes = 7 * np * s.esize;
-  std::vector<unsigned char> blob(wbytes + tbytes);
+  KnotHost& kh = s.knots[k];
+  const std::vector<double> kt = knot_tables(t, (int)s.n[k], s.p[k], s.esize == 4, &kh);
+  kh.off = (wbytes + tbytes + 255) & ~(size_t)255;
+  std::vector<unsigned char> blob(kh.off + kt.size() * s.esize);
+  for (size_t i = 0; i < kt.size(); ++i) {
+    if (s.esize == 8) {
+      std::memcpy(blob.data() + kh.off + i * 8, &kt[i], 8);
+    } else {
+      const float v = (float)kt[i];
+      std::memcpy(blob.data() + kh.off + i * 4, &v, 4);
+    }
+  }
   std::memcpy(blob.data(), t.W.data(), wbytes);
   std::vector<double> hs(np, 0.0);
   for (size_t i = 0; i + 1 < np; ++i) hs[i] = x[i + 1] - x[i];
@@ -365,9 +412,42 @@ static void nu_args(const Shot& s, int k, int64_t py, int64_t pz, NuArgs<T>* pa)
   }
 }
 
+// Shape of k_knots for axis slot k: lines per block so that the GPU has a block per SM, 8 at most (a 32-byte sector of
+// neighbouring FP32 columns) unless short lines leave a block nearly empty.  False: a line does not fit a block, or
+// would leave a column block with single columns (4 of the 32 bytes of each sector); k_nu_deriv then.
+template <typename T>
+static bool knot_shape(const loss_ctx* h, const Shot& s, int k, int64_t py, int64_t pz, bool vec, KnotAxis<T>* g,
+                       KnotLines* kl, int* threads, size_t* smem) {
+  NuArgs<T> a{};
+  nu_args(s, k, py, pz, &a);
+  const KnotHost& kh = s.knots[k];
+  g->W = a.W;
+  g->tab = (const T*)((const unsigned char*)s.nu_tab[k] + kh.off);
+  g->seg = g->tab + 4 * 8 * kh.S;
+  g->n = a.n, g->p = a.p, g->M = a.M, g->n_nb = a.n_nb, g->S = kh.S, g->lf = kh.lf, g->lb = kh.lb;
+  auto bytes = [&](int c) { return ((size_t)(2 * kh.S + a.p + 1) << c) * sizeof(T); };
+  auto fits = [&](int c) { return (kh.S << c) <= kKnotThreads && bytes(c) <= 48 * 1024; };
+  const int cmin = k == 2 ? 0 : 1;
+  int c = 3;
+  while (c > cmin && !fits(c)) --c;
+  if (!fits(c)) return false;
+  while (c > (k == 2 ? 0 : 2) && (a.lines >> c) < h->num_sms) --c;
+  while (c < 5 && (kh.S << (c + 1)) <= 256 && fits(c + 1) && (a.lines >> (c + 1)) >= 2 * h->num_sms) ++c;
+  *kl = KnotLines{a.lines, a.stride, a.inner, a.inner_mul, a.outer_stride, c, vec ? 1 : 0};
+  *threads = std::max(64, ((kh.S << c) + 31) & ~31);
+  *smem = bytes(c);
+  return true;
+}
+template <typename T, bool ROW, class OP>
+static cudaError_t launch_knots(const KnotAxis<T>& g, const KnotLines& kl, int threads, size_t smem, const OP& op,
+                                double* phi, cudaStream_t st) {
+  k_knots<T, ROW, OP><<<(unsigned)((kl.lines + (1 << kl.logc) - 1) >> kl.logc), threads, smem, st>>>(g, kl, op, phi);
+  return cudaGetLastError();
+}
+
 template <typename T>
 static loss_status_t nu_launch(loss_ctx* h, Shot& s, int k, const T* f, T* d1, double* phi, int64_t py, int64_t pz,
-                               int kernel, T* d2 = nullptr) {
+                               int kernel, bool vec, T* d2 = nullptr) {
   NuArgs<T> a{};
   nu_args(s, k, py, pz, &a);
   a.f = f;
@@ -375,7 +455,16 @@ static loss_status_t nu_launch(loss_ctx* h, Shot& s, int k, const T* f, T* d1, d
   a.phi = phi;
   const int64_t threads = a.lines * a.p;
   LaunchScope ls(h, kernel);
-  k_nu_deriv<T><<<(unsigned)((threads + 127) / 128), 128, 0, h->stream>>>(a);
+  KnotAxis<T> g;
+  KnotLines kl;
+  int nt;
+  size_t smem;
+  if (d1 && knot_shape<T>(h, s, k, py, pz, vec, &g, &kl, &nt, &smem)) {
+    if (k == 2) launch_knots<T, true>(g, kl, nt, smem, KnotDeriv<T, true>{f, d1}, phi, h->stream);
+    else launch_knots<T, false>(g, kl, nt, smem, KnotDeriv<T, false>{f, d1}, phi, h->stream);
+  } else {
+    k_nu_deriv<T><<<(unsigned)((threads + 127) / 128), 128, 0, h->stream>>>(a);
+  }
   if (d2 && d1) {
     NU_TRY(cuda_check(h, cudaGetLastError(), "non-uniform derivative kernel"));
     k_nu_d2<T><<<(unsigned)((threads + 127) / 128), 128, 0, h->stream>>>(a, d2);
@@ -385,7 +474,7 @@ static loss_status_t nu_launch(loss_ctx* h, Shot& s, int k, const T* f, T* d1, d
 
 template <typename T>
 loss_status_t run_nu_derivative(loss_ctx* h, Shot& s, int k, const T* f, T* d1, double* phi, T* d2) {
-  return nu_launch<T>(h, s, k, f, d1, phi, s.len[2], s.len[2] * s.len[1], LOSS_KERNEL_DERIVATIVE, d2);
+  return nu_launch<T>(h, s, k, f, d1, phi, s.len[2], s.len[2] * s.len[1], LOSS_KERNEL_DERIVATIVE, false, d2);
 }
 
 // --- time step on grids with non-uniform axes (2-D acoustic) ------------------------------------------------
@@ -464,14 +553,7 @@ __global__ void __launch_bounds__(256) k_nu_sig_pml(T* __restrict__ u, T* __rest
   }
 }
 
-// Pressure source on knots: sigma += amp gz[oz] gx[ox] over the 25 x 25 knots around the source knot (zs, xs); gz,
-// gx: the Gaussian of width 2 h on the physical distance from the source knot (0 off the grid); amp: dt f_r(t)
-// times the amplitude over the cell-volume weighted sum of the profile.
-struct NuSrc {
-  int zs, xs;
-  double amp;
-  double gz[25], gx[25];
-};
+// Pressure source on knots (NuSrc).
 template <typename T, bool K>
 __global__ void __launch_bounds__(640) k_nu_source(T* __restrict__ u, T* __restrict__ c, NuSrc q, int64_t px) {
   const int i = threadIdx.x;
@@ -494,6 +576,7 @@ __global__ void __launch_bounds__(640) k_nu_source(T* __restrict__ u, T* __restr
 // The source of step n on knots (slots 0 = z, 2 = x), as above.
 static NuSrc nu_source(const Shot& s, int64_t n) {
   NuSrc q{};
+  q.on = 1;
   q.zs = (int)s.src_idx[0];
   q.xs = (int)s.src_idx[2];
   double sum[2] = {0.0, 0.0};
@@ -553,8 +636,83 @@ static PmlAxis<T> nu_pml_axis(const Shot& s, int k, double tau) {
   return PmlAxis<T>{(const T*)s.pml_tab[k][tau == s.d.dt ? 0 : 1], s.pml_width, (int)s.n[k], nullptr};
 }
 
+// The step with every update fused into the kernel that forms its derivative: V1 (rows), V3 (columns), the row
+// derivative of V1, then sigma and the source (columns).  The last half A of a step and the first of the next see the
+// same sigma: inside a call they are one pass that updates twice (head: the previous step did this step's first; more:
+// this step does the next one's), unless velocity receivers are read in between.
 template <typename T, bool K>
-static loss_status_t nu_step_t(loss_ctx* h, Shot& s) {
+static loss_status_t nu_fused_step(loss_ctx* h, Shot& s, const KnotAxis<T> (&g)[2], const KnotLines (&kl)[2],
+                                   const int (&nt)[2], const size_t (&smem)[2], bool head, bool more) {
+  const double dt = s.d.dt;
+  T* t0 = (T*)s.tmp[0];
+  auto comp = [&](int f) { return K ? (T*)s.comp[f] : (T*)s.field[f]; };
+  auto half_A = [&](int times) -> loss_status_t {
+    auto op = [&](auto row, int field, int k) {
+      KnotVel<T, decltype(row)::value, K> o{};
+      o.sigma = (const T*)s.field[LOSS_FIELD_SIGMA];
+      o.u = (T*)s.field[field];
+      o.c = comp(field);
+      o.bc = s.b_const ? 1 : 0;
+      o.b = s.b_const ? (const T*)o.u : (const T*)s.model[1];
+      o.b0 = (T)s.b0;
+      o.tau = (T)(0.5 * dt);
+      o.pml = s.pml_on ? 1 : 0;
+      o.times = times;
+      o.pa = PmlAxis<T>{o.sigma, 0, 0, nullptr}, o.mem = o.u;
+      if (s.pml_on) o.pa = nu_pml_axis<T>(s, k, 0.5 * dt), o.mem = (T*)s.psi[k];
+      return o;
+    };
+    {
+      LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
+      NU_TRY(cuda_check(h, launch_knots<T, true>(g[1], kl[1], nt[1], smem[1], op(std::true_type{}, LOSS_FIELD_V1, 2),
+                                                 nullptr, h->stream), "non-uniform velocity kernel"));
+    }
+    LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_Z);
+    return cuda_check(h, launch_knots<T, false>(g[0], kl[0], nt[0], smem[0], op(std::false_type{}, LOSS_FIELD_V3, 0),
+                                                nullptr, h->stream), "non-uniform velocity kernel");
+  };
+  if (!head) NU_TRY(half_A(1));
+  {
+    LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
+    NU_TRY(cuda_check(h, launch_knots<T, true>(g[1], kl[1], nt[1], smem[1],
+                                               KnotDeriv<T, true>{(const T*)s.field[LOSS_FIELD_V1], t0}, nullptr,
+                                               h->stream), "non-uniform derivative kernel"));
+  }
+  KnotSig<T, K> o{};
+  o.v3 = (const T*)s.field[LOSS_FIELD_V3];
+  o.u = (T*)s.field[LOSS_FIELD_SIGMA];
+  o.c = comp(LOSS_FIELD_SIGMA);
+  o.gx = t0;
+  o.kappa = (const T*)s.model[0];
+  o.dt = (T)dt;
+  o.pml = s.pml_on ? 1 : 0;
+  o.px = o.pz = PmlAxis<T>{o.v3, 0, 0, nullptr}, o.memx = o.memz = o.u;
+  if (s.pml_on) {
+    o.px = nu_pml_axis<T>(s, 2, dt), o.pz = nu_pml_axis<T>(s, 0, dt);
+    o.memx = (T*)s.phi[2], o.memz = (T*)s.phi[0];
+  }
+  if (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) o.q = nu_source(s, s.step);
+  {
+    LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_Z);
+    NU_TRY(cuda_check(h, launch_knots<T, false>(g[0], kl[0], nt[0], smem[0], o, nullptr, h->stream),
+                      "non-uniform stress kernel"));
+  }
+  return half_A(more ? 2 : 1);
+}
+
+template <typename T, bool K>
+static loss_status_t nu_step_t(loss_ctx* h, Shot& s, bool head, bool more) {
+  KnotAxis<T> ka[2];
+  KnotLines kl[2];
+  int nt[2];
+  size_t smem[2];
+  if (knot_shape<T>(h, s, 0, s.sy, s.sz, false, &ka[0], &kl[0], &nt[0], &smem[0]) &&
+      knot_shape<T>(h, s, 2, s.sy, s.sz, true, &ka[1], &kl[1], &nt[1], &smem[1])) {
+    bool merge = true;
+    for (int f = 0; f < LOSS_NUM_FIELDS; ++f)
+      if (is_velocity(f) && s.n_rcv && s.rcv_offsets[f + 1] > s.rcv_offsets[f]) merge = false;
+    return nu_fused_step<T, K>(h, s, ka, kl, nt, smem, head && merge, more && merge);
+  }
   const double dt = s.d.dt;
   T* t0 = (T*)s.tmp[0];
   T* t1 = (T*)s.tmp[1];
@@ -571,9 +729,9 @@ static loss_status_t nu_step_t(loss_ctx* h, Shot& s) {
   };
   auto half_A = [&]() -> loss_status_t {
     NU_TRY(nu_launch<T>(h, s, 2, (const T*)s.field[LOSS_FIELD_SIGMA], t0, nullptr, s.sy, s.sz,
-                        LOSS_KERNEL_ACOUSTIC_X));
+                        LOSS_KERNEL_ACOUSTIC_X, true));
     NU_TRY(nu_launch<T>(h, s, 0, (const T*)s.field[LOSS_FIELD_SIGMA], t1, nullptr, s.sy, s.sz,
-                        LOSS_KERNEL_ACOUSTIC_Z));
+                        LOSS_KERNEL_ACOUSTIC_Z, false));
     if (s.pml_on) {
       NU_TRY(vel_pml(LOSS_FIELD_V1, t0, 2));
       return vel_pml(LOSS_FIELD_V3, t1, 0);
@@ -582,8 +740,10 @@ static loss_status_t nu_step_t(loss_ctx* h, Shot& s) {
     return nu_update<T, K>(h, s, LOSS_FIELD_V3, t1, nullptr, b, s.b0, -0.5 * dt);
   };
   NU_TRY(half_A());
-  NU_TRY(nu_launch<T>(h, s, 2, (const T*)s.field[LOSS_FIELD_V1], t0, nullptr, s.sy, s.sz, LOSS_KERNEL_ACOUSTIC_X));
-  NU_TRY(nu_launch<T>(h, s, 0, (const T*)s.field[LOSS_FIELD_V3], t1, nullptr, s.sy, s.sz, LOSS_KERNEL_ACOUSTIC_Z));
+  NU_TRY(nu_launch<T>(h, s, 2, (const T*)s.field[LOSS_FIELD_V1], t0, nullptr, s.sy, s.sz, LOSS_KERNEL_ACOUSTIC_X,
+                      true));
+  NU_TRY(nu_launch<T>(h, s, 0, (const T*)s.field[LOSS_FIELD_V3], t1, nullptr, s.sy, s.sz, LOSS_KERNEL_ACOUSTIC_Z,
+                      false));
   if (s.pml_on) {
     LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X2);
     k_nu_sig_pml<T, K><<<grid, 256, 0, h->stream>>>(
@@ -602,15 +762,15 @@ static loss_status_t nu_step_t(loss_ctx* h, Shot& s) {
   return half_A();
 }
 
-loss_status_t nu_step(loss_ctx* h, Shot& s) {
+loss_status_t nu_step(loss_ctx* h, Shot& s, bool head, bool more) {
   if (s.d.physics != LOSS_ACOUSTIC || s.dim != 2)
     return fail_msg(h, LOSS_E_UNSUPPORTED, "time steps on non-uniform grids are built for 2-D acoustic grids");
   if (s.src_on && (s.src_kinds & ~(uint32_t)LOSS_SRC_PRESSURE))
     return fail_msg(h, LOSS_E_UNSUPPORTED, "non-uniform grids: pressure sources only");
   NU_TRY(nu_ensure_axes(h, s));
-  if (s.esize == 8) return nu_step_t<double, false>(h, s);
-  if (s.kahan) return nu_step_t<float, true>(h, s);
-  return nu_step_t<float, false>(h, s);
+  if (s.esize == 8) return nu_step_t<double, false>(h, s, head, more);
+  if (s.kahan) return nu_step_t<float, true>(h, s, head, more);
+  return nu_step_t<float, false>(h, s, head, more);
 }
 
 template <typename T>

@@ -1380,9 +1380,9 @@ loss_status_t step_batched(loss_ctx* h, int64_t n) {
   return step_batched_t<float, false>(h, n);
 }
 
-loss_status_t step_shot(loss_ctx* h, Shot& s) {
+loss_status_t step_shot(loss_ctx* h, Shot& s, bool head, bool more) {
   if (any_nonuniform(s)) {
-    LOSS_TRY(nu_step(h, s));
+    LOSS_TRY(nu_step(h, s, head, more));
     // receivers at the integer time level (the non-uniform step keeps no staggered velocities)
     if (s.esize == 8) {
       LOSS_TRY(gather_fields<double>(h, s, true, 0));
