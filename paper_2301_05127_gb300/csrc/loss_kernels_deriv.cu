@@ -8,7 +8,7 @@
 //
 // Memory bound: one read and one write of the array per output (257^3 FP32: 136 MB).  The line kernel they replace
 // (k_deriv, k_adj: whole lines staged in shared memory between barriers, a block's loads, elimination and stores in
-// turn) took 1.75 ms for first and second derivatives and transposes along the axes of a 257^3 FP32 array that these do in 0.64 ms (with the host between); 129^2 FP64 operators,
+// turn) took 1.75 ms for first and second derivatives and transposes along the axes of a 257^3 FP32 array that these do in 0.60 ms (with the host between); 129^2 FP64 operators,
 // which launches bound, 95 us -> 88 us.  The line kernel stays for PMBC values, short patches, arrays beyond 32-bit
 // offsets, arrays written over their input, and launch shapes that the caller asked for.
 #include <cuda_runtime.h>
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
   const int gl = lane & (gw - 1), k = lane / gw;
   const int items = rm.groups * rm.nwin;
   for (int item = blockIdx.x * 4 + warp; item < items; item += gridDim.x * 4) {
-    const int grp = item / rm.nwin, win = item - grp * rm.nwin;
+    const int grp = rm.nwin == 1 ? item : item / rm.nwin, win = item - grp * rm.nwin;
     const int c0 = win * (32 - 2 * Conv<T>::W);
     const int c1 = min(rm.nch, c0 + gw);
     const int o0 = win == 0 ? 0 : c0 + Conv<T>::W;
@@ -114,15 +114,28 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
     int j0 = 0, nj = 0;
     if (g.ntaps) {
       const int lo = 8 * o0, hi = o1 == rm.nch ? g.n : 8 * o1 - 1;
-      j0 = lo <= g.R ? 0 : (lo - g.R + g.M - 1) / g.M;
-      nj = min(g.p, (hi + g.R) / g.M) - j0 + 1;
+      j0 = lo <= g.R ? 0 : small_div(lo - g.R + g.M - 1, g.M);
+      nj = min(g.p, small_div(hi + g.R, g.M)) - j0 + 1;
     }
-    __syncwarp();
-    for (int i = lane; i < nrow * nj; i += 32) {
-      const int j = i % nj, kk = i / nj;
-      dsm[i] = trans_junction<T>(g, j0 + j, in + rbase(grp * rpw + kk), 0u, (uint32_t)sizeof(T), rs);
+    if (nj > 0) {  // G lanes per (row, junction)
+      __syncwarp();
+      const int tasks = nrow * nj, lg = tasks > 16 ? 0 : (tasks > 8 ? 1 : (tasks > 4 ? 2 : 3));
+      for (int i0 = 0; i0 < tasks; i0 += 32 >> lg) {
+        const int i = i0 + (lane >> lg), ii = min(i, tasks - 1);
+        const int kk = small_div(ii, nj), q0 = (j0 + ii - kk * nj) * g.M;
+        const T* f = in + (rpw == 1 ? rb : rbase(grp * rpw + kk));
+        T D = T(0);
+        for (int d = (lane & ((1 << lg) - 1)) - g.Q; d <= g.Q; d += 1 << lg) {
+          const int x = q0 + d;
+          const T v = f[min(max(x, 0), g.n)];
+          D += (x >= 0 && x <= g.n ? v : T(0)) * rs[64 + d];
+        }
+        __syncwarp();
+        for (int o = 1; o < 1 << lg; o <<= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
+        if (i < tasks) dsm[i] = D;
+      }
+      __syncwarp();
     }
-    __syncwarp();
     if (end && len < 8)
 #pragma unroll
       for (int j = 0; j < 8; ++j)

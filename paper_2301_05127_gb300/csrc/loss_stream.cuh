@@ -69,6 +69,37 @@ __device__ __forceinline__ T& at_off(T* p, uint32_t o) {
   return *reinterpret_cast<T*>(reinterpret_cast<C*>(p) + o);
 }
 
+// Sum of weight x sample over the taps of a junction, to the precision of T's FP64 sum rounded to T: in FP64, or for FP32
+// samples in two floats (error-free products and additions, about 46 bits).  The GPU's FP64 pipe takes 16 cycles of an SM
+// per warp instruction, however few lanes are active; eleven FP32 instructions take about three.  With that, and several
+// lanes of a row warp on one junction (one lane each had 5 of 32 at work on a row of four patches): derivative of
+// 257^3 FP32 along x 82 us -> 60 us, FP64 acoustic rows of 1025^2 102 us -> 94 us, elastic x part of 257^3 457 us -> 432 us.
+template <typename T>
+struct TapSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(const ConvTap& t, double v) { s = fma(t.w, v, s); }
+  __device__ __forceinline__ void merge(int o) { s += __shfl_xor_sync(0xffffffffu, s, o); }
+  __device__ __forceinline__ double get() const { return s; }
+};
+template <>
+struct TapSum<float> {
+  float s = 0.0f, c = 0.0f;
+  __device__ __forceinline__ void plus(float p, float e) {  // s + c += p + e
+    const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
+    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)), e));
+    s = t;
+  }
+  __device__ __forceinline__ void add(const ConvTap& t, float v) {
+    const float p = __fmul_rn(t.hi, v);
+    plus(p, __fmaf_rn(t.lo, v, __fmaf_rn(t.hi, v, -p)));
+  }
+  __device__ __forceinline__ void merge(int o) {
+    const float p = __shfl_xor_sync(0xffffffffu, s, o), e = __shfl_xor_sync(0xffffffffu, c, o);
+    plus(p, e);
+  }
+  __device__ __forceinline__ float get() const { return __fadd_rn(s, c); }
+};
+
 // Junction corrections D[f] of junction j of NF lines with their samples at byte offset o + (jM + m) * sb of src[f]; taps:
 // the axis's taps (a shared-memory copy or g.taps); four taps' samples in flight at a time.
 template <typename T, int NF>
@@ -76,17 +107,14 @@ __device__ __forceinline__ void conv_junction(const ConvAxis& g, const ConvTap* 
                                               uint32_t o, uint32_t sb, T (&D)[NF]) {
   int t = __ldg(g.js + j);
   const int t1 = __ldg(g.js + j + 1);
-  double s[NF];
-#pragma unroll
-  for (int f = 0; f < NF; ++f) s[f] = 0.0;
+  TapSum<T> s[NF];
   for (; t < t1; t += 4) {
-    double w[4];
+    ConvTap w[4];
     T v[4][NF];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const ConvTap tap = taps[min(t + k, t1 - 1)];
-      w[k] = t + k < t1 ? tap.w : 0.0;
-      const uint32_t ot = o + (uint32_t)(j * g.M + tap.m) * sb;
+      w[k] = taps[min(t + k, t1 - 1)];
+      const uint32_t ot = o + (uint32_t)(j * g.M + w[k].m) * sb;
 #pragma unroll
       for (int f = 0; f < NF; ++f) v[k][f] = at_off(src[f], ot);
     }
@@ -94,11 +122,30 @@ __device__ __forceinline__ void conv_junction(const ConvAxis& g, const ConvTap* 
     for (int k = 0; k < 4; ++k)
       if (t + k < t1)
 #pragma unroll
-        for (int f = 0; f < NF; ++f) s[f] = fma(w[k], to_f64(v[k][f]), s[f]);
+        for (int f = 0; f < NF; ++f) s[f].add(w[k], v[k][f]);
   }
 #pragma unroll
-  for (int f = 0; f < NF; ++f) D[f] = (T)s[f];
+  for (int f = 0; f < NF; ++f) D[f] = (T)s[f].get();
 }
+// The same for one line at f by G lanes (a power of two; sub: the lane's number among them); called by the whole warp.
+template <typename T>
+__device__ __forceinline__ T conv_junction_part(const ConvAxis& g, const ConvTap* taps, int j, const T* f, int sub,
+                                                int G) {
+  const int t1 = __ldg(g.js + j + 1);
+  const T* fj = f + j * g.M;
+  TapSum<T> s;
+  for (int t = __ldg(g.js + j) + sub; t < t1; t += 2 * G) {
+    const ConvTap w0 = taps[t], w1 = taps[min(t + G, t1 - 1)];
+    const T v0 = fj[w0.m], v1 = fj[w1.m];
+    s.add(w0, v0);
+    if (t + G < t1) s.add(w1, v1);
+  }
+  __syncwarp();
+  for (int o = 1; o < G; o <<= 1) s.merge(o);
+  return (T)s.get();
+}
+// a / b for 0 <= a < 2^21, b > 0 (a quotient is 1 / (2 b) or more from the next integer, its error below 2^-22 of it)
+__device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
 
 // Block-wide copy of a launch descriptor into shared memory (no barrier).
 template <class J>
@@ -629,7 +676,7 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
   const int gl = lane & (gw - 1), k = lane / gw;
   const int items = rm.groups * rm.nwin;
   for (int item = bid * 4 + warp; item < items; item += nblk * 4) {
-    const int grp = item / rm.nwin, win = item - grp * rm.nwin;
+    const int grp = rm.nwin == 1 ? item : item / rm.nwin, win = item - grp * rm.nwin;
     const int c0 = win * (32 - 2 * Conv<T>::W);              // first chunk of the window
     const int c1 = min(rm.nch, c0 + gw);                     // past its last
     const int o0 = win == 0 ? 0 : c0 + Conv<T>::W;           // own chunks
@@ -657,22 +704,26 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
     int j0 = 0, nj = 0;
     if (g.ntaps) {
       const int lo = 8 * o0, hi = o1 == rm.nch ? g.n : 8 * o1 - 1;
-      j0 = lo <= g.Q ? 0 : (lo - g.Q + g.M - 1) / g.M;
-      nj = min(g.p, (hi + g.Q) / g.M) - j0 + 1;
+      j0 = lo <= g.Q ? 0 : small_div(lo - g.Q + g.M - 1, g.M);
+      nj = min(g.p, small_div(hi + g.Q, g.M)) - j0 + 1;
     }
     // e of the NF fields whose samples are in e and at s0 (fields 1 ..: at op.src)
     auto derive = [&](const T* s0) {
-      if (nj > 0) {  // one lane per (field, row, junction)
+      if (nj > 0) {  // G lanes per (field, row, junction)
         __syncwarp();
-        for (int i = lane; i < NF * nrow * nj; i += 32) {
-          const int j = i % nj, fk = i / nj, f = fk / nrow;
-          int64_t off = rbase(grp * rpw + fk - f * nrow);
+        const int tasks = NF * nrow * nj;
+        const int lg = tasks > 16 ? 0 : (tasks > 8 ? 1 : (tasks > 4 ? 2 : 3));
+        for (int i0 = 0; i0 < tasks; i0 += 32 >> lg) {
+          const int i = i0 + (lane >> lg), ii = min(i, tasks - 1);
+          const int fk = small_div(ii, nj), j = ii - fk * nj;
+          int f = 0;
+#pragma unroll
+          for (int s = 1; s < NF; ++s) f += fk >= s * nrow;
+          int64_t off = rpw == 1 ? rb : rbase(grp * rpw + fk - f * nrow);
 #pragma unroll
           for (int s = 1; s < NF; ++s) off += f == s ? op.src(s) - s0 : (int64_t)0;
-          const T* fs[1] = {s0 + off};
-          T D[1];
-          conv_junction<T, 1>(g, taps, j0 + j, fs, 0u, (uint32_t)sizeof(T), D);
-          dsm[i] = D[0];
+          const T D = conv_junction_part<T>(g, taps, j0 + j, s0 + off, lane & ((1 << lg) - 1), 1 << lg);
+          if (i < tasks) dsm[i] = D;
         }
         __syncwarp();
       }
@@ -683,7 +734,7 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
           for (int j = 0; j < 8; ++j)
             if (j >= len) e[f][j] = T(0);
       // the junctions before (or at the start of) the chunk and after it; at most one of each is within Q
-      const int ja = 8 * c / g.M, o0j = 8 * c - ja * g.M, o1j = o0j - g.M;  // the chunk's offsets from ja and ja + 1
+      const int ja = small_div(8 * c, g.M), o0j = 8 * c - ja * g.M, o1j = o0j - g.M;  // the chunk's offsets from ja and ja + 1
       const int ia = ja - j0, ib = ia + 1;
       const bool hasa = len > 0 && ia >= 0 && ia < nj && o0j <= g.Q;
       const bool hasb = len > 0 && ib >= 0 && ib < nj && -o1j - 8 <= g.Q;
@@ -718,7 +769,7 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
     if constexpr (OP::SECOND) {
       row_solve<T, kSecond>(q2, c, len, end, gl, gw, rlen, T(0), T(0));
       if (nj > 0 && len > 0) {
-        const int ja = 8 * c / g.M;
+        const int ja = small_div(8 * c, g.M);
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
           const int jj = ja + s - j0, o = 8 * c - (ja + s) * g.M;
