@@ -345,6 +345,7 @@ loss_status_t loss_set_coordinates(loss_handle_t handle, int32_t shot, int32_t a
  * limit) for its own copies in flight and stops, so the CUDA context stays usable, and the next loss_sync returns
  * LOSS_E_TIMEOUT and poisons the handle.  polls < 0 restores the default (2^24 polls, far beyond any copy's
  * latency); polls = 0 makes every such wait give up without polling, which is how the failure path is tested.
+ * Kernels without waits are taken where they are faster; a handle whose limit is not the default keeps those that wait.
  * This is a library control with no counterpart in the paper.  Takes effect from the next loss_step (a captured
  * graph is recaptured).  Returns LOSS_E_ARG for a NULL handle. */
 loss_status_t loss_set_wait_limit(loss_handle_t handle, int64_t polls);

@@ -772,7 +772,7 @@ loss_status_t loss_sync(loss_handle_t h) {
 
 loss_status_t loss_set_wait_limit(loss_handle_t h, int64_t polls) {
   LOSS_TRY(guard(h));
-  h->wait_polls = polls < 0 ? (1u << 24) : (unsigned)std::min<int64_t>(polls, 0xffffffffLL);
+  h->wait_polls = polls < 0 ? kDefaultWaitPolls : (unsigned)std::min<int64_t>(polls, 0xffffffffLL);
   return LOSS_OK;
 }
 

@@ -144,12 +144,15 @@ struct BatchState {
   bool stream = false;
   void* astab = nullptr;
   AcBatchKind ask[8];
+  bool rows = false;  // with conv: the x part runs on the row engine
   int64_t astab_version = 0;
   XpSmem xl{};
   int xpthreads = 0, xpgrid = 0, tztiles = 0;
   int tzthreads[2] = {0, 0}, tzlogc[2] = {4, 4}, tzgrid[2] = {0, 0};
   size_t tzsmem[2] = {0, 0};
 };
+
+constexpr unsigned kDefaultWaitPolls = 1u << 24;
 
 }  // namespace lossk
 
@@ -173,7 +176,7 @@ struct loss_ctx {
   int batched = 1;       // several 2-D acoustic shots: one persistent launch per kernel over all of them
   int tiled = 1;         // LOSS_KERNELS_* family of the FP32 2-D acoustic shots stepped one at a time
   int* dflag = nullptr;  // device error flag of kernels with bounded waits (read by loss_sync)
-  unsigned wait_polls = 1u << 24;  // poll limit of those waits (loss_set_wait_limit)
+  unsigned wait_polls = lossk::kDefaultWaitPolls;  // poll limit of those waits (loss_set_wait_limit)
   // non-finite watchdog (loss_set_watchdog): every watch_every steps (0 = off) a check of every field sets nflag to
   // 1 + shot * LOSS_NUM_FIELDS + field of the first non-finite field found (read and cleared by loss_sync)
   int64_t watch_every = 0, watch_count = 0;
@@ -334,8 +337,11 @@ loss_status_t deriv_stream(loss_ctx* h, const Shot& s, int k, const ConvAxis& g,
 // loss_kernels_acstream.cu: 2-D acoustic step on the barrier-free engines
 template <typename T, bool KAHAN>
 cudaError_t launch_ac_rows(const AcXArgs<T>& a, const ConvAxis& g, const RowMap& rm, cudaStream_t st);
-cudaError_t launch_ac_cols(const AcZArgs<double>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st);
-void ac_batch_tables(const std::vector<AcStreamShot>& shots, std::vector<unsigned char>& bytes, AcBatchKind (&k)[8]);
+template <typename T, bool K>
+cudaError_t launch_ac_cols(const AcZArgs<T>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st);
+template <typename T, bool K>
+void ac_batch_tables(const std::vector<AcStreamShot<T>>& shots, std::vector<unsigned char>& bytes, AcBatchKind (&k)[8]);
+template <typename T, bool K>
 cudaError_t launch_ac_batch(const void* base, const AcBatchKind& k, int kind, cudaStream_t st);
 // Blocks of a k_row launch (4 warps each, kblocks resident per SM).
 inline int row_blocks(const RowMap& rm, int kblocks) {

@@ -187,7 +187,7 @@ struct AcRowOp {
   }
 };
 
-template <typename T, int MODE, bool REC>
+template <typename T, bool KAHAN, int MODE, bool REC>
 struct AcColOp {
   static constexpr int NF = 1;
   static constexpr bool SECOND = false;
@@ -196,14 +196,25 @@ struct AcColOp {
   AcZArgs<T> a;
   int b_on, pad;
   struct Regs {
-    T v, b, m;
+    T v, b, m, c;
   };
   __device__ __forceinline__ const T* src(int) const { return MODE == 1 ? a.sigma : a.v3; }
   __device__ __forceinline__ void load(Regs& r, int pos, uint32_t o) const {
     if constexpr (MODE == 1) {
       r.v = at_off(a.v3, o);
+      if constexpr (KAHAN) r.c = at_off(a.cv3, o);
       if (b_on) r.b = at_off(a.b, o);
       if (a.pml && a.zA.in(pos)) r.m = at_off(a.psiz, o);
+    }
+  }
+  __device__ __forceinline__ void add(const Regs& r, uint32_t o, T delta) const {
+    if constexpr (KAHAN) {
+      float v = r.v, c = r.c;
+      kahan_add(v, c, delta);
+      at_off(a.v3, o) = v;
+      at_off(a.cv3, o) = c;
+    } else {
+      at_off(a.v3, o) = r.v + delta;
     }
   }
   __device__ __forceinline__ void apply(Regs& r, const T (&e)[1], int pos, uint32_t o, int, int) const {
@@ -223,11 +234,13 @@ struct AcColOp {
         at_off(a.dlt, o) = bb * (ih - T(0.5) * inc);
       }
       at_off(a.psiz, o) = m1;
-      at_off(a.v3, o) = r.v + bb * inc;
+      add(r, o, b_on || sizeof(T) == 8 ? bb * inc : mulc(inc, a.b0, a.b0_lo));
+    } else if constexpr (sizeof(T) == 8) {
+      at_off(a.v3, o) = b_on ? fma(r.b * -(a.s3h * a.acoef), e[0], r.v) : fma(e[0], a.sc, r.v);
     } else if (b_on) {
-      at_off(a.v3, o) = fma(r.b * -(a.s3h * a.acoef), e[0], r.v);
+      add(r, o, r.b * mulc(e[0], -(a.s3h * a.acoef), -(a.s3h * a.acoef_lo + a.s3h_lo * a.acoef)));
     } else {
-      at_off(a.v3, o) = fma(e[0], a.sc, r.v);
+      add(r, o, mulc(e[0], a.sc, a.sc_lo));
     }
   }
 };
@@ -290,36 +303,45 @@ cudaError_t launch_ac_rows(const AcXArgs<T>& a, const ConvAxis& g, const RowMap&
   if (rec) return go_row<T>(g, rm, AcRowOp<T, KAHAN, true, false, true, false>{f, b_on, 0}, st);
   return go_row<T>(g, rm, AcRowOp<T, KAHAN, false, false, true, false>{f, b_on, 0}, st);
 }
-// mode 1: Z1, mode 2: Z2 (FP64).
-cudaError_t launch_ac_cols(const AcZArgs<double>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st) {
+// mode 1: Z1, mode 2: Z2.
+template <typename T, bool K>
+cudaError_t launch_ac_cols(const AcZArgs<T>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st) {
   const int b_on = a.b ? 1 : 0;
-  AcZArgs<double> f = a;
+  AcZArgs<T> f = a;
   fill_unused(f);
-  if (mode == 2) return go_col<double>(g, cm, AcColOp<double, 2, false>{f, b_on, 0}, st);
-  if (a.pml && a.dlt) return go_col<double>(g, cm, AcColOp<double, 1, true>{f, b_on, 0}, st);
-  return go_col<double>(g, cm, AcColOp<double, 1, false>{f, b_on, 0}, st);
+  if (mode == 2) return go_col<T>(g, cm, AcColOp<T, K, 2, false>{f, b_on, 0}, st);
+  if (a.pml && a.dlt) return go_col<T>(g, cm, AcColOp<T, K, 1, true>{f, b_on, 0}, st);
+  return go_col<T>(g, cm, AcColOp<T, K, 1, false>{f, b_on, 0}, st);
 }
+template cudaError_t launch_ac_cols<float, false>(const AcZArgs<float>&, const ConvAxis&, const ColMap&, int, cudaStream_t);
+template cudaError_t launch_ac_cols<float, true>(const AcZArgs<float>&, const ConvAxis&, const ColMap&, int, cudaStream_t);
+template cudaError_t launch_ac_cols<double, false>(const AcZArgs<double>&, const ConvAxis&, const ColMap&, int,
+                                                   cudaStream_t);
 template cudaError_t launch_ac_rows<float, false>(const AcXArgs<float>&, const ConvAxis&, const RowMap&, cudaStream_t);
 template cudaError_t launch_ac_rows<float, true>(const AcXArgs<float>&, const ConvAxis&, const RowMap&, cudaStream_t);
 template cudaError_t launch_ac_rows<double, false>(const AcXArgs<double>&, const ConvAxis&, const RowMap&,
                                                    cudaStream_t);
 
 // ---------------------------------------------------------------------------------------------------------------
-// Batched FP64 step.  Every shot keeps the kernels and the block-to-work mapping of its own launches (so the results are
+// Batched step.  Every shot keeps the kernels and the block-to-work mapping of its own launches (so the results are
 // theirs bit for bit); one launch runs the blocks of all shots of one kind.  Kinds: 0, 1 rows B + A of one-window rows
-// (without and with receiver corrections), 2 rows B, 3, 4 rows A, 5, 6 cols Z1, 7 cols Z2.
-template <class F>
+// (without and with receiver corrections), 2 rows B, 3, 4 rows A, 5, 6 cols Z1, 7 cols Z2 (FP64).  FP32: kinds 2
+// to 4, rows of at least 513 points; the columns are the batched z tiles'.
+template <typename D, bool K, class F>
 static void with_kind(int kind, F&& f) {
-  using D = double;
   switch (kind) {
-    case 0: return f(RowJob<D, AcRowOp<D, false, false, true, true, true>>{});
-    case 1: return f(RowJob<D, AcRowOp<D, false, true, true, true, true>>{});
-    case 2: return f(RowJob<D, AcRowOp<D, false, false, true, false, true>>{});
-    case 3: return f(RowJob<D, AcRowOp<D, false, false, false, true, true>>{});
-    case 4: return f(RowJob<D, AcRowOp<D, false, true, false, true, true>>{});
-    case 5: return f(ColJob<D, AcColOp<D, 1, false>>{});
-    case 6: return f(ColJob<D, AcColOp<D, 1, true>>{});
-    default: return f(ColJob<D, AcColOp<D, 2, false>>{});
+    case 2: return f(RowJob<D, AcRowOp<D, K, false, true, false, true>>{});
+    case 3: return f(RowJob<D, AcRowOp<D, K, false, false, true, true>>{});
+    case 4: return f(RowJob<D, AcRowOp<D, K, true, false, true, true>>{});
+  }
+  if constexpr (sizeof(D) == 8) {
+    switch (kind) {
+      case 0: return f(RowJob<D, AcRowOp<D, K, false, true, true, true>>{});
+      case 1: return f(RowJob<D, AcRowOp<D, K, true, true, true, true>>{});
+      case 5: return f(ColJob<D, AcColOp<D, false, 1, false>>{});
+      case 6: return f(ColJob<D, AcColOp<D, false, 1, true>>{});
+      default: return f(ColJob<D, AcColOp<D, false, 2, false>>{});
+    }
   }
 }
 template <class J>
@@ -327,13 +349,13 @@ struct JobTraits;
 template <typename T, class OP>
 struct JobTraits<RowJob<T, OP>> {
   static constexpr int kInts = 4;  // ints per entry of the block table
-  static RowJob<T, OP> make(const AcStreamShot& s) {
+  static RowJob<T, OP> make(const AcStreamShot<T>& s) {
     RowJob<T, OP> j{s.gx, s.rm, {s.x, s.x.b ? 1 : 0, 0}};
     fill_unused(j.op.a);
     return j;
   }
-  static int blocks(const AcStreamShot& s) { return row_blocks(s.rm, OP::kBlocks); }
-  static size_t smem(const AcStreamShot& s) { return (size_t)4 * s.rm.wbytes; }
+  static int blocks(const AcStreamShot<T>& s) { return row_blocks(s.rm, OP::kBlocks); }
+  static size_t smem(const AcStreamShot<T>& s) { return (size_t)4 * s.rm.wbytes; }
   static cudaError_t launch(const unsigned char* base, const AcBatchKind& k, cudaStream_t st) {
     auto kern = k_row_batch<T, OP>;
     if (k.smem > 32 * 1024) {
@@ -347,13 +369,13 @@ struct JobTraits<RowJob<T, OP>> {
 template <typename T, class OP>
 struct JobTraits<ColJob<T, OP>> {
   static constexpr int kInts = 2;
-  static ColJob<T, OP> make(const AcStreamShot& s) {
+  static ColJob<T, OP> make(const AcStreamShot<T>& s) {
     ColJob<T, OP> j{s.gz, s.cm, {s.z, s.z.b ? 1 : 0, 0}};
     fill_unused(j.op.a);
     return j;
   }
-  static int blocks(const AcStreamShot& s) { return (int)((s.cm.groups * s.cm.nseg + 3) / 4); }
-  static size_t smem(const AcStreamShot&) { return col_smem<T>(OP::NF); }
+  static int blocks(const AcStreamShot<T>& s) { return (int)((s.cm.groups * s.cm.nseg + 3) / 4); }
+  static size_t smem(const AcStreamShot<T>&) { return col_smem<T>(OP::NF); }
   static cudaError_t launch(const unsigned char* base, const AcBatchKind& k, cudaStream_t st) {
     auto kern = k_col_batch<T, OP>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
@@ -362,7 +384,8 @@ struct JobTraits<ColJob<T, OP>> {
     return cudaGetLastError();
   }
 };
-static bool in_kind(int kind, const AcStreamShot& s) {
+template <typename T>
+static bool in_kind(int kind, const AcStreamShot<T>& s) {
   const bool one = s.rm.nwin == 1, rx = s.x.pml && s.x.dlt, rz = s.z.pml && s.z.dlt;
   switch (kind) {
     case 0: return one && !rx;
@@ -377,17 +400,18 @@ static bool in_kind(int kind, const AcStreamShot& s) {
 }
 
 // The job and block tables of every kind in `bytes` (uploaded to a 16-byte aligned address) and where they lie.
-void ac_batch_tables(const std::vector<AcStreamShot>& shots, std::vector<unsigned char>& bytes, AcBatchKind (&k)[8]) {
+template <typename T, bool K>
+void ac_batch_tables(const std::vector<AcStreamShot<T>>& shots, std::vector<unsigned char>& bytes, AcBatchKind (&k)[8]) {
   bytes.clear();
   for (int kind = 0; kind < 8; ++kind) {
-    with_kind(kind, [&](auto proto) {
+    k[kind] = AcBatchKind{};
+    with_kind<T, K>(kind, [&](auto proto) {
       using J = decltype(proto);
       using Tr = JobTraits<J>;
       std::vector<J> jobs;
       std::vector<int> blk;
       AcBatchKind& q = k[kind];
-      q = AcBatchKind{};
-      for (const AcStreamShot& s : shots) {
+      for (const AcStreamShot<T>& s : shots) {
         if (!in_kind(kind, s)) continue;
         const int nb = Tr::blocks(s);
         for (int b = 0; b < nb; ++b) {
@@ -411,11 +435,22 @@ void ac_batch_tables(const std::vector<AcStreamShot>& shots, std::vector<unsigne
   }
 }
 
+template <typename T, bool K>
 cudaError_t launch_ac_batch(const void* base, const AcBatchKind& k, int kind, cudaStream_t st) {
   if (k.blocks == 0) return cudaSuccess;
   cudaError_t e = cudaSuccess;
-  with_kind(kind, [&](auto proto) { e = JobTraits<decltype(proto)>::launch((const unsigned char*)base, k, st); });
+  with_kind<T, K>(kind, [&](auto proto) { e = JobTraits<decltype(proto)>::launch((const unsigned char*)base, k, st); });
   return e;
 }
+
+template void ac_batch_tables<float, false>(const std::vector<AcStreamShot<float>>&, std::vector<unsigned char>&,
+                                            AcBatchKind (&)[8]);
+template void ac_batch_tables<float, true>(const std::vector<AcStreamShot<float>>&, std::vector<unsigned char>&,
+                                           AcBatchKind (&)[8]);
+template void ac_batch_tables<double, false>(const std::vector<AcStreamShot<double>>&, std::vector<unsigned char>&,
+                                             AcBatchKind (&)[8]);
+template cudaError_t launch_ac_batch<float, false>(const void*, const AcBatchKind&, int, cudaStream_t);
+template cudaError_t launch_ac_batch<float, true>(const void*, const AcBatchKind&, int, cudaStream_t);
+template cudaError_t launch_ac_batch<double, false>(const void*, const AcBatchKind&, int, cudaStream_t);
 
 }  // namespace lossk

@@ -259,19 +259,39 @@ static loss_status_t acs_rows(loss_ctx* h, Shot& s, int do_B, double acoef, doub
   return cuda_check(h, launch_ac_rows<T, K>(a, g, row_map(h->num_sms, s, 1, g, s.sy, s.sz, true), h->stream), "acoustic x kernel");
 }
 // Z1 (mode 1) or Z2 (mode 2) of the FP64 step on the engines.
+template <typename T, bool K>
 static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
   ConvAxis g;
   bool ok;
   LOSS_TRY(conv_axis(h, s, 0, &g, &ok));
-  AcZArgs<double> a = ac_z_args<double>(h, s, LineGeom{}, acoef, 0);
+  AcZArgs<T> a = ac_z_args<T>(h, s, LineGeom{}, acoef, 0);
   conv_scale(a, s, 0, acoef);
   LaunchScope ls(h, mode == 1 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2);
-  return cuda_check(h, launch_ac_cols(a, g, col_map(h->num_sms, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
+  return cuda_check(h, launch_ac_cols<T, K>(a, g, col_map(h->num_sms, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
+}
+
+// Whether the FP32 rows of this handle that the pipelined kernel would take run on the row engine: all of its shots have
+// rows of at least 513 points that qualify (a batch has one x kernel, and every shot's results are those of its own
+// schedule), outside gradients, with the default limit of the pipelined kernel's waits (a limit of the caller's own is
+// a request for them).  x part, engine against pipelined kernel: 513^2 19.9 / 21.7 us, 1025^2 28.9 / 33.8 us, 2049^2
+// 51.4 / 62.4 us, with Kahan summation 61.4 / 67.0 us; rows of 257 points and less are bound by launches either way.
+static loss_status_t rows_on_engine(loss_ctx* h, bool* on) {
+  *on = false;
+  if (h->tiled == LOSS_KERNELS_CONVOLUTION_ITEMS || h->in_gradient || h->wait_polls != kDefaultWaitPolls) return LOSS_OK;
+  for (Shot& s : h->shots) {
+    if (s.n[2] < 512 || any_nonuniform(s) || !tiled_ok(h, s) || !conv_size_ok(s)) return LOSS_OK;
+    ConvAxis g;
+    bool ok;
+    LOSS_TRY(conv_axis(h, s, 2, &g, &ok));
+    if (!ok) return LOSS_OK;
+  }
+  *on = true;
+  return LOSS_OK;
 }
 
 // x part of the FP32 step (sub-step B and the x part of A, or the latter alone): the pipelined row kernel when a
-// row fits its shared-memory stages; else the row engine; else (and in the forward runs of a gradient, and for the
-// family that asks for them) the (row, patch) item kernels, two launches.
+// row fits its shared-memory stages, unless rows_on_engine; else the row engine; else (and in the forward runs of a
+// gradient, and for the family that asks for them) the (row, patch) item kernels, two launches.
 template <bool K>
 static loss_status_t xpart(loss_ctx* h, Shot& s, int do_B, double acoef, double amp) {
   int threads;
@@ -279,6 +299,9 @@ static loss_status_t xpart(loss_ctx* h, Shot& s, int do_B, double acoef, double 
   LOSS_TRY(ensure_delta_weights(h, s, 2));
   t.Wd = s.Wd[2];
   t.ncross = (int)s.len[0];
+  bool rows;
+  LOSS_TRY(rows_on_engine(h, &rows));
+  if (rows && xp_ok(h, s, t)) return acs_rows<float, K>(h, s, do_B, acoef, amp);
   if (!xp_ok(h, s, t) && h->tiled != LOSS_KERNELS_CONVOLUTION_ITEMS && !h->in_gradient && conv_size_ok(s) &&
       xt_smem(t) <= (size_t)h->smem_optin) {
     ConvAxis g;
@@ -361,8 +384,8 @@ static loss_status_t acoustic2d_start(loss_ctx* h, Shot& s) {
   LOSS_TRY(acs_ok(h, s, &stream));
   if (stream) {
     LOSS_TRY((acs_rows<T, K>(h, s, 0, 0.5 * dt, 0.0)));
-    LOSS_TRY(acs_cols(h, s, 1, 0.5 * dt));
-    return acs_cols(h, s, 2, 0.0);
+    LOSS_TRY((acs_cols<T, K>(h, s, 1, 0.5 * dt)));
+    return acs_cols<T, K>(h, s, 2, 0.0);
   }
   LOSS_TRY((ac_x<T, K>(h, s, 0, 0.5 * dt, 0.0)));
   return ac_z<T, K>(h, s, 0.5 * dt, 1);
@@ -408,8 +431,8 @@ static loss_status_t acoustic2d_step(loss_ctx* h, Shot& s) {
     LOSS_TRY(tz<K>(h, s, 1, dt));
     LOSS_TRY(tz<K>(h, s, 2, 0.0));
   } else if (stream) {
-    LOSS_TRY(acs_cols(h, s, 1, dt));
-    LOSS_TRY(acs_cols(h, s, 2, 0.0));
+    LOSS_TRY((acs_cols<T, K>(h, s, 1, dt)));
+    LOSS_TRY((acs_cols<T, K>(h, s, 2, 0.0)));
   } else {
     LOSS_TRY((ac_z<T, K>(h, s, dt, 1)));
   }
@@ -433,7 +456,7 @@ static loss_status_t acoustic2d_unstagger(loss_ctx* h, Shot& s) {
   LOSS_TRY(acs_ok(h, s, &stream));
   if (stream) {
     LOSS_TRY((acs_rows<T, K>(h, s, 0, -0.5 * dt, 0.0)));
-    LOSS_TRY(acs_cols(h, s, 1, -0.5 * dt));
+    LOSS_TRY((acs_cols<T, K>(h, s, 1, -0.5 * dt)));
     s.staggered = false;
     return LOSS_OK;
   }
@@ -980,7 +1003,12 @@ static loss_status_t batch_launch_step(loss_ctx* h) {
       const int* bunit = unit0 + S + 1;
       const int* bshot = bunit + B.xpgrid + 1;
       const int* zt0 = bshot + B.xpgrid;
-      {
+      for (int k = 0; B.rows && k < 5; ++k) {
+        if (B.ask[k].blocks == 0) continue;
+        LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
+        LOSS_TRY(cuda_check(h, launch_ac_batch<T, K>(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
+      }
+      if (!B.rows) {
         LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
         LOSS_TRY(cuda_check(h, launch_xp_batch<K>((const XpShot*)B.xptab, unit0, bunit, bshot, B.xl, B.xpthreads,
                                                   B.xpgrid, h->dflag, h->wait_polls, h->stream),
@@ -1008,7 +1036,7 @@ static loss_status_t batch_launch_step(loss_ctx* h) {
     for (int k = 0; k < 8; ++k) {
       if (B.ask[k].blocks == 0) continue;
       LaunchScope ls(h, kid[k]);
-      LOSS_TRY(cuda_check(h, launch_ac_batch(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
+      LOSS_TRY(cuda_check(h, launch_ac_batch<T, K>(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
     }
     if (B.npost) {
       LaunchScope ls(h, LOSS_KERNEL_GATHER);
@@ -1201,29 +1229,32 @@ static loss_status_t conv_tables(loss_ctx* h) {
   return LOSS_OK;
 }
 
-// Tables of the batched FP64 step on the engines.
+// Tables of the batched step on the engines (FP32: of its rows).
+template <typename T, bool K>
 static loss_status_t acs_tables(loss_ctx* h) {
   BatchState& B = h->batch;
-  std::vector<AcStreamShot> v;
+  std::vector<AcStreamShot<T>> v;
   for (size_t i = 0; i < h->shots.size(); ++i) {
     Shot& s = h->shots[i];
-    AcStreamShot q{};
+    AcStreamShot<T> q{};
     bool ok;
     LOSS_TRY(conv_axis(h, s, 2, &q.gx, &ok));
-    LOSS_TRY(conv_axis(h, s, 0, &q.gz, &ok));
     q.rm = row_map(h->num_sms, s, 1, q.gx, s.sy, s.sz, true);
-    q.cm = col_map(h->num_sms, s, 0, s.sy, s.sz);
-    q.x = ac_x_args<double>(h, s, LineGeom{}, 1, s.d.dt, 0.0);
+    q.x = ac_x_args<T>(h, s, LineGeom{}, 1, s.d.dt, 0.0);
     q.x.src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
     q.x.src.amp_tab = s.amp_tab;
     q.x.src.clk = B.clk + i;
     conv_scale(q.x, s, 2, s.d.dt);
-    q.z = ac_z_args<double>(h, s, LineGeom{}, s.d.dt, 0);
-    conv_scale(q.z, s, 0, s.d.dt);
+    if (sizeof(T) == 8) {
+      LOSS_TRY(conv_axis(h, s, 0, &q.gz, &ok));
+      q.cm = col_map(h->num_sms, s, 0, s.sy, s.sz);
+      q.z = ac_z_args<T>(h, s, LineGeom{}, s.d.dt, 0);
+      conv_scale(q.z, s, 0, s.d.dt);
+    }
     v.push_back(q);
   }
   std::vector<unsigned char> bytes;
-  ac_batch_tables(v, bytes, B.ask);
+  ac_batch_tables<T, K>(v, bytes, B.ask);
   if (bytes != B.host[6]) ++B.astab_version;  // the launch shapes may differ with the contents: capture again
   return upload_table(h, 6, bytes, &B.astab);
 }
@@ -1234,6 +1265,8 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   const int S = (int)h->shots.size();
   B.conv = false;
   if constexpr (sizeof(T) == 4) B.conv = conv_batch_ok(h);
+  B.rows = false;
+  if (B.conv) LOSS_TRY(rows_on_engine(h, &B.rows));
   B.stream = sizeof(T) == 8;  // every FP64 shot on the engines (batch_eligible leaves mixed handles per shot)
   for (Shot& s : h->shots) {
     bool ok = false;
@@ -1321,8 +1354,9 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   jobs.insert(jobs.end(), post.begin(), post.end());
   if (B.conv) {
     if constexpr (sizeof(T) == 4) LOSS_TRY(conv_tables<K>(h));
+    if (B.rows) LOSS_TRY((acs_tables<T, K>(h)));
   } else if (B.stream) {
-    LOSS_TRY(acs_tables(h));
+    LOSS_TRY((acs_tables<T, K>(h)));
   } else {
     LOSS_TRY(upload_table(h, 0, as_bytes(xa), &B.xtab));
     LOSS_TRY(upload_table(h, 1, as_bytes(za), &B.ztab));
@@ -1360,7 +1394,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
                                       B.xl.total, B.tzthreads[0], B.tzthreads[1], B.tzlogc[0], B.tzlogc[1],
                                       B.tztiles, B.tzgrid[0], B.tzgrid[1],
                                       (int64_t)B.tzsmem[0], (int64_t)B.tzsmem[1], (int64_t)h->wait_polls,
-                                      B.stream ? 1 : 0, (int64_t)(intptr_t)B.astab, B.astab_version};
+                                      B.stream ? 1 : 0, B.rows ? 1 : 0, (int64_t)(intptr_t)B.astab, B.astab_version};
     if (!B.gexec || sig != B.gsig) {
       LOSS_TRY((capture_graph<T, K>(h, k)));
       B.gsig = sig;

@@ -322,14 +322,15 @@ struct RowMap {
   int64_t sz, sy;
   int rows, groups, ny, nch, gw, nwin, vec, wbytes, sms;
 };
-// One shot of a batched FP64 acoustic step on these engines, and one launch of it: its job and block tables at byte
-// offsets of the uploaded tables.
+// One shot of a batched acoustic step on these engines (FP32: its rows), and one launch of it: its job and block tables
+// at byte offsets of the uploaded tables.
+template <typename T>
 struct AcStreamShot {
   ConvAxis gx, gz;
   RowMap rm;
   ColMap cm;
-  AcXArgs<double> x;
-  AcZArgs<double> z;
+  AcXArgs<T> x;
+  AcZArgs<T> z;
 };
 struct AcBatchKind {
   int blocks = 0;

@@ -187,3 +187,30 @@ def test_derivative_operators(pkg, prec, geom):
         g.sync()
         assert np.abs(over.cpu().numpy() - r1).max() < t1 * np.abs(r1).max(), axis
     g.close()
+
+
+@pytest.mark.parametrize("graph", [0, 3])
+@pytest.mark.parametrize("prec", ["fp32", "fp32_kahan"])
+def test_batched_long_rows(pkg, prec, graph):
+    """FP32 rows of 513 points and more in one launch for all shots (row engine): the per-shot schedule's bits, and the
+    fields of the pipelined row kernel (the items family's rounding apart) to the run tolerance."""
+    geoms = [((64, 512), (2, 4), 20), ((96, 1024), (3, 8), 12), ((48, 520), (1, 13), 16)]
+    ws = [_acoustic(pkg, n, p, n_nb, prec, 50 + k) for k, (n, p, n_nb) in enumerate(geoms)]
+    res = []
+    for mode in range(3):
+        g = pkg.Grid.from_workloads(ws)
+        g.set_schedule(mode == 0, graph if mode == 0 else 0)
+        if mode == 2:
+            g.set_wait_limit(1 << 20)  # a limit of one's own keeps the kernel that waits
+        for s, w in enumerate(ws):
+            for f, a in _fields(w, prec, 90 + s).items():
+                g.set_field(s, f, a)
+        g.step(3)
+        g.get_field(0, "v1")  # back to the integer time level in between
+        g.step(7)
+        res.append([[g.get_field(s, f) for f in ("sigma", "v1", "v3")] + [g.record(s)["_all"]] for s in range(len(ws))])
+        g.close()
+    for s in range(len(ws)):
+        for a, b, c in zip(res[0][s], res[1][s], res[2][s]):
+            assert np.array_equal(a, b), s
+            assert np.abs(a - c).max() <= 1e-5 * np.abs(c).max(), s
