@@ -344,10 +344,14 @@ void ac_batch_tables(const std::vector<AcStreamShot<T>>& shots, std::vector<unsi
 template <typename T, bool K>
 cudaError_t launch_ac_batch(const void* base, const AcBatchKind& k, int kind, cudaStream_t st);
 // Blocks of a k_row launch (4 warps each, kblocks resident per SM).
-inline int row_blocks(const RowMap& rm, int kblocks) {
-  const int need = (rm.groups * rm.nwin + 3) / 4, most = rm.sms * kblocks;
+// Blocks of 4 warps, or of one when there are fewer than 8 warps for each SM: a block's warps share the SM's FP64 pipe (16
+// cycles per warp instruction), and 263 column warps in 66 blocks left 86 SMs idle.
+inline int engine_warps(int64_t warps, int sms) { return warps < 8LL * sms ? 1 : 4; }
+inline int row_blocks(const RowMap& rm, int kblocks, int warps) {
+  const int need = (rm.groups * rm.nwin + warps - 1) / warps, most = rm.sms * kblocks * 4 / warps;
   return need < most ? need : most;
 }
+inline unsigned col_blocks(const ColMap& cm, int warps) { return (unsigned)((cm.groups * cm.nseg + warps - 1) / warps); }
 // loss_kernels_elastic.cu: elastic y / z tile passes (FP32)
 size_t elt_smem(const ElTile& g, int logc);
 template <bool KAHAN>

@@ -266,22 +266,23 @@ static void fill_unused(AcZArgs<T>& a) {
 
 template <typename T, class OP>
 static cudaError_t go_row(const ConvAxis& g, const RowMap& rm, const OP& op, cudaStream_t st) {
-  const size_t smem = (size_t)4 * rm.wbytes;
+  const size_t smem = (size_t)rm.warps * rm.wbytes;
   auto kern = k_row<T, OP>;
   if (smem > 32 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
     if (e != cudaSuccess) return e;
   }
-  kern<<<row_blocks(rm, OP::kBlocks), 128, smem, st>>>(g, rm, op);
+  kern<<<row_blocks(rm, OP::kBlocks, rm.warps), 32 * rm.warps, smem, st>>>(g, rm, op);
   return cudaGetLastError();
 }
 template <typename T, class OP>
 static cudaError_t go_col(const ConvAxis& g, const ColMap& cm, const OP& op, cudaStream_t st) {
-  const size_t smem = col_smem<T>(OP::NF);
+  const size_t smem = col_smem<T>(OP::NF, cm.warps);
   auto kern = k_col<T, OP>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)col_smem<T>(OP::NF, 4));
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)((cm.groups * cm.nseg + 3) / 4), 128, smem, st>>>(g, cm, op);
+  kern<<<col_blocks(cm, cm.warps), 32 * cm.warps, smem, st>>>(g, cm, op);
   return cudaGetLastError();
 }
 
@@ -354,12 +355,12 @@ struct JobTraits<RowJob<T, OP>> {
     fill_unused(j.op.a);
     return j;
   }
-  static int blocks(const AcStreamShot<T>& s) { return row_blocks(s.rm, OP::kBlocks); }
+  static int blocks(const AcStreamShot<T>& s) { return row_blocks(s.rm, OP::kBlocks, 4); }
   static size_t smem(const AcStreamShot<T>& s) { return (size_t)4 * s.rm.wbytes; }
   static cudaError_t launch(const unsigned char* base, const AcBatchKind& k, cudaStream_t st) {
     auto kern = k_row_batch<T, OP>;
     if (k.smem > 32 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
       if (e != cudaSuccess) return e;
     }
     kern<<<k.blocks, 128, k.smem, st>>>((const RowJob<T, OP>*)(base + k.jobs), (const int4*)(base + k.blk));
@@ -374,8 +375,8 @@ struct JobTraits<ColJob<T, OP>> {
     fill_unused(j.op.a);
     return j;
   }
-  static int blocks(const AcStreamShot<T>& s) { return (int)((s.cm.groups * s.cm.nseg + 3) / 4); }
-  static size_t smem(const AcStreamShot<T>&) { return col_smem<T>(OP::NF); }
+  static int blocks(const AcStreamShot<T>& s) { return (int)col_blocks(s.cm, 4); }
+  static size_t smem(const AcStreamShot<T>&) { return col_smem<T>(OP::NF, 4); }
   static cudaError_t launch(const unsigned char* base, const AcBatchKind& k, cudaStream_t st) {
     auto kern = k_col_batch<T, OP>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);

@@ -89,7 +89,8 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
   T* dsm = reinterpret_cast<T*>(sm + (size_t)warp * rm.wbytes);
   const int gl = lane & (gw - 1), k = lane / gw;
   const int items = rm.groups * rm.nwin;
-  for (int item = blockIdx.x * 4 + warp; item < items; item += gridDim.x * 4) {
+  const int nw = blockDim.x >> 5;
+  for (int item = blockIdx.x * nw + warp; item < items; item += gridDim.x * nw) {
     const int grp = rm.nwin == 1 ? item : item / rm.nwin, win = item - grp * rm.nwin;
     const int c0 = win * (32 - 2 * Conv<T>::W);
     const int c1 = min(rm.nch, c0 + gw);
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, con
   fill_reach(rs, g);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t item = (int64_t)blockIdx.x * 4 + warp;
+  const int64_t item = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (item >= cm.groups * cm.nseg) return;
   const int seg = (int)(item / cm.groups);
   const int64_t q0 = (item - (int64_t)seg * cm.groups) * 32 + lane;
@@ -318,48 +319,49 @@ template <typename T>
 cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, const T* f, T* d1, T* d2,
                                 T s1, T s2, cudaStream_t st) {
   if (x) {
-    const size_t smem = (size_t)4 * rm.wbytes;
+    const size_t smem = (size_t)rm.warps * rm.wbytes;
     auto go = [&](auto op, auto kern) {
       if (smem > 32 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
         if (e != cudaSuccess) return e;
       }
-      kern<<<row_blocks(rm, decltype(op)::kBlocks), 128, smem, st>>>(g, rm, op);
+      kern<<<row_blocks(rm, decltype(op)::kBlocks, rm.warps), 32 * rm.warps, smem, st>>>(g, rm, op);
       return cudaGetLastError();
     };
     if (d2) return go(DerivRowOp<T, true>{f, d1, d2, s1, s2, rm.vec, 0}, k_row<T, DerivRowOp<T, true>>);
     return go(DerivRowOp<T, false>{f, d1, d1, s1, s2, rm.vec, 0}, k_row<T, DerivRowOp<T, false>>);
   }
-  const unsigned grid = (unsigned)((cm.groups * cm.nseg + 3) / 4);
   auto go = [&](auto op, auto kern, size_t smem) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)col_smem<T>(1, 4, true));
     if (e != cudaSuccess) return e;
-    kern<<<grid, 128, smem, st>>>(g, cm, op);
+    kern<<<col_blocks(cm, cm.warps), 32 * cm.warps, smem, st>>>(g, cm, op);
     return cudaGetLastError();
   };
   if constexpr (sizeof(T) == 4)
-    if (d2) return go(DerivColOp<T, true>{f, d1, d2, s1, s2}, k_col<T, DerivColOp<T, true>>, col_smem<T>(1, true));
-  return go(DerivColOp<T, false>{f, d1, d1, s1, s2}, k_col<T, DerivColOp<T, false>>, col_smem<T>(1));
+    if (d2) return go(DerivColOp<T, true>{f, d1, d2, s1, s2}, k_col<T, DerivColOp<T, true>>, col_smem<T>(1, cm.warps, true));
+  return go(DerivColOp<T, false>{f, d1, d1, s1, s2}, k_col<T, DerivColOp<T, false>>, col_smem<T>(1, cm.warps));
 }
 
 template <typename T>
 cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, bool acc, const T* in,
                                 T* out, T scale, cudaStream_t st) {
   if (x) {
-    const size_t smem = (size_t)4 * rm.wbytes;
+    const size_t smem = (size_t)rm.warps * rm.wbytes;
     auto kern = acc ? k_row_trans<T, true> : k_row_trans<T, false>;
     if (smem > 32 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
       if (e != cudaSuccess) return e;
     }
-    kern<<<row_blocks(rm, 4), 128, smem, st>>>(g, rm, in, out, scale);
+    kern<<<row_blocks(rm, 4, rm.warps), 32 * rm.warps, smem, st>>>(g, rm, in, out, scale);
     return cudaGetLastError();
   }
-  const size_t smem = col_smem<T>(1);
+  const size_t smem = col_smem<T>(1, cm.warps);
   auto kern = acc ? k_col_trans<T, true> : k_col_trans<T, false>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)col_smem<T>(1, 4, true));
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)((cm.groups * cm.nseg + 3) / 4), 128, smem, st>>>(g, cm, in, out, scale);
+  kern<<<col_blocks(cm, cm.warps), 32 * cm.warps, smem, st>>>(g, cm, in, out, scale);
   return cudaGetLastError();
 }
 

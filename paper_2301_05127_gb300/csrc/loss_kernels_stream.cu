@@ -232,23 +232,24 @@ struct ElRowOp {
 
 template <typename T, class OP>
 static cudaError_t launch_col(const ConvAxis& g, const ColMap& cm, const OP& op, cudaStream_t st) {
-  const size_t smem = col_smem<T>(OP::NF);
+  const size_t smem = col_smem<T>(OP::NF, cm.warps);
   auto kern = k_col<T, OP>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)col_smem<T>(OP::NF, 4));
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)((cm.groups * cm.nseg + 3) / 4), 128, smem, st>>>(g, cm, op);
+  kern<<<col_blocks(cm, cm.warps), 32 * cm.warps, smem, st>>>(g, cm, op);
   return cudaGetLastError();
 }
 
 template <typename T, class OP>
 static cudaError_t launch_row(const ConvAxis& g, const RowMap& rm, const OP& op, cudaStream_t st) {
-  const size_t smem = (size_t)4 * rm.wbytes;
+  const size_t smem = (size_t)rm.warps * rm.wbytes;
   auto kern = k_row<T, OP>;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 32 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
     if (e != cudaSuccess) return e;
   }
-  kern<<<row_blocks(rm, OP::kBlocks), 128, smem, st>>>(g, rm, op);
+  kern<<<row_blocks(rm, OP::kBlocks, rm.warps), 32 * rm.warps, smem, st>>>(g, rm, op);
   return cudaGetLastError();
 }
 

@@ -672,6 +672,7 @@ ColMap col_map(int num_sms, const Shot& s, int k, int64_t py, int64_t pz) {
   const int nseg = (int)std::min<int64_t>(std::max<int64_t>(want / m.groups, 1), std::max(np / 40, 1));
   m.seglen = ((np + nseg - 1) / nseg + 7) & ~7;
   m.nseg = (np + m.seglen - 1) / m.seglen;
+  m.warps = engine_warps(m.groups * m.nseg, num_sms);
   return m;
 }
 
@@ -691,6 +692,7 @@ RowMap row_map(int num_sms, const Shot& s, int nf, const ConvAxis& g, int64_t py
   const int nj = std::min(g.p + 1, (8 * m.gw + 1 + 2 * std::max(g.Q, g.R)) / g.M + 2);
   m.wbytes = (nf * (32 / m.gw) * nj * es + 15) & ~15;
   m.sms = num_sms;
+  m.warps = engine_warps((int64_t)m.groups * m.nwin, num_sms);
   return m;
 }
 

@@ -189,7 +189,7 @@ __device__ __forceinline__ void col_block(const ConvAxis& g, const ColMap& cm, c
   const ConvTap* taps = stage_taps(g, tsm);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t item = (int64_t)bid * 4 + warp;
+  const int64_t item = (int64_t)bid * (blockDim.x >> 5) + warp;
   if (item >= cm.groups * cm.nseg) return;
   const int seg = (int)(item / cm.groups);
   const int64_t q0 = (item - (int64_t)seg * cm.groups) * 32 + lane;
@@ -496,10 +496,12 @@ __global__ void __launch_bounds__(128, OP::kBlocks)
   col_block<T>(j.g, j.cm, j.op, w.y, sm);
 }
 
-// Dynamic shared memory of a k_col block.
+// Dynamic shared memory of a k_col block.  (The kernels' limits are set to one size whatever the launch, so that threads
+// with handles of their own do not lower each other's.)
+constexpr int kRowSmemMax = 220 * 1024;
 template <typename T>
-constexpr size_t col_smem(int nf, bool second = false) {
-  return (size_t)4 * (Conv<T>::W + 2 + (second ? 1 : 0)) * 8 * nf * 32 * sizeof(T);
+constexpr size_t col_smem(int nf, int warps, bool second = false) {
+  return (size_t)warps * (Conv<T>::W + 2 + (second ? 1 : 0)) * 8 * nf * 32 * sizeof(T);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -675,7 +677,8 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
   T* dsm = reinterpret_cast<T*>(sm + (size_t)warp * rm.wbytes);
   const int gl = lane & (gw - 1), k = lane / gw;
   const int items = rm.groups * rm.nwin;
-  for (int item = bid * 4 + warp; item < items; item += nblk * 4) {
+  const int nw = blockDim.x >> 5;
+  for (int item = bid * nw + warp; item < items; item += nblk * nw) {
     const int grp = rm.nwin == 1 ? item : item / rm.nwin, win = item - grp * rm.nwin;
     const int c0 = win * (32 - 2 * Conv<T>::W);              // first chunk of the window
     const int c1 = min(rm.nch, c0 + gw);                     // past its last

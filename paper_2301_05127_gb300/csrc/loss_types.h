@@ -314,13 +314,14 @@ struct ConvAxis {
 struct ColMap {
   int64_t lines, groups, inner, so, stride;
   int nseg, seglen;
+  int warps, pad;  // per block of the launch
 };
 // Contiguous rows of an array: row q starts at (q / ny) * sz + (q % ny) * sy; nch chunks per row, gw lanes per row
 // window, nwin windows per row, groups of 32 / gw rows; vec: rows start on 16-byte boundaries and are readable to the
 // next multiple of 8 positions; wbytes: shared memory of a warp; sms: multiprocessors.
 struct RowMap {
   int64_t sz, sy;
-  int rows, groups, ny, nch, gw, nwin, vec, wbytes, sms;
+  int rows, groups, ny, nch, gw, nwin, vec, wbytes, sms, warps;
 };
 // One shot of a batched acoustic step on these engines (FP32: its rows), and one launch of it: its job and block tables
 // at byte offsets of the uploaded tables.
