@@ -257,8 +257,8 @@ loss_status_t loss_set_tile(loss_handle_t handle, int32_t kernel, int32_t thread
  * instead).  batched != 0 (the default): a handle whose shots are all 2-D acoustic grids of one precision advances
  * them together, each step being one persistent launch per kernel over the work of all shots, one launch per
  * receiver phase and a clock tick.  The kernels are those of the per-shot step: with the truncated-convolution
- * family (FP32, when every shot qualifies) the x kernel over row units of all shots, then Z1 and Z2 over the z
- * tiles of all shots; otherwise the line kernels, x and z over bundles of whole lines.  The source amplitude and
+ * family (FP32, when every shot qualifies) the x kernel over rows of all shots, then Z1 and Z2 over the z
+ * tiles of all shots; FP64 shots that qualify likewise; otherwise the line kernels, x and z over bundles of whole lines.  The source amplitude and
  * the trace row of each step are read from per-shot device counters, so the launches of every step are
  * identical.  graph_steps > 0: such handles (also with a single shot) capture graph_steps steps
  * once in a CUDA graph and replay it (the remainder of a loss_step call runs as plain launches); the graph is
@@ -267,14 +267,17 @@ loss_status_t loss_set_tile(loss_handle_t handle, int32_t kernel, int32_t thread
  * for steps replayed from a graph; launches are counted.  LOSS_E_ARG if graph_steps < 0. */
 loss_status_t loss_set_schedule(loss_handle_t handle, int32_t batched, int32_t graph_steps);
 
-/* Kernel family of the per-shot FP32 2-D acoustic step: LOSS_KERNELS_LINE = whole grid lines on chip with the
- * chunked Thomas solve of the patch systems (the form every other grid and the batched schedule use);
+/* Kernel family of the time steps: LOSS_KERNELS_LINE = whole grid lines on chip with the
+ * chunked Thomas solve of the patch systems;
  * LOSS_KERNELS_CONVOLUTION (the default) = the truncated-convolution form: the same patch systems solved through
  * the closed-form inverse of the (1, 4, 1) operator, truncated where |sqrt(3) - 2|^k < 1e-9, with exact patch-end
  * corrections from the PMBC junction values (x rows pipelined through TMA bulk copies, z lines on independent
  * 32-column x one-patch tiles; rows the pipelined kernel does not take, longer than 2049 points or with patches
  * whose length is not a multiple of 8, go to independent (row, patch) items in two launches);
- * LOSS_KERNELS_CONVOLUTION_ITEMS = the same with every row on (row, patch) items.  All agree with the FP64 oracle
+ * LOSS_KERNELS_CONVOLUTION_ITEMS = the same with every row on (row, patch) items.  In the convolution family FP64 2-D
+ * steps, 3-D elastic steps, FP32 rows of 513 points and more and rows that the pipelined kernel does not take run on
+ * kernels that march lines and rows without block barriers, where patches are long enough for them (at least 8 points
+ * more than a junction's correction reaches, 40 points per axis) and arrays hold at most 4 GB.  All agree with the FP64 oracle
  * at the FP32 tolerance; they differ in rounding.  LOSS_E_ARG for another value. */
 enum { LOSS_KERNELS_LINE = 0, LOSS_KERNELS_CONVOLUTION = 1, LOSS_KERNELS_CONVOLUTION_ITEMS = 2 };
 loss_status_t loss_set_kernels(loss_handle_t handle, int32_t family);
