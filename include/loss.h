@@ -258,7 +258,8 @@ loss_status_t loss_set_tile(loss_handle_t handle, int32_t kernel, int32_t thread
  * them together, each step being one persistent launch per kernel over the work of all shots, one launch per
  * receiver phase and a clock tick.  The kernels are those of the per-shot step: with the truncated-convolution
  * family (FP32, when every shot qualifies) the x kernel over rows of all shots, then Z1 and Z2 over the z
- * tiles of all shots; FP64 shots that qualify likewise; otherwise the line kernels, x and z over bundles of whole lines.  The source amplitude and
+ * tiles of all shots; FP64 shots by themselves, those that qualify for the column and row kernels on these and the others
+ * on the line kernels; otherwise the line kernels, x and z over bundles of whole lines.  The source amplitude and
  * the trace row of each step are read from per-shot device counters, so the launches of every step are
  * identical.  graph_steps > 0: such handles (also with a single shot) capture graph_steps steps
  * once in a CUDA graph and replay it (the remainder of a loss_step call runs as plain launches); the graph is

@@ -140,8 +140,8 @@ struct BatchState {
   bool conv = false;
   void* xptab = nullptr;  // XpShot[n_shots]
   void* tztab = nullptr;  // TzShot[2 n_shots]
-  // FP64 form on the barrier-free engines: job and block tables of the launches of a step
-  bool stream = false;
+  // shots on the barrier-free engines (FP64; job and block tables of the launches of a step) and on the line kernels
+  int nengine = 0, nline = 0;
   void* astab = nullptr;
   AcBatchKind ask[8];
   bool rows = false;  // with conv: the x part runs on the row engine
@@ -264,7 +264,7 @@ RowMap row_map(int num_sms, const Shot& s, int nf, const ConvAxis& g, int64_t py
 loss_status_t step_shot(loss_ctx* h, Shot& s, bool head = false, bool more = false);  // head, more: as nu_step
 loss_status_t unstagger(loss_ctx* h, Shot& s);
 loss_status_t stagger_shot(loss_ctx* h, Shot& s);
-bool batch_eligible(loss_ctx* h);
+bool batch_eligible(const loss_ctx* h);
 bool conv_z_used(const loss_ctx* h);  // some shot's FP32 step runs the convolution z tiles
 loss_status_t step_batched(loss_ctx* h, int64_t n_steps);
 void batch_release(loss_ctx* h);

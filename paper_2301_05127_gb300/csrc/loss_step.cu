@@ -868,7 +868,7 @@ static loss_status_t elastic3d_unstagger(loss_ctx* h, Shot& s) {
 
 static bool conv_batch_ok(const loss_ctx* h);
 
-bool batch_eligible(loss_ctx* h) {
+bool batch_eligible(const loss_ctx* h) {
   if (h->shots.empty()) return false;
   if (!(h->graph_steps > 0 || (h->batched && h->shots.size() > 1))) return false;
   const Shot& s0 = h->shots[0];
@@ -881,16 +881,6 @@ bool batch_eligible(loss_ctx* h) {
   if (s0.esize == 4 && !conv_batch_ok(h))
     for (const Shot& s : h->shots)
       if (s.n[2] > 2048) return false;
-  // FP64: the batch takes the engines or the line kernels for all shots; handles that mix the two go per shot
-  if (s0.esize == 8) {
-    int n = 0;
-    for (Shot& s : h->shots) {
-      bool ok = false;
-      acs_ok(h, s, &ok);
-      n += ok ? 1 : 0;
-    }
-    if (n != 0 && n != (int)h->shots.size()) return false;
-  }
   return true;
 }
 
@@ -927,13 +917,14 @@ static loss_status_t ensure_amp(loss_ctx* h, Shot& s, int64_t upto) {
   return LOSS_OK;
 }
 
-// Geometry of every shot for one batched kernel, with one block size for all: the largest per-shot default
+// Geometry of the given shots for one batched line kernel, with one block size for all: the largest per-shot default
 // block (or the loss_set_tile target), each shot taking the widest bundle that fits in it.
-static loss_status_t batch_geoms(loss_ctx* h, int k, int kid, int nbuf, int nstage, std::vector<LineGeom>& gs,
-                                 int* logc, int* threads, size_t* smem) {
+static loss_status_t batch_geoms(loss_ctx* h, const std::vector<int>& shots, int k, int kid, int nbuf, int nstage,
+                                 std::vector<LineGeom>& gs, int* logc, int* threads, size_t* smem) {
   int target = h->tile_threads[kid];
   if (target <= 0 && h->lines_per_block[kid] <= 0) {
-    for (Shot& s : h->shots) {
+    for (int i : shots) {
+      Shot& s = h->shots[i];
       LineGeom g;
       int lc, t;
       LOSS_TRY(line_geom(h, s, k, s.sz, s.sy, &g, &lc, &t, nbuf, nstage, 0, h->chunk_log2[kid]));
@@ -941,12 +932,12 @@ static loss_status_t batch_geoms(loss_ctx* h, int k, int kid, int nbuf, int nsta
     }
   }
   if (target > kBatchThreads) target = kBatchThreads;
-  gs.resize(h->shots.size());
+  gs.resize(shots.size());
   *logc = -1;
   *threads = 0;
   *smem = 0;
-  for (size_t i = 0; i < h->shots.size(); ++i) {
-    Shot& s = h->shots[i];
+  for (size_t i = 0; i < shots.size(); ++i) {
+    Shot& s = h->shots[shots[i]];
     int lc, t;
     LOSS_TRY(line_geom(h, s, k, s.sz, s.sy, &gs[i], &lc, &t, nbuf, nstage, h->lines_per_block[kid], h->chunk_log2[kid],
                        target));
@@ -1032,32 +1023,27 @@ static loss_status_t batch_launch_step(loss_ctx* h) {
       return cuda_check(h, launch_tick(B.clk, S, h->stream), "clock tick");
     }
   }
-  if (B.stream) {
-    const int kid[8] = {LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_X,
-                        LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_Z, LOSS_KERNEL_ACOUSTIC_Z, LOSS_KERNEL_ACOUSTIC_Z2};
-    for (int k = 0; k < 8; ++k) {
+  // shots on the engines and shots on the line kernels, x then z (a shot has its launches from one of the two)
+  auto engine = [&](int k0, int k1) -> loss_status_t {
+    for (int k = k0; k < k1; ++k) {
       if (B.ask[k].blocks == 0) continue;
-      LaunchScope ls(h, kid[k]);
+      LaunchScope ls(h, k < 5 ? LOSS_KERNEL_ACOUSTIC_X : (k < 7 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2));
       LOSS_TRY(cuda_check(h, launch_ac_batch<T, K>(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
     }
-    if (B.npost) {
-      LaunchScope ls(h, LOSS_KERNEL_GATHER);
-      LOSS_TRY(cuda_check(h, launch_gather_batch<T>(jobs + B.npre, B.npost, B.post_max, h->stream),
-                          "batched receiver gather"));
-    }
-    LaunchScope ls(h, LOSS_KERNEL_CLOCK);
-    return cuda_check(h, launch_tick(B.clk, S, h->stream), "clock tick");
-  }
-  {
+    return LOSS_OK;
+  };
+  if (B.nengine) LOSS_TRY(engine(0, 5));
+  if (B.nline) {
     LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
-    LOSS_TRY(cuda_check(h, launch_ac_x_batch<T, K>((const AcXArgs<T>*)B.xtab, B.tile0, S, B.xtiles, B.xlogc,
+    LOSS_TRY(cuda_check(h, launch_ac_x_batch<T, K>((const AcXArgs<T>*)B.xtab, B.tile0, B.nline, B.xtiles, B.xlogc,
                                                    B.xthreads, B.xsmem, B.xgrid, h->stream),
                         "batched acoustic x kernel"));
   }
-  {
+  if (B.nengine) LOSS_TRY(engine(5, 8));
+  if (B.nline) {
     LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_Z);
-    LOSS_TRY(cuda_check(h, launch_ac_z_batch<T, K>((const AcZArgs<T>*)B.ztab, B.tile0 + S + 1, S, B.ztiles, B.zlogc,
-                                                   B.zthreads, B.zsmem, B.zgrid, h->stream),
+    LOSS_TRY(cuda_check(h, launch_ac_z_batch<T, K>((const AcZArgs<T>*)B.ztab, B.tile0 + B.nline + 1, B.nline, B.ztiles,
+                                                   B.zlogc, B.zthreads, B.zsmem, B.zgrid, h->stream),
                         "batched acoustic z kernel"));
   }
   if (B.npost) {
@@ -1231,12 +1217,12 @@ static loss_status_t conv_tables(loss_ctx* h) {
   return LOSS_OK;
 }
 
-// Tables of the batched step on the engines (FP32: of its rows).
+// Tables of the batched step on the engines (FP32: of its rows) for the given shots.
 template <typename T, bool K>
-static loss_status_t acs_tables(loss_ctx* h) {
+static loss_status_t acs_tables(loss_ctx* h, const std::vector<int>& shots) {
   BatchState& B = h->batch;
   std::vector<AcStreamShot<T>> v;
-  for (size_t i = 0; i < h->shots.size(); ++i) {
+  for (int i : shots) {
     Shot& s = h->shots[i];
     AcStreamShot<T> q{};
     bool ok;
@@ -1269,18 +1255,23 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   if constexpr (sizeof(T) == 4) B.conv = conv_batch_ok(h);
   B.rows = false;
   if (B.conv) LOSS_TRY(rows_on_engine(h, &B.rows));
-  B.stream = sizeof(T) == 8;  // every FP64 shot on the engines (batch_eligible leaves mixed handles per shot)
-  for (Shot& s : h->shots) {
+  // each shot of a handle without the FP32 convolution kernels takes the engines or the line kernels by itself
+  std::vector<int> eng, line, all;
+  for (int i = 0; i < S; ++i) {
     bool ok = false;
-    if (B.stream) LOSS_TRY(acs_ok(h, s, &ok));
-    B.stream = B.stream && ok;
+    if (!B.conv) LOSS_TRY(acs_ok(h, h->shots[i], &ok));
+    if (!B.conv) (ok ? eng : line).push_back(i);
+    all.push_back(i);
   }
+  B.nengine = (int)eng.size();
+  B.nline = (int)line.size();
   // per-shot preparation: receiver corrections, staggered start (that of the per-shot schedule of the same
   // kernels), source amplitudes
-  for (Shot& s : h->shots) {
+  for (int i = 0; i < S; ++i) {
+    Shot& s = h->shots[i];
     LOSS_TRY(ensure_rdelta(h, s));
     if (!s.staggered) {
-      if (B.conv || B.stream) {
+      if (B.conv || std::count(eng.begin(), eng.end(), i)) {
         LOSS_TRY((acoustic2d_start<T, K>(h, s)));
       } else {
         LOSS_TRY((ac_x<T, K>(h, s, 0, 0.5 * s.d.dt, 0.0)));
@@ -1292,9 +1283,9 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   }
   // launch shapes and descriptors
   std::vector<LineGeom> gx, gz;
-  if (!B.conv && !B.stream) {
-    LOSS_TRY(batch_geoms(h, 2, LOSS_KERNEL_ACOUSTIC_X, 3, 4, gx, &B.xlogc, &B.xthreads, &B.xsmem));
-    LOSS_TRY(batch_geoms(h, 0, LOSS_KERNEL_ACOUSTIC_Z, 2, 0, gz, &B.zlogc, &B.zthreads, &B.zsmem));
+  if (B.nline) {
+    LOSS_TRY(batch_geoms(h, line, 2, LOSS_KERNEL_ACOUSTIC_X, 3, 4, gx, &B.xlogc, &B.xthreads, &B.xsmem));
+    LOSS_TRY(batch_geoms(h, line, 0, LOSS_KERNEL_ACOUSTIC_Z, 2, 0, gz, &B.zlogc, &B.zthreads, &B.zsmem));
   }
   if (B.clk_cap < S) {
     if (B.clk) dev_free(h, B.clk);
@@ -1304,22 +1295,24 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
     B.clk_cap = S;
     B.clk_host.clear();
   }
-  std::vector<AcXArgs<T>> xa(S);
-  std::vector<AcZArgs<T>> za(S);
-  std::vector<int> t0(2 * (S + 1), 0);
+  const int NL = B.nline;
+  std::vector<AcXArgs<T>> xa(NL);
+  std::vector<AcZArgs<T>> za(NL);
+  std::vector<int> t0(2 * (NL + 1), 0);
+  for (int q = 0; q < NL; ++q) {
+    Shot& s = h->shots[line[q]];
+    xa[q] = ac_x_args<T>(h, s, gx[q], 1, s.d.dt, 0.0);
+    xa[q].src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
+    xa[q].src.amp_tab = s.amp_tab;
+    xa[q].src.clk = B.clk + line[q];
+    za[q] = ac_z_args<T>(h, s, gz[q], s.d.dt, 1);
+    t0[q + 1] = t0[q] + gx[q].nbundles;
+    t0[NL + 1 + q + 1] = t0[NL + 1 + q] + gz[q].nbundles;
+  }
   std::vector<GatherJob<T>> pre, post;
   int64_t pre_max = 0, post_max = 0;
   for (int i = 0; i < S; ++i) {
     Shot& s = h->shots[i];
-    if (!B.conv && !B.stream) {
-      xa[i] = ac_x_args<T>(h, s, gx[i], 1, s.d.dt, 0.0);
-      xa[i].src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
-      xa[i].src.amp_tab = s.amp_tab;
-      xa[i].src.clk = B.clk + i;
-      za[i] = ac_z_args<T>(h, s, gz[i], s.d.dt, 1);
-      t0[i + 1] = t0[i] + gx[i].nbundles;
-      t0[S + 1 + i + 1] = t0[S + 1 + i] + gz[i].nbundles;
-    }
     for (int f = 0; f < LOSS_NUM_FIELDS; ++f) {
       if (s.n_rcv == 0) break;
       const int64_t off = s.rcv_offsets[f], cnt = s.rcv_offsets[f + 1] - off;
@@ -1346,8 +1339,8 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
       post_max = std::max(post_max, cnt);
     }
   }
-  B.xtiles = t0[S];
-  B.ztiles = t0[2 * S + 1];
+  B.xtiles = t0[NL];
+  B.ztiles = t0[2 * NL + 1];
   B.npre = (int)pre.size();
   B.npost = (int)post.size();
   B.pre_max = pre_max;
@@ -1356,10 +1349,10 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   jobs.insert(jobs.end(), post.begin(), post.end());
   if (B.conv) {
     if constexpr (sizeof(T) == 4) LOSS_TRY(conv_tables<K>(h));
-    if (B.rows) LOSS_TRY((acs_tables<T, K>(h)));
-  } else if (B.stream) {
-    LOSS_TRY((acs_tables<T, K>(h)));
-  } else {
+    if (B.rows) LOSS_TRY((acs_tables<T, K>(h, all)));
+  }
+  if (B.nengine) LOSS_TRY((acs_tables<T, K>(h, eng)));
+  if (B.nline) {
     LOSS_TRY(upload_table(h, 0, as_bytes(xa), &B.xtab));
     LOSS_TRY(upload_table(h, 1, as_bytes(za), &B.ztab));
     void* t0p = B.tile0;
@@ -1377,7 +1370,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
                         "upload clocks"));
     LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
   }
-  if (!B.conv && !B.stream) {
+  if (B.nline) {
     LOSS_TRY(cuda_check(h, batch_grid_ac_x<T, K>(B.xlogc, B.xthreads, B.xsmem, B.xtiles, h->num_sms, &B.xgrid),
                         "batched x kernel shape"));
     LOSS_TRY(cuda_check(h, batch_grid_ac_z<T, K>(B.zlogc, B.zthreads, B.zsmem, B.ztiles, h->num_sms, &B.zgrid),
@@ -1396,7 +1389,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
                                       B.xl.total, B.tzthreads[0], B.tzthreads[1], B.tzlogc[0], B.tzlogc[1],
                                       B.tztiles, B.tzgrid[0], B.tzgrid[1],
                                       (int64_t)B.tzsmem[0], (int64_t)B.tzsmem[1], (int64_t)h->wait_polls,
-                                      B.stream ? 1 : 0, B.rows ? 1 : 0, (int64_t)(intptr_t)B.astab, B.astab_version};
+                                      B.nengine, B.nline, B.rows ? 1 : 0, (int64_t)(intptr_t)B.astab, B.astab_version};
     if (!B.gexec || sig != B.gsig) {
       LOSS_TRY((capture_graph<T, K>(h, k)));
       B.gsig = sig;
