@@ -257,7 +257,8 @@ loss_status_t loss_set_tile(loss_handle_t handle, int32_t kernel, int32_t thread
  * instead).  batched != 0 (the default): a handle whose shots are all 2-D acoustic grids of one precision advances
  * them together, each step being one persistent launch per kernel over the work of all shots, one launch per
  * receiver phase and a clock tick.  The kernels are those of the per-shot step: with the truncated-convolution
- * family (FP32, when every shot qualifies) the x kernel over rows of all shots, then Z1 and Z2 over the z
+ * family (FP32, when every shot qualifies) one x kernel over the short rows of all shots and two launches (stress, then
+ * velocity sub-step) over the long ones, then Z1 and Z2 over the z
  * tiles of all shots; FP64 shots by themselves, those that qualify for the column and row kernels on these and the others
  * on the line kernels; otherwise the line kernels, x and z over bundles of whole lines.  The source amplitude and
  * the trace row of each step are read from per-shot device counters, so the launches of every step are
@@ -349,7 +350,8 @@ loss_status_t loss_set_coordinates(loss_handle_t handle, int32_t shot, int32_t a
  * limit) for its own copies in flight and stops, so the CUDA context stays usable, and the next loss_sync returns
  * LOSS_E_TIMEOUT and poisons the handle.  polls < 0 restores the default (2^24 polls, far beyond any copy's
  * latency); polls = 0 makes every such wait give up without polling, which is how the failure path is tested.
- * Kernels without waits are taken where they are faster; a handle whose limit is not the default keeps those that wait.
+ * Rows that a kernel without waits takes have none to bound (513 points and more, loss_set_kernels); with polls = 0 they
+ * go to the kernel that waits too.  Any other limit changes no result.
  * This is a library control with no counterpart in the paper.  Takes effect from the next loss_step (a captured
  * graph is recaptured).  Returns LOSS_E_ARG for a NULL handle. */
 loss_status_t loss_set_wait_limit(loss_handle_t handle, int64_t polls);

@@ -684,6 +684,7 @@ loss_status_t loss_autotune(loss_handle_t h, int32_t steps, loss_tune_entry_t* o
   }
   t->batched = h->batched;
   t->tiled = h->tiled;
+  t->wait_polls = h->wait_polls;
   t->graph_steps = 0;  // plain launches, so that every kernel can be timed
   for (int k = 0; k < LOSS_NUM_KERNELS; ++k) {
     t->tile_threads[k] = h->tile_threads[k];

@@ -140,11 +140,11 @@ struct BatchState {
   bool conv = false;
   void* xptab = nullptr;  // XpShot[n_shots]
   void* tztab = nullptr;  // TzShot[2 n_shots]
-  // shots on the barrier-free engines (FP64; job and block tables of the launches of a step) and on the line kernels
-  int nengine = 0, nline = 0;
+  // shots on the barrier-free engines (job and block tables of the launches of a step; with conv: their rows), on the
+  // line kernels, and with conv on the pipelined x kernel
+  int nengine = 0, nline = 0, npipe = 0;
   void* astab = nullptr;
   AcBatchKind ask[8];
-  bool rows = false;  // with conv: the x part runs on the row engine
   int64_t astab_version = 0;
   XpSmem xl{};
   int xpthreads = 0, xpgrid = 0, tztiles = 0;

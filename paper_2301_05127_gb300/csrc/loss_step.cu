@@ -270,23 +270,17 @@ static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
   return cuda_check(h, launch_ac_cols<T, K>(a, g, col_map(h->num_sms, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
 }
 
-// Whether the FP32 rows of this handle that the pipelined kernel would take run on the row engine: all of its shots have
-// rows of at least 513 points that qualify (a batch has one x kernel, and every shot's results are those of its own
-// schedule), outside gradients, with the default limit of the pipelined kernel's waits (a limit of the caller's own is
-// a request for them).  x part, engine against pipelined kernel: 513^2 19.9 / 21.7 us, 1025^2 28.9 / 33.8 us, 2049^2
-// 51.4 / 62.4 us, with Kahan summation 61.4 / 67.0 us; rows of 257 points and less are bound by launches either way.
-static loss_status_t rows_on_engine(loss_ctx* h, bool* on) {
+// Whether the FP32 rows of this shot that the pipelined kernel would take run on the row engine: rows of at least 513
+// points that qualify, in the convolution family, outside gradients.  Other shots of the handle and the length of the
+// pipelined kernel's waits have no part in it; only a limit of 0 polls, which fails the run, keeps the kernel that
+// waits.  x part, engine against pipelined kernel: 513^2 19.9 / 21.7 us, 1025^2 28.9 / 33.8 us, 2049^2 51.4 / 62.4 us, with
+// Kahan summation 61.4 / 67.0 us; rows of 257 points and less are bound by launches either way.
+static loss_status_t rows_on_engine(loss_ctx* h, Shot& s, bool* on) {
   *on = false;
-  if (h->tiled == LOSS_KERNELS_CONVOLUTION_ITEMS || h->in_gradient || h->wait_polls != kDefaultWaitPolls) return LOSS_OK;
-  for (Shot& s : h->shots) {
-    if (s.n[2] < 512 || any_nonuniform(s) || !tiled_ok(h, s) || !conv_size_ok(s)) return LOSS_OK;
-    ConvAxis g;
-    bool ok;
-    LOSS_TRY(conv_axis(h, s, 2, &g, &ok));
-    if (!ok) return LOSS_OK;
-  }
-  *on = true;
-  return LOSS_OK;
+  if (h->tiled == LOSS_KERNELS_CONVOLUTION_ITEMS || h->in_gradient || h->wait_polls == 0) return LOSS_OK;
+  if (s.n[2] < 512 || any_nonuniform(s) || !tiled_ok(h, s) || !conv_size_ok(s)) return LOSS_OK;
+  ConvAxis g;
+  return conv_axis(h, s, 2, &g, on);
 }
 
 // x part of the FP32 step (sub-step B and the x part of A, or the latter alone): the pipelined row kernel when a
@@ -300,7 +294,7 @@ static loss_status_t xpart(loss_ctx* h, Shot& s, int do_B, double acoef, double 
   t.Wd = s.Wd[2];
   t.ncross = (int)s.len[0];
   bool rows;
-  LOSS_TRY(rows_on_engine(h, &rows));
+  LOSS_TRY(rows_on_engine(h, s, &rows));
   if (rows && xp_ok(h, s, t)) return acs_rows<float, K>(h, s, do_B, acoef, amp);
   if (!xp_ok(h, s, t) && h->tiled != LOSS_KERNELS_CONVOLUTION_ITEMS && !h->in_gradient && conv_size_ok(s) &&
       xt_smem(t) <= (size_t)h->smem_optin) {
@@ -990,18 +984,22 @@ static loss_status_t batch_launch_step(loss_ctx* h) {
     LaunchScope ls(h, LOSS_KERNEL_GATHER);
     LOSS_TRY(cuda_check(h, launch_gather_batch<T>(jobs, B.npre, B.pre_max, h->stream), "batched receiver gather"));
   }
+  auto engine = [&](int k0, int k1) -> loss_status_t {
+    for (int k = k0; k < k1; ++k) {
+      if (B.ask[k].blocks == 0) continue;
+      LaunchScope ls(h, k < 5 ? LOSS_KERNEL_ACOUSTIC_X : (k < 7 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2));
+      LOSS_TRY(cuda_check(h, launch_ac_batch<T, K>(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
+    }
+    return LOSS_OK;
+  };
   if constexpr (sizeof(T) == 4) {
     if (B.conv) {
       const int* unit0 = B.tile0;
-      const int* bunit = unit0 + S + 1;
+      const int* bunit = unit0 + B.npipe + 1;
       const int* bshot = bunit + B.xpgrid + 1;
       const int* zt0 = bshot + B.xpgrid;
-      for (int k = 0; B.rows && k < 5; ++k) {
-        if (B.ask[k].blocks == 0) continue;
-        LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
-        LOSS_TRY(cuda_check(h, launch_ac_batch<T, K>(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
-      }
-      if (!B.rows) {
+      if (B.nengine) LOSS_TRY(engine(0, 5));
+      if (B.npipe) {
         LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
         LOSS_TRY(cuda_check(h, launch_xp_batch<K>((const XpShot*)B.xptab, unit0, bunit, bshot, B.xl, B.xpthreads,
                                                   B.xpgrid, h->dflag, h->wait_polls, h->stream),
@@ -1024,14 +1022,6 @@ static loss_status_t batch_launch_step(loss_ctx* h) {
     }
   }
   // shots on the engines and shots on the line kernels, x then z (a shot has its launches from one of the two)
-  auto engine = [&](int k0, int k1) -> loss_status_t {
-    for (int k = k0; k < k1; ++k) {
-      if (B.ask[k].blocks == 0) continue;
-      LaunchScope ls(h, k < 5 ? LOSS_KERNEL_ACOUSTIC_X : (k < 7 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2));
-      LOSS_TRY(cuda_check(h, launch_ac_batch<T, K>(B.astab, B.ask[k], k, h->stream), "batched acoustic kernel"));
-    }
-    return LOSS_OK;
-  };
   if (B.nengine) LOSS_TRY(engine(0, 5));
   if (B.nline) {
     LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
@@ -1120,28 +1110,28 @@ static bool conv_batch_ok(const loss_ctx* h) {
 }
 
 // Descriptors, work ranges and launch shapes of the batched convolution kernels (the shots are staggered and their
-// amplitude tables exist).  The x blocks take whole units of rows in about equal numbers of points.
+// amplitude tables exist).  pipe: the shots whose rows the pipelined x kernel takes; its blocks take whole units of rows
+// in about equal numbers of points.
 template <bool K>
-static loss_status_t conv_tables(loss_ctx* h) {
+static loss_status_t conv_tables(loss_ctx* h, const std::vector<int>& pipe) {
   BatchState& B = h->batch;
-  const int S = (int)h->shots.size();
-  std::vector<XpShot> xs(S);
+  const int S = (int)h->shots.size(), SP = (int)pipe.size();
+  std::vector<XpShot> xs(SP);
   std::vector<TzShot> zs(2 * S);
-  std::vector<TileGeom> txs(S);
-  std::vector<int> unit0(S + 1, 0), zt0(S + 1, 0), rs(S);
+  std::vector<TileGeom> txs(SP);
+  std::vector<int> unit0(SP + 1, 0), zt0(S + 1, 0), rs(SP);
   int xthreads = 32, zthreads[2] = {32, 32};
   const int zlc[2] = {zchunk_log2(h, 1), zchunk_log2(h, 2)};
   size_t zsm[2] = {0, 0};
   int64_t ptot = 0;
-  for (int i = 0; i < S; ++i) {
+  for (int i : pipe) {
     int thr;
     tile_geom(h->shots[i], 2, &thr);
     xthreads = std::max(xthreads, thr);
   }
   while (xthreads & (xthreads - 1)) xthreads += 32;  // a power of two of warps, so that short rows form groups
-  for (int i = 0; i < S; ++i) {
-    Shot& s = h->shots[i];
-    LOSS_TRY(ensure_delta_weights(h, s, 0));
+  for (int i = 0; i < SP; ++i) {
+    Shot& s = h->shots[pipe[i]];
     LOSS_TRY(ensure_delta_weights(h, s, 2));
     int thr;
     TileGeom tx = tile_geom(s, 2, &thr);
@@ -1150,7 +1140,7 @@ static loss_status_t conv_tables(loss_ctx* h) {
     x.a = ac_x_args<float>(h, s, LineGeom{}, 1, s.d.dt, 0.0);
     x.a.src.on = (s.src_on && (s.src_kinds & LOSS_SRC_PRESSURE)) ? 1 : 0;
     x.a.src.amp_tab = s.amp_tab;
-    x.a.src.clk = B.clk + i;
+    x.a.src.clk = B.clk + pipe[i];
     x.t = tx;
     x.mmagic = (unsigned)((((uint64_t)1 << 32) + (uint64_t)tx.M - 1) / (uint64_t)tx.M);
     rs[i] = xp_rows_per_unit(tx.n, xthreads);
@@ -1160,6 +1150,11 @@ static loss_status_t conv_tables(loss_ctx* h) {
     unit0[i + 1] = unit0[i] + (tx.ncross + rs[i] - 1) / rs[i];
     ptot += (int64_t)(tx.n + 1) * tx.ncross;
     txs[i] = tx;
+  }
+  for (int i = 0; i < S; ++i) {
+    Shot& s = h->shots[i];
+    LOSS_TRY(ensure_delta_weights(h, s, 0));
+    int thr;
     for (int m = 0; m < 2; ++m) {
       const TileGeom tz = tile_geom(s, 0, &thr, zlc[m]);
       zs[m * S + i] = TzShot{ac_z_args<float>(h, s, LineGeom{}, m == 0 ? s.d.dt : 0.0, 0), tz, thr >> 5, 0};
@@ -1168,21 +1163,25 @@ static loss_status_t conv_tables(loss_ctx* h) {
       if (m == 0) zt0[i + 1] = zt0[i] + tz.ntl * tz.p;
     }
   }
-  B.xl = xp_batch_layout(txs, rs, K);
+  int per = 0, G = 0;
+  B.npipe = SP;
+  B.xl = XpSmem{};
   B.xpthreads = xthreads;
-  int per = 0;
-  LOSS_TRY(cuda_check(h, xp_batch_per_sm<K>(B.xl, xthreads, &per), "batched x kernel shape"));
-  if (per < 1) {
-    h->err = "batched x kernel does not fit an SM";
-    return LOSS_E_UNSUPPORTED;
+  if (SP) {
+    B.xl = xp_batch_layout(txs, rs, K);
+    LOSS_TRY(cuda_check(h, xp_batch_per_sm<K>(B.xl, xthreads, &per), "batched x kernel shape"));
+    if (per < 1) {
+      h->err = "batched x kernel does not fit an SM";
+      return LOSS_E_UNSUPPORTED;
+    }
+    G = (int)std::min<int64_t>(unit0[SP], (int64_t)per * h->num_sms);
   }
-  const int G = (int)std::min<int64_t>(unit0[S], (int64_t)per * h->num_sms);
   // block b starts at the first unit whose preceding points reach b * ptot / G
-  std::vector<int> brow(G + 1, unit0[S]), bshot(G, S - 1);
+  std::vector<int> brow(G + 1, unit0[SP]), bshot(G, SP - 1);
   {
     int b = 0, u = 0;
     int64_t before = 0;
-    for (int i = 0; i < S && b < G; ++i)
+    for (int i = 0; i < SP && b < G; ++i)
       for (int w = 0; w < unit0[i + 1] - unit0[i] && b < G; ++w, ++u) {
         while (b < G && before >= (ptot * b + G - 1) / G) {
           brow[b] = u;
@@ -1253,15 +1252,14 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   const int S = (int)h->shots.size();
   B.conv = false;
   if constexpr (sizeof(T) == 4) B.conv = conv_batch_ok(h);
-  B.rows = false;
-  if (B.conv) LOSS_TRY(rows_on_engine(h, &B.rows));
-  // each shot of a handle without the FP32 convolution kernels takes the engines or the line kernels by itself
-  std::vector<int> eng, line, all;
+  // each shot by itself takes the engines (with the FP32 convolution kernels: its rows) or the pipelined x kernel, else
+  // the line kernels
+  std::vector<int> eng, pipe, line;
   for (int i = 0; i < S; ++i) {
     bool ok = false;
-    if (!B.conv) LOSS_TRY(acs_ok(h, h->shots[i], &ok));
-    if (!B.conv) (ok ? eng : line).push_back(i);
-    all.push_back(i);
+    if (B.conv) LOSS_TRY(rows_on_engine(h, h->shots[i], &ok));
+    else LOSS_TRY(acs_ok(h, h->shots[i], &ok));
+    (ok ? eng : (B.conv ? pipe : line)).push_back(i);
   }
   B.nengine = (int)eng.size();
   B.nline = (int)line.size();
@@ -1348,8 +1346,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
   std::vector<GatherJob<T>> jobs = pre;
   jobs.insert(jobs.end(), post.begin(), post.end());
   if (B.conv) {
-    if constexpr (sizeof(T) == 4) LOSS_TRY(conv_tables<K>(h));
-    if (B.rows) LOSS_TRY((acs_tables<T, K>(h, all)));
+    if constexpr (sizeof(T) == 4) LOSS_TRY(conv_tables<K>(h, pipe));
   }
   if (B.nengine) LOSS_TRY((acs_tables<T, K>(h, eng)));
   if (B.nline) {
@@ -1389,7 +1386,7 @@ static loss_status_t step_batched_t(loss_ctx* h, int64_t n) {
                                       B.xl.total, B.tzthreads[0], B.tzthreads[1], B.tzlogc[0], B.tzlogc[1],
                                       B.tztiles, B.tzgrid[0], B.tzgrid[1],
                                       (int64_t)B.tzsmem[0], (int64_t)B.tzsmem[1], (int64_t)h->wait_polls,
-                                      B.nengine, B.nline, B.rows ? 1 : 0, (int64_t)(intptr_t)B.astab, B.astab_version};
+                                      B.nengine, B.nline, B.npipe, (int64_t)(intptr_t)B.astab, B.astab_version};
     if (!B.gexec || sig != B.gsig) {
       LOSS_TRY((capture_graph<T, K>(h, k)));
       B.gsig = sig;

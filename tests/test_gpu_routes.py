@@ -79,3 +79,22 @@ def test_mixed_fp64_handle_stays_batched(pkg, graph):
         for k, f in enumerate(FIELDS):
             err = np.linalg.norm(got[s][k] - sim.state[f]) / np.linalg.norm(sim.state[f])
             assert err < 1e-12, (s, f, err)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_kahan"])
+def test_long_rows_do_not_depend_on_other_shots(pkg, prec):
+    """FP32: a shot with long rows has the same bits alone and beside shots with short rows, in both schedules and with
+    graphs, whatever the (non-zero) limit of the bounded waits; the batched step has a launch for each kind of rows."""
+    long_, short = ((64, 512), (2, 4), 20), ((96, 256), (3, 2), 12)
+    ws = [_shot(*g, prec, 50 + k) for k, g in enumerate([long_, short, ((96, 1024), (3, 8), 12)])]
+    alone, _ = _run(pkg, ws[:1], batched=False)
+    ref, _ = _run(pkg, ws, batched=False)
+    assert _same(ref[0], alone[0])
+    for graph, wait in ((0, None), (3, None), (0, 1 << 20)):
+        got, counts = _run(pkg, ws, graph=graph, wait=wait)
+        assert all(_same(a, b) for a, b in zip(got, ref)), (graph, wait)
+        assert counts["acoustic_x"] == 21  # sub-steps B and A of the long rows, the pipelined kernel for the others
+    other, _ = _run(pkg, ws[:1], batched=False, wait=1 << 20)
+    assert _same(other[0], alone[0])
+    pair, _ = _run(pkg, ws[1:2], batched=False, seeds=[1])
+    assert _same(pair[0], ref[1])
