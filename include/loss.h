@@ -205,6 +205,10 @@ loss_status_t loss_derivative_adjoint(loss_handle_t handle, int32_t shot, int32_
  * acoustic grids), g_rho: dense arrays of the grid shape, doubles, written.  mem says where d_obs and the
  * gradients live.  The gradient is dJ/d(model) with the time step, the absorbing profile (whose damping uses
  * the largest vp) and the source fixed.  Afterwards the shot is at step n_steps with its traces recorded.
+ * The forward run is that of loss_step bit for bit, so that traces recorded by loss_step at the same model give
+ * J = 0 and zero gradients, in FP64 and in the families LOSS_KERNELS_LINE and LOSS_KERNELS_CONVOLUTION_ITEMS; in FP32 on
+ * LOSS_KERNELS_CONVOLUTION it keeps the tile and pipelined-row kernels where loss_step takes the column and row kernels
+ * (loss_set_kernels), and the traces of the two agree to FP32 rounding.
  * Built for 2-D acoustic and 3-D elastic grids with stress-type sources; LOSS_E_UNSUPPORTED for a body force,
  * LOSS_E_STATE without a model or receivers, LOSS_E_ARG for bad arguments. */
 loss_status_t loss_gradient(loss_handle_t handle, int32_t shot, const double* d_obs, int32_t checkpoint_every,
@@ -276,10 +280,11 @@ loss_status_t loss_set_schedule(loss_handle_t handle, int32_t batched, int32_t g
  * corrections from the PMBC junction values (x rows pipelined through TMA bulk copies, z lines on independent
  * 32-column x one-patch tiles; rows the pipelined kernel does not take, longer than 2049 points or with patches
  * whose length is not a multiple of 8, go to independent (row, patch) items in two launches);
- * LOSS_KERNELS_CONVOLUTION_ITEMS = the same with every row on (row, patch) items.  In the convolution family FP64 2-D
- * steps, 3-D elastic steps, FP32 rows of 513 points and more and rows that the pipelined kernel does not take run on
- * kernels that march lines and rows without block barriers, where patches are long enough for them (at least 8 points
- * more than a junction's correction reaches, 40 points per axis) and arrays hold at most 4 GB.  All agree with the FP64 oracle
+ * LOSS_KERNELS_CONVOLUTION_ITEMS = the same with every row on (row, patch) items.  In the convolution family FP32 3-D
+ * elastic steps, FP32 rows of 513 points and more and rows that the pipelined kernel does not take, and in both families
+ * FP64 2-D and 3-D elastic steps, run on column and row kernels that march lines and rows without block barriers, where
+ * patches are long enough for them (at least 8 points more than a junction's correction reaches, 40 points per axis)
+ * and arrays hold at most 4 GB.  All agree with the FP64 oracle
  * at the FP32 tolerance; they differ in rounding.  LOSS_E_ARG for another value. */
 enum { LOSS_KERNELS_LINE = 0, LOSS_KERNELS_CONVOLUTION = 1, LOSS_KERNELS_CONVOLUTION_ITEMS = 2 };
 loss_status_t loss_set_kernels(loss_handle_t handle, int32_t family);

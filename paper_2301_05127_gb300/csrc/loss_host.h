@@ -189,8 +189,9 @@ struct loss_ctx {
   size_t stage_bytes = 0;
   int graph_steps = 0;   // > 0: steps are replayed from a captured CUDA graph of this many steps
   bool capturing = false;
-  // forward runs of loss_gradient: FP32 steps keep the tile, row and line kernels.  The gradient is an FP64 result, and
-  // these kernels' rounding is part of the gradients users compare and store.
+  // forward runs of loss_gradient: FP32 steps of the convolution family keep the tile, pipelined-row and line kernels.
+  // The gradient is returned in FP64 and does not move by the rounding (1e-7) that another forward kernel would bring;
+  // in the other families, and in FP64, it changes no kernel.
   bool in_gradient = false;
   lossk::BatchState batch;
   // launch accounting (loss_profile / loss_profile_read)

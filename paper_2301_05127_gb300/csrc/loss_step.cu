@@ -711,12 +711,14 @@ template loss_status_t deriv_stream<float>(loss_ctx*, const Shot&, int, const Co
 template loss_status_t deriv_stream<double>(loss_ctx*, const Shot&, int, const ConvAxis&, int, const double*, double*,
                                             double*);
 
-// The elastic step on those engines: the convolution family (loss_set_kernels) when every axis qualifies.  The line
-// kernels' limit on the length of a row stays the limit of the step.
+// The elastic step on those engines: the convolution family (loss_set_kernels) when every axis qualifies; in FP32 neither
+// the gradient's forward runs nor the items family, which keeps the kernels that both loss_step and loss_gradient take.
+// The line kernels' limit on the length of a row stays the limit of the step.
 template <typename T>
 static loss_status_t els_ok(loss_ctx* h, Shot& s, bool* ok) {
   *ok = false;
-  if (!h->tiled || s.dim != 3 || (s.esize == 4 && h->in_gradient)) return LOSS_OK;
+  if (!h->tiled || s.dim != 3) return LOSS_OK;
+  if (s.esize == 4 && (h->in_gradient || h->tiled == LOSS_KERNELS_CONVOLUTION_ITEMS)) return LOSS_OK;
   if ((uint64_t)s.total * s.esize > UINT32_MAX) return LOSS_OK;  // the engines use 32-bit byte offsets
   for (int k = 0; k < 3; ++k) {
     ConvAxis g;
