@@ -604,12 +604,6 @@ std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
   std::vector<double> wd((size_t)(p + 1) * wr, 0.0);
   for (int j = 0; j <= p; ++j)
     for (int t = js[j]; t < js[j + 1]; ++t) wd[(size_t)j * wr + c->R + taps[t].m] = taps[t].w;
-  if (f32)
-    for (ConvTap& t : taps) {
-      const double w = t.w;
-      t.hi = (float)w;
-      t.lo = (float)(w - (double)t.hi);
-    }
   double pw[64];
   pw[0] = 1.0;
   for (int i = 1; i < 64; ++i) pw[i] = pw[i - 1] * kConvRHost;

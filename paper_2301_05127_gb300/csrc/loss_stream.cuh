@@ -69,37 +69,9 @@ __device__ __forceinline__ T& at_off(T* p, uint32_t o) {
   return *reinterpret_cast<T*>(reinterpret_cast<C*>(p) + o);
 }
 
-// Sum of weight x sample over the taps of a junction, to the precision of T's FP64 sum rounded to T: in FP64, or for FP32
-// samples in two floats (error-free products and additions, about 46 bits).  The GPU's FP64 pipe takes 16 cycles of an SM
-// per warp instruction, however few lanes are active; eleven FP32 instructions take about three.  With that, and several
-// lanes of a row warp on one junction (one lane each had 5 of 32 at work on a row of four patches): derivative of
-// 257^3 FP32 along x 82 us -> 60 us, FP64 acoustic rows of 1025^2 102 us -> 94 us, elastic x part of 257^3 457 us -> 432 us.
-template <typename T>
-struct TapSum {
-  double s = 0.0;
-  __device__ __forceinline__ void add(const ConvTap& t, double v) { s = fma(t.w, v, s); }
-  __device__ __forceinline__ void merge(int o) { s += __shfl_xor_sync(0xffffffffu, s, o); }
-  __device__ __forceinline__ double get() const { return s; }
-};
-template <>
-struct TapSum<float> {
-  float s = 0.0f, c = 0.0f;
-  __device__ __forceinline__ void plus(float p, float e) {  // s + c += p + e
-    const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
-    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)), e));
-    s = t;
-  }
-  __device__ __forceinline__ void add(const ConvTap& t, float v) {
-    const float p = __fmul_rn(t.hi, v);
-    plus(p, __fmaf_rn(t.lo, v, __fmaf_rn(t.hi, v, -p)));
-  }
-  __device__ __forceinline__ void merge(int o) {
-    const float p = __shfl_xor_sync(0xffffffffu, s, o), e = __shfl_xor_sync(0xffffffffu, c, o);
-    plus(p, e);
-  }
-  __device__ __forceinline__ float get() const { return __fadd_rn(s, c); }
-};
-
+// The sums of weight x sample over the taps of a junction are FP64, whatever T: the GPU's FP64 pipe takes 16 cycles of an
+// SM per warp instruction, however few lanes are active, so several lanes of a row warp share one junction (one lane each
+// had 5 of 32 at work on a row of four patches) and FP32 samples are widened on the integer units.
 // Junction corrections D[f] of junction j of NF lines with their samples at byte offset o + (jM + m) * sb of src[f]; taps:
 // the axis's taps (a shared-memory copy or g.taps); four taps' samples in flight at a time.
 template <typename T, int NF>
@@ -107,7 +79,9 @@ __device__ __forceinline__ void conv_junction(const ConvAxis& g, const ConvTap* 
                                               uint32_t o, uint32_t sb, T (&D)[NF]) {
   int t = __ldg(g.js + j);
   const int t1 = __ldg(g.js + j + 1);
-  TapSum<T> s[NF];
+  double s[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) s[f] = 0.0;
   for (; t < t1; t += 4) {
     ConvTap w[4];
     T v[4][NF];
@@ -122,10 +96,10 @@ __device__ __forceinline__ void conv_junction(const ConvAxis& g, const ConvTap* 
     for (int k = 0; k < 4; ++k)
       if (t + k < t1)
 #pragma unroll
-        for (int f = 0; f < NF; ++f) s[f].add(w[k], v[k][f]);
+        for (int f = 0; f < NF; ++f) s[f] = fma(w[k].w, to_f64(v[k][f]), s[f]);
   }
 #pragma unroll
-  for (int f = 0; f < NF; ++f) D[f] = (T)s[f].get();
+  for (int f = 0; f < NF; ++f) D[f] = (T)s[f];
 }
 // The same for one line at f by G lanes (a power of two; sub: the lane's number among them); called by the whole warp.
 template <typename T>
@@ -133,16 +107,16 @@ __device__ __forceinline__ T conv_junction_part(const ConvAxis& g, const ConvTap
                                                 int G) {
   const int t1 = __ldg(g.js + j + 1);
   const T* fj = f + j * g.M;
-  TapSum<T> s;
+  double s = 0.0;
   for (int t = __ldg(g.js + j) + sub; t < t1; t += 2 * G) {
     const ConvTap w0 = taps[t], w1 = taps[min(t + G, t1 - 1)];
     const T v0 = fj[w0.m], v1 = fj[w1.m];
-    s.add(w0, v0);
-    if (t + G < t1) s.add(w1, v1);
+    s = fma(w0.w, to_f64(v0), s);
+    if (t + G < t1) s = fma(w1.w, to_f64(v1), s);
   }
   __syncwarp();
-  for (int o = 1; o < G; o <<= 1) s.merge(o);
-  return (T)s.get();
+  for (int o = 1; o < G; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return (T)s;
 }
 // a / b for 0 <= a < 2^21, b > 0 (a quotient is 1 / (2 b) or more from the next integer, its error below 2^-22 of it)
 __device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
@@ -726,7 +700,7 @@ __device__ __forceinline__ void row_block(const ConvAxis& g, const RowMap& rm, c
 #pragma unroll
           for (int s = 1; s < NF; ++s) off += f == s ? op.src(s) - s0 : (int64_t)0;
           const T D = conv_junction_part<T>(g, taps, j0 + j, s0 + off, lane & ((1 << lg) - 1), 1 << lg);
-          if (i < tasks) dsm[i] = D;
+          if (i < tasks && (lane & ((1 << lg) - 1)) == 0) dsm[i] = D;
         }
         __syncwarp();
       }

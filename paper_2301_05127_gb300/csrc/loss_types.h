@@ -288,16 +288,10 @@ struct ElTile {
   int nx;           // x columns
 };
 // Axis of the barrier-free engines (loss_stream.cuh): n intervals in p patches of M; the taps of junction j are
-// taps[js[j]] .. taps[js[j + 1] - 1] (weights over a, in FP32 axes as the sum hi + lo of two floats; offsets m from the
-// junction), ntaps in all; a junction's correction
+// taps[js[j]] .. taps[js[j + 1] - 1] (weights over a, offsets m from the junction), ntaps in all; a junction's correction
 // reaches Q positions; pw: r^d, d = 0 .. 63; wd: the same weights dense, [p + 1][2 R + 1] for the offsets -R .. R.
 struct ConvTap {
-  union {
-    double w;
-    struct {
-      float hi, lo;
-    };
-  };
+  double w;
   int m;
   int pad;
 };
