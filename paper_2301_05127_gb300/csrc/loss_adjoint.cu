@@ -447,11 +447,12 @@ static loss_status_t derivative_adjoint_t(loss_ctx* h, Shot& s, int k, const T* 
     if (ok && conv_operator_ok(s, k, s.conv[k])) {
       ColMap cm{};
       RowMap rm{};
-      if (k == 2) rm = row_map(h->num_sms, s, 1, ca, sy, sz, false);
+      if (k == 2) rm = row_map(h->num_sms, s, 2, ca, sy, sz, false);
       else cm = col_map(h->num_sms, s, k, sy, sz);
       LaunchScope ls(h, kid);
-      return cuda_check(h, launch_trans_stream<T>(ca, cm, rm, k == 2, false, g, out,
-                                                  (T)(fir_const(ca.M).a * 3.0 / s.h[k]), h->stream), "adjoint kernel");
+      const double sc = fir_const(ca.M).a * 3.0 / s.h[k];
+      return cuda_check(h, launch_trans_stream<T>(ca, cm, rm, k == 2, false, g, out, (T)sc, lo_part<T>(sc), h->stream),
+                        "adjoint kernel");
     }
   }
   AdjArgs<T> a{};

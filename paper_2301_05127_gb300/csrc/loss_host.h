@@ -317,13 +317,13 @@ template <bool KAHAN>
 cudaError_t launch_xt(const AcXArgs<float>& a, const TileGeom& t, cudaStream_t st);
 size_t xt_smem(const TileGeom& t);
 // loss_kernels_deriv.cu: derivative operators on the barrier-free engines (s1 = 3 a / h, s2 = 6 / (2 sqrt(3) h^2); d2 may
-// be null), and out (+)= scale * transpose
+// be null), and out (+)= (scale + scale_lo) * transpose; rm for two FP32 values per junction
 template <typename T>
 cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, const T* f, T* d1, T* d2,
                                 T s1, T s2, cudaStream_t st);
 template <typename T>
 cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, bool acc, const T* in,
-                                T* out, T scale, cudaStream_t st);
+                                T* out, T scale, T scale_lo, cudaStream_t st);
 // Whether the operators of axis slot k run on the engines, for tables of c.bytes bytes: those fit the static array of
 // loss_derivative_noalloc (which launches the same kernels), and the dense array fits the engines' 32-bit offsets.
 constexpr size_t kNoAllocScratchBytes = 64 * 1024;

@@ -61,32 +61,56 @@ struct DerivColOp {
   __device__ __forceinline__ void apply2nd(T v, uint32_t o) const { at_off(d2, o) = s2 * v; }
 };
 
+// Dbar_j as an unevaluated sum h + l (l = 0 in FP64): the sample at the junction plus the two tails, which round as the
+// recursions do; their sum and the product with the junction's weights do not.  (The line kernel's form: FP32 solves
+// joined, weighted and scaled in FP64.  The FP64 pipe would take 288 cycles for the products of a row window.)
+template <typename T>
+struct TransD {
+  T h, l;
+};
+template <typename T>
+__device__ __forceinline__ TransD<T> trans_sum(T f, T tails) {
+  if constexpr (sizeof(T) == 8) {
+    return {f + tails, T(0)};
+  } else {
+    const T h = __fadd_rn(f, tails), z = __fadd_rn(h, -f);
+    return {h, __fadd_rn(__fadd_rn(f, -__fadd_rn(h, -z)), __fadd_rn(tails, -z))};
+  }
+}
+// Weight i of the dense weights of an axis: a double, in FP32 axes a float and its rounding error.
+template <typename T>
+using TransW = std::conditional_t<sizeof(T) == 8, double, float2>;
+template <typename T>
+__device__ __forceinline__ T trans_add(T e, TransW<T> w, const TransD<T>& D) {
+  if constexpr (sizeof(T) == 8) return fma(w, D.h, e);
+  else return fmaf(w.x, D.h, e + fmaf(w.y, D.h, w.x * D.l));
+}
 // Dbar_j of the line whose samples start at byte offset o and step by sb.
 template <typename T>
-__device__ __forceinline__ T trans_junction(const ConvAxis& g, int j, const T* f, uint32_t o, uint32_t sb,
-                                            const T* rs) {
+__device__ __forceinline__ TransD<T> trans_junction(const ConvAxis& g, int j, const T* f, uint32_t o, uint32_t sb) {
+  constexpr T r = (T)kConvR;
   const int q = j * g.M;
-  T s = T(0);
+  T a = T(0), b = T(0);
 #pragma unroll 4
-  for (int d = -g.Q; d <= g.Q; ++d) {
-    const int i = q + d;
-    const T v = at_off(f, o + (uint32_t)min(max(i, 0), g.n) * sb);
-    s += (i >= 0 && i <= g.n ? v : T(0)) * rs[64 + d];
+  for (int d = g.Q; d >= 1; --d) {
+    const T va = at_off(f, o + (uint32_t)max(q - d, 0) * sb), vb = at_off(f, o + (uint32_t)min(q + d, g.n) * sb);
+    a = (q - d >= 0 ? va : T(0)) + r * a;
+    b = (q + d <= g.n ? vb : T(0)) + r * b;
   }
-  return s;
+  return trans_sum(at_off(f, o + (uint32_t)q * sb), r * (a + b));
 }
 
 // out (+)= scale * transpose along rows.  ACC: add to out.
 template <typename T, bool ACC>
 __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, const T* __restrict__ in, T* out,
-                                                      T scale) {
+                                                      T scale, T scale_lo) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ T rs[kReach];
   fill_reach(rs, g);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gw = rm.gw, rpw = 32 / gw;
-  T* dsm = reinterpret_cast<T*>(sm + (size_t)warp * rm.wbytes);
+  TransD<T>* dsm = reinterpret_cast<TransD<T>*>(sm + (size_t)warp * rm.wbytes);
   const int gl = lane & (gw - 1), k = lane / gw;
   const int items = rm.groups * rm.nwin;
   const int nw = blockDim.x >> 5;
@@ -125,15 +149,16 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
         const int i = i0 + (lane >> lg), ii = min(i, tasks - 1);
         const int kk = small_div(ii, nj), q0 = (j0 + ii - kk * nj) * g.M;
         const T* f = in + (rpw == 1 ? rb : rbase(grp * rpw + kk));
+        const int sub = lane & ((1 << lg) - 1);
         T D = T(0);
-        for (int d = (lane & ((1 << lg) - 1)) - g.Q; d <= g.Q; d += 1 << lg) {
+        for (int d = sub - g.Q; d <= g.Q; d += 1 << lg) {
           const int x = q0 + d;
           const T v = f[min(max(x, 0), g.n)];
-          D += (x >= 0 && x <= g.n ? v : T(0)) * rs[64 + d];
+          D += (x >= 0 && x <= g.n && d != 0 ? v : T(0)) * rs[64 + d];
         }
         __syncwarp();
         for (int o = 1; o < 1 << lg; o <<= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
-        if (i < tasks) dsm[i] = D;
+        if (i < tasks && sub == 0) dsm[i] = trans_sum(f[q0], D);
       }
       __syncwarp();
     }
@@ -147,18 +172,18 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
       if (nj > 0) {
         const int ja = p0 <= g.R ? 0 : (p0 - g.R + g.M - 1) / g.M, jb = min(g.p, (p0 + 8 + g.R) / g.M);
         for (int j = ja; j <= jb; ++j) {
-          const T D = dsm[k * nj + min(max(j - j0, 0), nj - 1)];
-          const double* w = g.wd + (size_t)j * (2 * g.R + 1) + g.R;
+          const TransD<T> D = dsm[k * nj + min(max(j - j0, 0), nj - 1)];
+          const TransW<T>* w = (const TransW<T>*)g.wd + (size_t)j * (2 * g.R + 1) + g.R;
 #pragma unroll
           for (int i = 0; i < 9; ++i) {
             const int m = p0 + i - j * g.M;
-            const T wi = (T)__ldg(w + min(max(m, -g.R), g.R));
-            if (m >= -g.R && m <= g.R) e[i] += wi * D;
+            const TransW<T> wi = __ldg(w + min(max(m, -g.R), g.R));
+            if (m >= -g.R && m <= g.R) e[i] = trans_add<T>(e[i], wi, D);
           }
         }
       }
 #pragma unroll
-      for (int j = 0; j < 9; ++j) e[j] *= scale;
+      for (int j = 0; j < 9; ++j) e[j] = mulc(e[j], scale, scale_lo);
       if constexpr (ACC) {
         T u[9];
         ld9(out + gi, rm.vec, len, u);
@@ -173,14 +198,11 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
 // out (+)= scale * transpose along strided lines, marched as k_col.
 template <typename T, bool ACC>
 __global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, const T* __restrict__ in, T* out,
-                                                      T scale) {
+                                                      T scale, T scale_lo) {
   constexpr int W = Conv<T>::W, NR = W + 2, NJ = 4;
   constexpr T r = (T)kConvR, r8 = (T)conv_pow(8), r16 = (T)conv_pow(16);
   constexpr T i1r = (T)(2.0 / (1.0 - kConvR)), ir = (T)(1.0 / kConvR);
   extern __shared__ __align__(16) unsigned char sm[];
-  __shared__ T rs[kReach];
-  fill_reach(rs, g);
-  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t item = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (item >= cm.groups * cm.nseg) return;
@@ -214,9 +236,9 @@ __global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, con
     for (int k = Conv<T>::K; k >= 1; --k) L = at_off(in, base + (uint32_t)max(s0 - k, 0) * sb) + r * L;
   }
   T pb[W], Rn = T(0), endv = T(0), E0 = T(0);
-  T Dj[NJ];  // Dbar of the junctions jn - NJ .. jn - 1
+  TransD<T> Dj[NJ];  // Dbar of the junctions jn - NJ .. jn - 1
 #pragma unroll
-  for (int i = 0; i < NJ; ++i) Dj[i] = T(0);
+  for (int i = 0; i < NJ; ++i) Dj[i] = {T(0), T(0)};
   int jn = s0 <= g.R ? 0 : (s0 - g.R + g.M - 1) / g.M;
   bool tailed = false;
   auto sums = [&](int c, int k) {
@@ -283,7 +305,7 @@ __global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, con
     while (g.ntaps && jn <= g.p && jn * g.M <= p0 + 7 + g.R) {
 #pragma unroll
       for (int i = 0; i + 1 < NJ; ++i) Dj[i] = Dj[i + 1];
-      Dj[NJ - 1] = trans_junction<T>(g, jn, in, base, sb, rs);
+      Dj[NJ - 1] = trans_junction<T>(g, jn, in, base, sb);
       ++jn;
     }
 #pragma unroll
@@ -291,12 +313,12 @@ __global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, con
       const int j = jn - NJ + i;
       const int o = p0 - j * g.M;
       if (g.ntaps && j >= 0 && o <= g.R && o + 7 >= -g.R) {
-        const double* w = g.wd + (size_t)j * (2 * g.R + 1) + g.R;
+        const TransW<T>* w = (const TransW<T>*)g.wd + (size_t)j * (2 * g.R + 1) + g.R;
 #pragma unroll
         for (int l = 0; l < 8; ++l) {
           const int m = o + l;
-          const T wi = (T)__ldg(w + min(max(m, -g.R), g.R));
-          if (m >= -g.R && m <= g.R) e[l] += wi * Dj[i];
+          const TransW<T> wi = __ldg(w + min(max(m, -g.R), g.R));
+          if (m >= -g.R && m <= g.R) e[l] = trans_add<T>(e[l], wi, Dj[i]);
         }
       }
     }
@@ -309,7 +331,7 @@ __global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, con
     if (valid)
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (j < len) at_off(out, base + (uint32_t)(p0 + j) * sb) = ACC ? u[j] + scale * e[j] : scale * e[j];
+        if (j < len) at_off(out, base + (uint32_t)(p0 + j) * sb) = (ACC ? u[j] : T(0)) + mulc(e[j], scale, scale_lo);
   }
   cp_async_wait<0>();
 }
@@ -345,7 +367,7 @@ cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMa
 
 template <typename T>
 cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, bool acc, const T* in,
-                                T* out, T scale, cudaStream_t st) {
+                                T* out, T scale, T scale_lo, cudaStream_t st) {
   if (x) {
     const size_t smem = (size_t)rm.warps * rm.wbytes;
     auto kern = acc ? k_row_trans<T, true> : k_row_trans<T, false>;
@@ -353,7 +375,7 @@ cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMa
       const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
       if (e != cudaSuccess) return e;
     }
-    kern<<<row_blocks(rm, 4, rm.warps), 32 * rm.warps, smem, st>>>(g, rm, in, out, scale);
+    kern<<<row_blocks(rm, 4, rm.warps), 32 * rm.warps, smem, st>>>(g, rm, in, out, scale, scale_lo);
     return cudaGetLastError();
   }
   const size_t smem = col_smem<T>(1, cm.warps);
@@ -361,7 +383,7 @@ cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMa
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)col_smem<T>(1, 4, true));
   if (e != cudaSuccess) return e;
-  kern<<<col_blocks(cm, cm.warps), 32 * cm.warps, smem, st>>>(g, cm, in, out, scale);
+  kern<<<col_blocks(cm, cm.warps), 32 * cm.warps, smem, st>>>(g, cm, in, out, scale, scale_lo);
   return cudaGetLastError();
 }
 
@@ -370,8 +392,8 @@ template cudaError_t launch_deriv_stream<float>(const ConvAxis&, const ColMap&, 
 template cudaError_t launch_deriv_stream<double>(const ConvAxis&, const ColMap&, const RowMap&, bool, const double*,
                                                  double*, double*, double, double, cudaStream_t);
 template cudaError_t launch_trans_stream<float>(const ConvAxis&, const ColMap&, const RowMap&, bool, bool, const float*,
-                                                float*, float, cudaStream_t);
+                                                float*, float, float, cudaStream_t);
 template cudaError_t launch_trans_stream<double>(const ConvAxis&, const ColMap&, const RowMap&, bool, bool,
-                                                 const double*, double*, double, cudaStream_t);
+                                                 const double*, double*, double, double, cudaStream_t);
 
 }  // namespace lossk

@@ -604,6 +604,11 @@ std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
   std::vector<double> wd((size_t)(p + 1) * wr, 0.0);
   for (int j = 0; j <= p; ++j)
     for (int t = js[j]; t < js[j + 1]; ++t) wd[(size_t)j * wr + c->R + taps[t].m] = taps[t].w;
+  if (f32)  // a float and its rounding error in the place of each
+    for (double& v : wd) {
+      const float hl[2] = {(float)v, (float)(v - (double)(float)v)};
+      std::memcpy(&v, hl, sizeof(v));
+    }
   double pw[64];
   pw[0] = 1.0;
   for (int i = 1; i < 64; ++i) pw[i] = pw[i - 1] * kConvRHost;

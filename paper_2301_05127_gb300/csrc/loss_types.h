@@ -289,7 +289,8 @@ struct ElTile {
 };
 // Axis of the barrier-free engines (loss_stream.cuh): n intervals in p patches of M; the taps of junction j are
 // taps[js[j]] .. taps[js[j + 1] - 1] (weights over a, offsets m from the junction), ntaps in all; a junction's correction
-// reaches Q positions; pw: r^d, d = 0 .. 63; wd: the same weights dense, [p + 1][2 R + 1] for the offsets -R .. R.
+// reaches Q positions; pw: r^d, d = 0 .. 63; wd: the same weights dense, [p + 1][2 R + 1] for the offsets -R .. R (FP32 axes:
+// a float and its rounding error in each).
 struct ConvTap {
   double w;
   int m;
