@@ -87,7 +87,9 @@ std::vector<double> pmbc_weights_scaled(int n, int p, int n_nb) {
 // eF_j = a sum_{k=1..K} r^{k-1} (f_{c+k} - f_{c-k}) with the line continued by odd reflection beyond its ends
 // (f_{-q} = 2 f_0 - f_q, f_{n+q} = 2 f_n - f_{n-q}, q clamped to the line).  Formed in FP64; away from the
 // physical ends the two weight sets agree to O(r^K), so the FP32 sum of D f carries no cancellation.
-std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K) {
+// mag (may be null): at each position a bound on the terms whose difference the weight is, for its rounding error: those of
+// eF_j, and |r|^max(|m| - 1, 0), above the terms (b_{c+1} - b_{c-1}) / 6 of a PMBC weight.
+std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K, std::vector<double>* mag) {
   const std::vector<double> W = pmbc_weights_scaled(n, p, n_nb);
   const int M = n / p;
   const int R = std::max(n_nb, K);
@@ -95,22 +97,31 @@ std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K) {
   const double r = std::sqrt(3.0) - 2.0;
   const double a = (1.0 - r * r) / (2.0 * std::sqrt(3.0));
   std::vector<double> D((size_t)(p + 1) * wl, 0.0);
+  if (mag) mag->assign(D.size(), 0.0);
   for (int j = 0; j <= p; ++j) {
     const int c = j * M;
     double* Dj = D.data() + (size_t)j * wl + R;  // Dj[m], m = -R..R
+    double* Gj = mag ? mag->data() + (size_t)j * wl + R : nullptr;
     for (int m = -n_nb; m <= n_nb; ++m)
-      if (c + m >= 0 && c + m <= n) Dj[m] += W[(size_t)j * (2 * n_nb + 1) + (m + n_nb)];
+      if (c + m >= 0 && c + m <= n) {
+        Dj[m] += W[(size_t)j * (2 * n_nb + 1) + (m + n_nb)];
+        if (Gj) Gj[m] += std::pow(-r, std::max(std::abs(m) - 1, 0));
+      }
+    auto term = [&](int m, double w) {
+      Dj[m] += w;
+      if (Gj) Gj[m] += std::fabs(w);
+    };
     auto add = [&](int pos, double w) {
       if (pos >= 0 && pos <= n) {
-        Dj[pos - c] += w;
+        term(pos - c, w);
       } else if (pos < 0) {
         const int q = std::min(-pos, n);
-        Dj[0 - c] += 2.0 * w;
-        Dj[q - c] -= w;
+        term(0 - c, 2.0 * w);
+        term(q - c, -w);
       } else {
         const int q = std::max(n - (pos - n), 0);
-        Dj[n - c] += 2.0 * w;
-        Dj[q - c] -= w;
+        term(n - c, 2.0 * w);
+        term(q - c, -w);
       }
     };
     double rk = 1.0;

@@ -25,11 +25,12 @@ inline int force_components(uint32_t kinds) {
 }
 
 // Host side of an axis's tables (conv_host): the bytes to upload, laid out as double r^d (d < 64), ConvTap taps[ntaps],
-// double wd[p + 1][2 R + 1], int js[p + 2]; ok: the engines take the axis.
+// int js[p + 2] (with one more where that is odd), double wd[p + 1][2 R + 1]; the first `forward` of them, without wd, are
+// what the derivative reads (the transpose reads wd); ok: the engines take the axis.
 struct ConvHost {
   int Q = 0, ntaps = 0, R = 0;
   bool ok = false;
-  size_t bytes = 0;
+  size_t forward = 0;
 };
 
 // One independent grid (shot).  Internal axis slots: 0 = z, 1 = y, 2 = x; 2-D grids have a y extent of 1.
@@ -233,7 +234,7 @@ loss_status_t run_derivative_adjoint(loss_ctx* h, Shot& s, int k, const void* g,
 loss_status_t run_gradient(loss_ctx* h, Shot& s, const double* d_obs, int32_t checkpoint_every, int64_t n_steps,
                            double* misfit, double* g_vp, double* g_vs, double* g_rho, int32_t mem);
 std::vector<double> pmbc_weights_scaled(int n, int p, int n_nb);
-std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K);
+std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K, std::vector<double>* mag = nullptr);
 void thomas_tables(std::vector<double>& t64, std::vector<float>& t32);
 
 // Counts one launch of `kernel` and, when profiling is on, brackets it with CUDA events on the stream.
@@ -324,7 +325,7 @@ cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMa
 template <typename T>
 cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, bool acc, const T* in,
                                 T* out, T scale, T scale_lo, cudaStream_t st);
-// Whether the operators of axis slot k run on the engines, for tables of c.bytes bytes: those fit the static array of
+// Whether the operators of axis slot k run on the engines: the derivative's tables fit the static array of
 // loss_derivative_noalloc (which launches the same kernels), and the dense array fits the engines' 32-bit offsets.
 constexpr size_t kNoAllocScratchBytes = 64 * 1024;
 bool conv_operator_ok(const Shot& s, int k, const ConvHost& c);

@@ -55,7 +55,7 @@ static loss_status_t noalloc_run(loss_ctx* h, Shot& s, int k, const T* f, T* d1,
   ConvHost ch;
   const std::vector<unsigned char> blob = conv_host(s, k, &ch);
   if (conv_operator_ok(s, k, ch) && !overlaps(s, f, d1)) {  // the kernels that loss_derivative takes for this axis
-    if (cudaMemcpyAsync(scratch, blob.data(), blob.size(), cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
+    if (cudaMemcpyAsync(scratch, blob.data(), ch.forward, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
       return LOSS_E_CUDA;
     return deriv_stream<T>(h, s, k, conv_axis_at(s, k, ch, scratch), h->num_sms, f, d1, nullptr);
   }

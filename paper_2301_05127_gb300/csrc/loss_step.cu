@@ -572,19 +572,36 @@ std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
   const bool f32 = s.esize == 4;
   const int K = f32 ? 16 : 32;
   const int R0 = std::max(s.d.n_nb, K), wl = 2 * R0 + 1;
-  const std::vector<double> D = fir_delta_weights(n, p, s.d.n_nb, K);
+  std::vector<double> mag;
+  const std::vector<double> D = fir_delta_weights(n, p, s.d.n_nb, K, &mag);
   const double a = fir_const(M).a;
-  // weights that are rounding noise of the difference (or reach less than the last digit) are left out
-  const double tiny = f32 ? 0x1p-44 : 0x1p-52;
-  std::vector<int> js(p + 2, 0);
+  // Left out are weights within the rounding error of their difference (4 x 2^-53 of its terms; the exact ones vanish
+  // there, or are of order r^K), and of the others the smallest whose magnitudes sum to no more than `tiny` per junction.
+  const double tiny = f32 ? 0x1p-44 : 0x1p-58;
+  std::vector<int> js((p + 3) & ~1, 0);
   std::vector<ConvTap> taps;
+  std::vector<double> size;
   double dmax = 0.0;
   for (int j = 0; j <= p; ++j) {
     js[j] = (int)taps.size();
+    const double *Dj = &D[(size_t)j * wl], *Gj = &mag[(size_t)j * wl];
+    size.clear();
+    for (int i = 0; i < wl; ++i)
+      if (std::fabs(Dj[i]) > 0x1p-51 * Gj[i]) size.push_back(std::fabs(Dj[i]));
+    std::sort(size.begin(), size.end());
+    double cut = 0.0, prev = 0.0, left = 0.0;  // weights up to cut go, all equal ones or none
+    for (double v : size) {
+      left += v;
+      if (left > tiny) {
+        if (v == cut) cut = prev;
+        break;
+      }
+      if (v != cut) prev = cut, cut = v;
+    }
     double sum = 0.0;
     for (int m = -R0; m <= R0; ++m) {
-      const double w = D[(size_t)j * wl + R0 + m];
-      if (std::fabs(w) <= tiny) continue;
+      const double w = Dj[R0 + m];
+      if (std::fabs(w) <= std::max(cut, 0x1p-51 * Gj[R0 + m])) continue;
       ConvTap t{};
       t.w = w / a;
       t.m = m;
@@ -594,7 +611,7 @@ std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
     }
     dmax = std::max(dmax, sum);
   }
-  js[p + 1] = (int)taps.size();
+  for (size_t i = p + 1; i < js.size(); ++i) js[i] = (int)taps.size();
   // reach of a correction: |r|^Q dmax below the working precision
   const double eps = f32 ? 0x1p-40 : 0x1p-58;
   for (double q = dmax; q > eps && c->Q < 64; q *= -kConvRHost) ++c->Q;
@@ -619,9 +636,9 @@ std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
   };
   put(pw, sizeof(pw));
   put(taps.data(), taps.size() * sizeof(ConvTap));
-  put(wd.data(), wd.size() * sizeof(double));
   put(js.data(), js.size() * sizeof(int));
-  c->bytes = blob.size();
+  c->forward = blob.size();
+  put(wd.data(), wd.size() * sizeof(double));
   return blob;
 }
 ConvAxis conv_axis_at(const Shot& s, int k, const ConvHost& c, const void* tab) {
@@ -629,8 +646,8 @@ ConvAxis conv_axis_at(const Shot& s, int k, const ConvHost& c, const void* tab) 
   g.n = (int)s.n[k], g.p = s.p[k], g.M = g.n / g.p, g.Q = c.Q, g.ntaps = c.ntaps, g.R = c.R;
   g.pw = (const double*)tab;
   g.taps = (const ConvTap*)(g.pw + 64);
-  g.wd = (const double*)(g.taps + g.ntaps);
-  g.js = (const int*)(g.wd + (size_t)(g.p + 1) * (2 * g.R + 1));
+  g.js = (const int*)(g.taps + g.ntaps);
+  g.wd = (const double*)(g.js + ((g.p + 3) & ~1));
   return g;
 }
 loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok) {
@@ -690,7 +707,7 @@ RowMap row_map(int num_sms, const Shot& s, int nf, const ConvAxis& g, int64_t py
 }
 
 bool conv_operator_ok(const Shot& s, int k, const ConvHost& c) {
-  return c.ok && c.bytes <= kNoAllocScratchBytes && (uint64_t)s.dense * s.esize <= UINT32_MAX &&
+  return c.ok && c.forward <= kNoAllocScratchBytes && (uint64_t)s.dense * s.esize <= UINT32_MAX &&
          s.len[0] * s.len[1] * ((s.n[2] + 191) / 192) < INT32_MAX / 2 && 4 * (s.n[k] / s.p[k]) > 8 + 2 * c.R;
 }
 // d1 (and d2) along slot k of dense arrays.

@@ -38,3 +38,55 @@ def test_fp32_transpose_at_small_halos(pkg, axis, n_nb):
     tol = tol[:, None] if axis == 0 else tol[None, :]
     assert (np.abs(out[0] - out[1]) <= tol).all()
     assert np.sqrt(np.mean((out[0] - out[1]) ** 2)) <= 0.25 * 3.0 * A * u * (2.0 * q + 6.0)
+
+
+@pytest.mark.parametrize("axis", [0, 1])
+def test_left_out_weights_stay_below_the_last_digit(pkg, axis):
+    """FP64: a sample beyond the halo of a junction (n_nb < m <= 32) has no weight there, so its derivative at the
+    junction is 0, and so is the transpose at the sample.  The convolution's own term cancels against the correction's
+    weight: what is left is at most the sum of the weights left out, 2^-58, and the term beyond 32 positions, A |r|^32."""
+    n, p, n_nb = 128, 2, 12
+    g = pkg.Grid([pkg.make_desc(2, pkg.LOSS_ACOUSTIC, pkg.LOSS_FP64, n_nb, (n, n), (p, p), (1.0, 1.0), 1e-3)])
+    f = np.zeros(g.shape())
+    t = np.zeros(g.shape())
+    dist = [(k, m) for k, m in enumerate([s * m for m in range(n_nb + 1, 33) for s in (1, -1)])]
+    for k, m in dist:
+        f[k, 64 + m] = 1.0
+        t[k, 64] = 1.0
+    if axis == 0:
+        f, t = f.T.copy(), t.T.copy()
+    d = g.derivative(0, axis, f)
+    a = g.derivative_adjoint(0, axis, t)
+    if axis == 0:
+        d, a = d.T, a.T
+    g.close()
+    bound = 3.0 * (2.0 ** -58 + A * 0.26794919243112270647 ** 32)
+    assert max(abs(d[k, 64]) for k, _ in dist) <= bound
+    assert max(abs(a[k, 64 + m]) for k, m in dist) <= bound
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_axes_of_many_patches(pkg, prec):
+    """120 patches: the derivative's tables still fit the static array of the variant without allocations, the transpose's
+    are larger.  Against dense matrices of the oracle, and the same bits from the variant."""
+    import ctypes
+
+    import torch
+
+    from oracle import spline
+
+    n, p, n_nb = 3360, 120, 20
+    tol = 1e-12 if prec == "fp64" else 2e-5
+    d = pkg.make_desc(2, pkg.LOSS_ACOUSTIC, pkg.PRECISIONS[prec], n_nb, (n, 20), (p, 1), (1.0, 1.0), 1e-3)
+    g = pkg.Grid([d])
+    f = np.random.default_rng(4).standard_normal(g.shape()).astype(g.dtype)
+    D = spline.derivative(np.eye(n + 1), 0, n, p, 1.0, n_nb)
+    for op, ref in ((g.derivative, D @ f), (g.derivative_adjoint, D.T @ f)):
+        assert np.abs(op(0, 0, f) - ref).max() < tol * np.abs(ref).max()
+    x = torch.from_numpy(f).cuda()
+    out = torch.empty_like(x)
+    st = pkg.lib().loss_derivative_noalloc(ctypes.byref(d), 0, x.data_ptr(), out.data_ptr(),
+                                           ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == pkg.LOSS_OK
+    assert np.array_equal(out.cpu().numpy(), g.derivative(0, 0, f))
+    g.close()
