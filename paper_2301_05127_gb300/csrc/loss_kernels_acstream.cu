@@ -146,7 +146,6 @@ struct AcRowOp {
     if constexpr (KAHAN) ld9(a.cv1 + gi, true, len, c);
     if (b_on) ld9(a.b + gi, true, len, bb);
     if (lay) ld9(a.psix + gi, true, len, m);
-    const T sa = -(a.s3h * a.acoef), sa_lo = -(a.s3h * a.acoef_lo + a.s3h_lo * a.acoef);  // with an array of b
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
       if (j == 8 && len < 9) break;
@@ -161,7 +160,7 @@ struct AcRowOp {
         }
         e[j] = b_on ? bb[j] * e[j] : mulc(e[j], a.b0, a.b0_lo);
       } else if (b_on) {
-        e[j] = bb[j] * mulc(e[j], sa, sa_lo);
+        e[j] = bb[j] * mulc(e[j], a.sa, a.sa_lo);
       } else if constexpr (sizeof(T) == 8) {
         v[j] = fma(e[j], a.sc, v[j]);
         e[j] = T(0);

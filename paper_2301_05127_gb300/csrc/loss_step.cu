@@ -224,6 +224,8 @@ static void conv_scale(A& a, const Shot& s, int k, double acoef) {
   if constexpr (std::is_same_v<A, AcXArgs<T>>) {
     a.sdt = (T)(sc * s.d.dt);
     a.sdt_lo = lo_part<T>(sc * s.d.dt);
+    a.sa = (T)(-acoef * sc);
+    a.sa_lo = lo_part<T>(-acoef * sc);
   }
 }
 // A 2-D shot's arrays are within the engines' 32-bit byte offsets and row counts.

@@ -152,6 +152,7 @@ struct AcXArgs {
   T dt_lo, acoef_lo, s3h_lo, b0_lo;  // rounding errors of dt, acoef, s3h, b0 (mulc; 0 in FP64)
   T sc, sc_lo;       // -acoef * b0 * s3h and its rounding error (the velocity update with constant density)
   T sdt, sdt_lo;     // s3h * dt and its rounding error (row engine)
+  T sa, sa_lo;       // -acoef * s3h and its rounding error (row engine: the velocity update with an array of b)
   T minf;
   int do_B;
   SourceArgs src;
