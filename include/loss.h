@@ -244,7 +244,10 @@ enum {
 /* Launch shape of one kernel family of the handle: lines_per_block = number of whole grid lines one thread block
  * holds on chip (power of two, 1..32) and chunk_log2 = log2 of the number of unknowns one thread solves serially
  * (3 or 4; FP64 grids always use 4); 0 = the built-in choice.  Applies to every shot; shapes that do not fit
- * fall back to smaller bundles at launch.  Used by the autotuner. */
+ * fall back to smaller bundles at launch.  Shapes are those of the kernels that hold whole lines on chip: a derivative,
+ * its transpose, an FP64 acoustic step or an elastic step for one of whose kernels a shape is set runs on them
+ * (loss_set_kernels); the truncated-convolution kernels of the FP32 acoustic step take none but the z chunk
+ * (loss_set_tile).  Used by the autotuner. */
 loss_status_t loss_set_launch(loss_handle_t handle, int32_t kernel, int32_t lines_per_block, int32_t chunk_log2);
 
 /* Tile shape of one kernel family given as a block size: threads_per_block (32..1024, 512 at most for FP64 grids)
@@ -301,7 +304,9 @@ typedef struct {
  * block 128..1024, chunk_log2 3 or 4; for the convolution kernels the z chunk of Z1 and Z2) of each kernel family the
  * handle's time step uses, on a scratch copy of the handle (same grids, models, absorbing layers, kernel family
  * and schedule; zero fields), with `steps` timed steps per candidate
- * after one warm-up step, and applies the fastest shape of each family to the handle (loss_set_tile).  The
+ * after one warm-up step, and applies the fastest shape of each family to the handle (loss_set_tile).  Where the built-in
+ * step runs on kernels without shapes (FP64 acoustic and elastic steps, loss_set_kernels), it is timed too and kept when its
+ * kernels together take no longer than those with the shapes: entries of threads_per_block = chunk_log2 = 0.  The
  * handle's own state is not touched.  out (capacity cap entries, may be NULL) receives one entry per tuned
  * family and *n_out their number.  Needs device memory for a second copy of the handle's arrays.
  * Returns LOSS_E_ARG for steps < 1, the error of the first failing call otherwise. */

@@ -704,6 +704,27 @@ loss_status_t loss_autotune(loss_handle_t h, int32_t steps, loss_tune_entry_t* o
   const double inf = 1e300;
   std::vector<double> best(kids.size(), inf);
   std::vector<int> best_c(kids.size(), -1);
+  // Steps that run on the engines run on the line kernels with any shape, so there the built-in choice is a candidate of
+  // its own, for all kernels of the step together: base[f], and base_z2 for the launches that only the engines have.
+  const bool z2 = std::find(kids.begin(), kids.end(), (int)LOSS_KERNEL_ACOUSTIC_Z2) != kids.end();
+  bool ac_engine = false, el_engine = false;
+  std::vector<double> base(kids.size(), 0.0);
+  double base_z2 = 0.0;
+  for (int kid : kids) t->lines_per_block[kid] = t->tile_threads[kid] = t->chunk_log2[kid] = 0;
+  if (ac) LOSS_TRY(relay(engine_steps(t, LOSS_ACOUSTIC, &ac_engine)));
+  if (el) LOSS_TRY(relay(engine_steps(t, LOSS_ELASTIC, &el_engine)));
+  if (ac_engine || el_engine) {
+    LOSS_TRY(relay(loss_step(t, 1)));
+    LOSS_TRY(relay(loss_profile(t, 1)));
+    LOSS_TRY(relay(loss_step(t, steps)));
+    for (size_t f = 0; f < kids.size(); ++f) {
+      LOSS_TRY(relay(loss_profile_read(t, kids[f], &base[f], nullptr)));
+      base[f] /= steps;
+    }
+    if (!z2) LOSS_TRY(relay(loss_profile_read(t, LOSS_KERNEL_ACOUSTIC_Z2, &base_z2, nullptr)));
+    base_z2 /= steps;
+    LOSS_TRY(relay(loss_profile(t, 0)));
+  }
   for (size_t c = 0; c < cand.size(); ++c) {
     for (int kid : kids) {
       t->lines_per_block[kid] = 0;
@@ -724,13 +745,26 @@ loss_status_t loss_autotune(loss_handle_t h, int32_t steps, loss_tune_entry_t* o
     }
     LOSS_TRY(relay(loss_profile(t, 0)));
   }
+  // (a kernel for which no shape fits has best = inf: the built-in choice)
+  double built_in[2] = {base_z2, 0.0}, chosen[2] = {0.0, 0.0};  // of the acoustic and the elastic kernels
+  auto elastic = [](int kid) { return kid == LOSS_KERNEL_ELASTIC_X || kid == LOSS_KERNEL_ELASTIC_Y || kid == LOSS_KERNEL_ELASTIC_Z; };
+  for (size_t f = 0; f < kids.size(); ++f) {
+    const int e = elastic(kids[f]) ? 1 : 0;
+    built_in[e] += base[f];
+    chosen[e] += best[f];
+  }
+  const bool keep[2] = {ac_engine && built_in[0] <= chosen[0], el_engine && built_in[1] <= chosen[1]};
   int32_t n = 0;
   for (size_t f = 0; f < kids.size(); ++f) {
-    if (best_c[f] < 0) continue;
+    loss_tune_entry_t r{kids[f], 0, 0, base[f]};
+    if (!keep[elastic(kids[f]) ? 1 : 0]) {
+      if (best_c[f] < 0) continue;
+      r = loss_tune_entry_t{kids[f], cand[best_c[f]].first, cand[best_c[f]].second, best[f]};
+    }
     h->lines_per_block[kids[f]] = 0;
-    h->tile_threads[kids[f]] = cand[best_c[f]].first;
-    h->chunk_log2[kids[f]] = cand[best_c[f]].second;
-    if (out && n < cap) out[n] = loss_tune_entry_t{kids[f], cand[best_c[f]].first, cand[best_c[f]].second, best[f]};
+    h->tile_threads[kids[f]] = r.threads_per_block;
+    h->chunk_log2[kids[f]] = r.chunk_log2;
+    if (out && n < cap) out[n] = r;
     ++n;
   }
   if (n_out) *n_out = n;

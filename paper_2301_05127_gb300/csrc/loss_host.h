@@ -267,6 +267,8 @@ loss_status_t step_shot(loss_ctx* h, Shot& s, bool head = false, bool more = fal
 loss_status_t unstagger(loss_ctx* h, Shot& s);
 loss_status_t stagger_shot(loss_ctx* h, Shot& s);
 bool batch_eligible(const loss_ctx* h);
+// Whether some shot of a physics has the step that launch shapes take off the engines (FP64 acoustic, elastic) on them now.
+loss_status_t engine_steps(loss_ctx* h, int physics, bool* on);
 bool conv_z_used(const loss_ctx* h);  // some shot's FP32 step runs the convolution z tiles
 loss_status_t step_batched(loss_ctx* h, int64_t n_steps);
 void batch_release(loss_ctx* h);

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -233,11 +234,20 @@ static bool conv_size_ok(const Shot& s) {
   return (uint64_t)s.total * s.esize <= UINT32_MAX && s.len[0] * ((s.n[2] + 191) / 192) < INT32_MAX / 2;
 }
 
-// The FP64 step of a 2-D acoustic shot on the barrier-free engines (the convolution family, axes that qualify).  The
-// line kernels' limits on the length of lines stay the limits of the step.
+// Whether the caller asked for a launch shape of one of these kernels (loss_set_launch, loss_set_tile).  Shapes are the line
+// kernels'; a step with one runs on them.
+static bool shaped(const loss_ctx* h, std::initializer_list<int> kids) {
+  for (int k : kids)
+    if (h->lines_per_block[k] > 0 || h->tile_threads[k] > 0 || h->chunk_log2[k] > 0) return true;
+  return false;
+}
+
+// The FP64 step of a 2-D acoustic shot on the barrier-free engines (the convolution family, axes that qualify, no launch
+// shape asked for).  The line kernels' limits on the length of lines stay the limits of the step.
 static loss_status_t acs_ok(loss_ctx* h, Shot& s, bool* ok) {
   *ok = false;
   if (!h->tiled || s.esize != 8 || s.dim != 2 || s.d.physics != LOSS_ACOUSTIC || !conv_size_ok(s)) return LOSS_OK;
+  if (shaped(h, {LOSS_KERNEL_ACOUSTIC_X, LOSS_KERNEL_ACOUSTIC_Z})) return LOSS_OK;
   for (int k : {0, 2}) {
     ConvAxis g;
     LOSS_TRY(conv_axis(h, s, k, &g, ok));
@@ -729,13 +739,14 @@ template loss_status_t deriv_stream<float>(loss_ctx*, const Shot&, int, const Co
 template loss_status_t deriv_stream<double>(loss_ctx*, const Shot&, int, const ConvAxis&, int, const double*, double*,
                                             double*);
 
-// The elastic step on those engines: the convolution family (loss_set_kernels) when every axis qualifies; in FP32 neither
-// the gradient's forward runs nor the items family, which keeps the kernels that both loss_step and loss_gradient take.
+// The elastic step on those engines: the convolution family (loss_set_kernels) when every axis qualifies and no launch
+// shape is asked for; in FP32 neither the gradient's forward runs nor the items family, which keeps the kernels that both loss_step and loss_gradient take.
 // The line kernels' limit on the length of a row stays the limit of the step.
 template <typename T>
 static loss_status_t els_ok(loss_ctx* h, Shot& s, bool* ok) {
   *ok = false;
   if (!h->tiled || s.dim != 3) return LOSS_OK;
+  if (shaped(h, {LOSS_KERNEL_ELASTIC_X, LOSS_KERNEL_ELASTIC_Y, LOSS_KERNEL_ELASTIC_Z})) return LOSS_OK;
   if (s.esize == 4 && (h->in_gradient || h->tiled == LOSS_KERNELS_CONVOLUTION_ITEMS)) return LOSS_OK;
   if ((uint64_t)s.total * s.esize > UINT32_MAX) return LOSS_OK;  // the engines use 32-bit byte offsets
   for (int k = 0; k < 3; ++k) {
@@ -746,6 +757,17 @@ static loss_status_t els_ok(loss_ctx* h, Shot& s, bool* ok) {
     int logc, threads;
     if (k == 2 && s.len[0] * s.len[1] * ((g.n + 223) / 224) > INT32_MAX / 2) return *ok = false, LOSS_OK;
     if (k == 2 || s.esize == 8) LOSS_TRY(line_geom(h, s, k, s.sz, s.sy, &lg, &logc, &threads, 6, 0, 0, 0, 0));
+  }
+  return LOSS_OK;
+}
+
+loss_status_t engine_steps(loss_ctx* h, int physics, bool* on) {
+  *on = false;
+  for (Shot& s : h->shots) {
+    if (*on || s.d.physics != physics || any_nonuniform(s)) continue;
+    if (physics == LOSS_ACOUSTIC) LOSS_TRY(acs_ok(h, s, on));
+    else if (s.esize == 8) LOSS_TRY(els_ok<double>(h, s, on));
+    else LOSS_TRY(els_ok<float>(h, s, on));
   }
   return LOSS_OK;
 }

@@ -98,3 +98,64 @@ def test_long_rows_do_not_depend_on_other_shots(pkg, prec):
     assert _same(other[0], alone[0])
     pair, _ = _run(pkg, ws[1:2], batched=False, seeds=[1])
     assert _same(pair[0], ref[1])
+
+
+ELASTIC = ("v1", "v2", "v3", "s11", "s22", "s33", "s12", "s13", "s23")
+SHAPED = [("acoustic", "fp64", "acoustic_x", "line"), ("acoustic", "fp64", "acoustic_z", "line"),
+          ("elastic", "fp64", "elastic_y", "line"), ("elastic", "fp32", "elastic_x", "convolution_items"),
+          ("elastic", "fp32_kahan", "elastic_x", "convolution_items")]
+
+
+def _engine_workload(physics, prec):
+    """A grid whose FP64 acoustic or elastic step runs without launch shapes by default."""
+    if physics == "acoustic":
+        return _shot((64, 128), (1, 2), 12, prec, 61)
+    return dataclasses.replace(elastic3d_homogeneous(n=48, p=1, n_nb=8, steps=5, precision=prec, pml_width=8), receivers={}, f0=40.0,
+                               t0=0.004)
+
+
+def _steps(pkg, w, n, family="convolution", shapes=()):
+    g = pkg.Grid.from_workloads([w])
+    g.set_kernels(family)
+    for kernel, threads, chunk in shapes:
+        g.set_tile(kernel, threads, chunk)
+    g.step(n)
+    names = FIELDS if len(w.n) == 2 else ELASTIC
+    out = [g.get_field(0, f) for f in names]
+    z2 = g.profile_read("acoustic_z2")[1]
+    g.close()
+    return out, z2
+
+
+@pytest.mark.parametrize("physics,prec,kernel,family", SHAPED)
+def test_shape_asked_for_is_used(pkg, physics, prec, kernel, family):
+    """A launch shape belongs to the kernels that hold whole lines: with one the step is theirs, bit for bit, and without
+    it again the built-in choice's."""
+    w = _engine_workload(physics, prec)
+    plain, z2 = _steps(pkg, w, 5)
+    ref, _ = _steps(pkg, w, 5, family, [(kernel, 128, 4)])
+    got, got_z2 = _steps(pkg, w, 5, shapes=[(kernel, 128, 4)])
+    assert np.abs(ref[0]).max() > 0 and not _same(plain, ref)  # the two families differ in rounding
+    assert _same(got, ref)
+    assert got_z2 == 0 and (physics == "elastic" or z2 > 0)
+    back, _ = _steps(pkg, w, 5, shapes=[(kernel, 128, 4), (kernel, 0, 0)])
+    assert _same(back, plain)
+
+
+@pytest.mark.parametrize("physics,prec", [("acoustic", "fp64"), ("elastic", "fp64"), ("elastic", "fp32_kahan")])
+def test_autotune_reports_what_runs(pkg, physics, prec):
+    """Steps without launch shapes: the tuner's entries are the built-in choice for all kernels or a shape for each, and
+    the tuned handle runs what they say."""
+    w = _engine_workload(physics, prec)
+    g = pkg.Grid.from_workloads([w])
+    res = g.autotune(steps=2)
+    assert set(res) == ({"acoustic_x", "acoustic_z"} if physics == "acoustic" else {"elastic_x", "elastic_y", "elastic_z"})
+    assert all(r["ms"] > 0 for r in res.values())
+    built_in = [r["threads_per_block"] == 0 and r["chunk_log2"] == 0 for r in res.values()]
+    assert all(built_in) or not any(built_in)
+    g.step(5)
+    got = [g.get_field(0, f) for f in (FIELDS if physics == "acoustic" else ELASTIC)]
+    assert physics == "elastic" or (g.profile_read("acoustic_z2")[1] > 0) == built_in[0]
+    g.close()
+    ref, _ = _steps(pkg, w, 5, shapes=[(k, r["threads_per_block"], r["chunk_log2"]) for k, r in res.items()])
+    assert _same(got, ref)
