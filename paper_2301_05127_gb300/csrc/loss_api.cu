@@ -87,10 +87,10 @@ std::vector<double> pmbc_weights_scaled(int n, int p, int n_nb) {
 // eF_j = a sum_{k=1..K} r^{k-1} (f_{c+k} - f_{c-k}) with the line continued by odd reflection beyond its ends
 // (f_{-q} = 2 f_0 - f_q, f_{n+q} = 2 f_n - f_{n-q}, q clamped to the line).  Formed in FP64; away from the
 // physical ends the two weight sets agree to O(r^K), so the FP32 sum of D f carries no cancellation.
-// mag (may be null): at each position a bound on the terms whose difference the weight is, for its rounding error: those of
+// W: pmbc_weights_scaled of the axis.  mag (may be null): at each position a bound on the terms whose difference the weight is, for its rounding error: those of
 // eF_j, and |r|^max(|m| - 1, 0), above the terms (b_{c+1} - b_{c-1}) / 6 of a PMBC weight.
-std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K, std::vector<double>* mag) {
-  const std::vector<double> W = pmbc_weights_scaled(n, p, n_nb);
+std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K, const std::vector<double>& W,
+                                      std::vector<double>* mag) {
   const int M = n / p;
   const int R = std::max(n_nb, K);
   const int wl = 2 * R + 1;
@@ -414,7 +414,7 @@ static loss_status_t setup_shot(loss_ctx* h, Shot& s) {
     // now, so that the operators may be captured on a caller's stream
     ConvAxis g;
     bool ok;
-    LOSS_TRY(conv_axis(h, s, k, &g, &ok));
+    LOSS_TRY(conv_axis(h, s, k, &g, &ok, &W));
   }
   return LOSS_OK;
 }

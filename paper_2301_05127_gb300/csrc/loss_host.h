@@ -234,7 +234,8 @@ loss_status_t run_derivative_adjoint(loss_ctx* h, Shot& s, int k, const void* g,
 loss_status_t run_gradient(loss_ctx* h, Shot& s, const double* d_obs, int32_t checkpoint_every, int64_t n_steps,
                            double* misfit, double* g_vp, double* g_vs, double* g_rho, int32_t mem);
 std::vector<double> pmbc_weights_scaled(int n, int p, int n_nb);
-std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K, std::vector<double>* mag = nullptr);
+std::vector<double> fir_delta_weights(int n, int p, int n_nb, int K, const std::vector<double>& W,
+                                      std::vector<double>* mag = nullptr);
 void thomas_tables(std::vector<double>& t64, std::vector<float>& t32);
 
 // Counts one launch of `kernel` and, when profiling is on, brackets it with CUDA events on the stream.
@@ -257,9 +258,9 @@ struct LaunchScope {
 
 // loss_step.cu
 // Axis slot k of a shot on the barrier-free engines (loss_stream.cuh): uploads its tables on first use; *ok = false
-// when the axis does not qualify.
-loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok);
-std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c);
+// when the axis does not qualify.  W: the axis's pmbc_weights_scaled where the caller has them.
+loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok, const std::vector<double>* W = nullptr);
+std::vector<unsigned char> conv_host(const Shot& s, int k, const std::vector<double>& W, ConvHost* c);
 ConvAxis conv_axis_at(const Shot& s, int k, const ConvHost& c, const void* tab);  // the tables at a device address
 ColMap col_map(int num_sms, const Shot& s, int k, int64_t py, int64_t pz);  // strided lines, slot 0 or 1
 RowMap row_map(int num_sms, const Shot& s, int nf, const ConvAxis& g, int64_t py, int64_t pz, bool vec);  // rows along x

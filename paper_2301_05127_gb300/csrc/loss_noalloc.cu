@@ -53,7 +53,7 @@ static loss_status_t noalloc_run(loss_ctx* h, Shot& s, int k, const T* f, T* d1,
   loss_status_t st = line_geom(h, s, k, s.len[2] * s.len[1], s.len[2], &g, &logc, &threads, 2, 0, 0, 0);
   if (st != LOSS_OK) return st;
   ConvHost ch;
-  const std::vector<unsigned char> blob = conv_host(s, k, &ch);
+  const std::vector<unsigned char> blob = conv_host(s, k, W, &ch);
   if (conv_operator_ok(s, k, ch) && !overlaps(s, f, d1)) {  // the kernels that loss_derivative takes for this axis
     if (cudaMemcpyAsync(scratch, blob.data(), ch.forward, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
       return LOSS_E_CUDA;

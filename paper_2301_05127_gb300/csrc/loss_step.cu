@@ -196,7 +196,8 @@ static TileGeom tile_geom(const Shot& s, int k, int* threads, int zlogc = 4) {
 // Junction-correction weights of axis slot k in device memory (FP32 truncated-convolution kernels).
 static loss_status_t ensure_delta_weights(loss_ctx* h, Shot& s, int k) {
   if (s.Wd[k]) return LOSS_OK;
-  const std::vector<double> D = fir_delta_weights((int)s.n[k], s.p[k], s.d.n_nb, FirLen<float>::K);
+  const int n = (int)s.n[k], n_nb = s.d.n_nb;
+  const std::vector<double> D = fir_delta_weights(n, s.p[k], n_nb, FirLen<float>::K, pmbc_weights_scaled(n, s.p[k], n_nb));
   void* p = nullptr;
   LOSS_TRY(dev_alloc(h, D.size() * sizeof(double), &p));
   LOSS_TRY(cuda_check(h, cudaMemcpyAsync(p, D.data(), D.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream),
@@ -577,7 +578,7 @@ static loss_status_t elt_pass(loss_ctx* h, Shot& s, int pass, double acoef, doub
 
 // ---------------------------------------------------------------------------------------------------------------
 // Axes of the barrier-free engines (loss_stream.cuh).
-std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
+std::vector<unsigned char> conv_host(const Shot& s, int k, const std::vector<double>& W, ConvHost* c) {
   const int n = (int)s.n[k], p = s.p[k], M = n / p;
   *c = ConvHost{};
   if (n < 40) return {};  // the line ends' closed forms need whole warm-up sums beside them
@@ -585,7 +586,7 @@ std::vector<unsigned char> conv_host(const Shot& s, int k, ConvHost* c) {
   const int K = f32 ? 16 : 32;
   const int R0 = std::max(s.d.n_nb, K), wl = 2 * R0 + 1;
   std::vector<double> mag;
-  const std::vector<double> D = fir_delta_weights(n, p, s.d.n_nb, K, &mag);
+  const std::vector<double> D = fir_delta_weights(n, p, s.d.n_nb, K, W, &mag);
   const double a = fir_const(M).a;
   // Left out are weights within the rounding error of their difference (4 x 2^-53 of its terms; the exact ones vanish
   // there, or are of order r^K), and of the others the smallest whose magnitudes sum to no more than `tiny` per junction.
@@ -662,11 +663,12 @@ ConvAxis conv_axis_at(const Shot& s, int k, const ConvHost& c, const void* tab) 
   g.wd = (const double*)(g.js + ((g.p + 3) & ~1));
   return g;
 }
-loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok) {
+loss_status_t conv_axis(loss_ctx* h, Shot& s, int k, ConvAxis* g, bool* ok, const std::vector<double>* W) {
   *ok = false;
   if (s.n[k] < 40) return LOSS_OK;
   if (!s.conv_tab[k]) {
-    const std::vector<unsigned char> blob = conv_host(s, k, &s.conv[k]);
+    const std::vector<unsigned char> blob =
+        conv_host(s, k, W ? *W : pmbc_weights_scaled((int)s.n[k], s.p[k], s.d.n_nb), &s.conv[k]);
     void* d = nullptr;
     LOSS_TRY(dev_alloc(h, blob.size(), &d));
     LOSS_TRY(cuda_check(h, cudaMemcpyAsync(d, blob.data(), blob.size(), cudaMemcpyHostToDevice, h->stream),
