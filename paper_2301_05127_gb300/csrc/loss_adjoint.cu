@@ -404,13 +404,15 @@ loss_status_t run_gradient(loss_ctx* h, Shot& s, const double* d_obs, int32_t ch
                                     mem == LOSS_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
                       "copy d_obs"));
   LOSS_TRY(cuda_check(h, cudaStreamSynchronize(cudaStreamLegacy), "sync"));
-  // the model as loss_set_model got it, in FP64 on the device from the first gradient on (refreshed after a new model)
+  // the model as loss_set_model got it, in FP64 on the device from the first gradient on (refreshed after a new model):
+  // allocated, copied and read by k_chain in the order of the handle's stream
   if (!s.dmodel) LOSS_TRY(dev_alloc(h, (el ? 3 : 2) * N * sizeof(double), (void**)&s.dmodel));
   if (!s.dmodel_valid) {
     const std::vector<double>* src[3] = {&s.h_vp, &s.h_rho, &s.h_vs};
     for (int i = 0; i < (el ? 3 : 2); ++i)
-      LOSS_TRY(cuda_check(h, cudaMemcpy(s.dmodel + i * N, src[i]->data(), N * sizeof(double), cudaMemcpyHostToDevice),
-                          "copy model"));
+      LOSS_TRY(cuda_check(h, cudaMemcpyAsync(s.dmodel + i * N, src[i]->data(), N * sizeof(double), cudaMemcpyHostToDevice,
+                                             h->stream), "copy model"));
+    LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));  // the source may be replaced
     s.dmodel_valid = true;
   }
   struct Flag {  // (also reset when a call fails)

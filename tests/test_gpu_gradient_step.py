@@ -60,3 +60,32 @@ def test_own_traces_have_no_misfit(pkg, kind, prec, family):
         return
     assert J == 0.0 and np.array_equal(tr, obs)
     assert not any(np.any(v) for v in grads.values() if v is not None)
+
+
+def test_gradient_after_a_new_model(pkg):
+    """The chain rule's model follows loss_set_model, on a stream that does not wait for the legacy default stream: a
+    handle's second gradient, at another model, has the bits of a fresh handle's."""
+    import torch
+
+    w = _case("long rows", "fp64")
+    vp, vs, rho = w.model_fn()
+    models = [(vp, vs, rho), (np.ascontiguousarray(vp[::-1]), vs, 0.97 * rho)]  # (of one largest vp: the layer's)
+    st = torch.cuda.Stream()
+    obs = None
+    out = []
+    g = pkg.Grid.from_workloads([w], stream=st)
+    for m in models:
+        f = pkg.Grid.from_workloads([dataclasses.replace(w, model_fn=lambda: m)], stream=st)
+        if obs is None:
+            f.step(w.steps)
+            obs = 0.9 * f.record(0)["_all"].astype(np.float64)
+        fresh = f.gradient(0, obs, w.steps)
+        f.close()
+        g.set_model(0, *m)
+        out.append((g.gradient(0, obs, w.steps), fresh))
+    g.close()
+    for (J, a), (K, b) in out:
+        assert J == K and J > 0
+        for k in ("vp", "rho"):
+            assert np.any(a[k]) and np.array_equal(a[k], b[k]), k
+    assert not np.array_equal(out[0][0][1]["rho"], out[1][0][1]["rho"])
