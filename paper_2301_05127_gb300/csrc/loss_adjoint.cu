@@ -394,9 +394,7 @@ loss_status_t run_gradient(loss_ctx* h, Shot& s, const double* d_obs, int32_t ch
     }
   } tmp{h};
   LOSS_TRY(dev_alloc(h, nobs * sizeof(double), &tmp.p[0]));
-  LOSS_TRY(dev_alloc(h, 3 * N * sizeof(double), &tmp.p[1]));
   double* obs = (double*)tmp.p[0];
-  double* out = (double*)tmp.p[1];
   // caller buffers are read and written in the order of the legacy default stream, whatever the handle's stream is (a
   // device-to-device cudaMemcpy does not wait for its end by itself)
   LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
@@ -422,6 +420,8 @@ loss_status_t run_gradient(loss_ctx* h, Shot& s, const double* d_obs, int32_t ch
   h->in_gradient = true;
   if (s.esize == 8) LOSS_TRY(gradient_t<double>(h, s, obs, C, n_steps, misfit));
   else LOSS_TRY(gradient_t<float>(h, s, obs, C, n_steps, misfit));
+  LOSS_TRY(dev_alloc(h, 3 * N * sizeof(double), &tmp.p[1]));  // (the checkpoints have gone)
+  double* out = (double*)tmp.p[1];
   LOSS_TRY(cuda_check(h, launch_chain(s.grad[0], s.grad[1], s.grad[2], s.dmodel, el ? 1 : 0, (int64_t)N, s.len[2], s.px,
                                       out, h->num_sms, h->stream), "chain rule"));
   LOSS_TRY(cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
