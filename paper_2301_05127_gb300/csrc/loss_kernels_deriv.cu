@@ -360,8 +360,11 @@ cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMa
     kern<<<col_blocks(cm, cm.warps), 32 * cm.warps, smem, st>>>(g, cm, op);
     return cudaGetLastError();
   };
-  if constexpr (sizeof(T) == 4)
+  if constexpr (sizeof(T) == 4) {
     if (d2) return go(DerivColOp<T, true>{f, d1, d2, s1, s2}, k_col<T, DerivColOp<T, true>>, col_smem<T>(1, cm.warps, true));
+  } else if (d2) {
+    return cudaErrorNotSupported;  // not built: the line kernel takes them (run_derivative_t)
+  }
   return go(DerivColOp<T, false>{f, d1, d1, s1, s2}, k_col<T, DerivColOp<T, false>>, col_smem<T>(1, cm.warps));
 }
 
