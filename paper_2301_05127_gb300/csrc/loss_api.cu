@@ -1221,7 +1221,10 @@ loss_status_t loss_derivative_adjoint(loss_handle_t h, int32_t shot, int32_t axi
   LOSS_TRY(get_shot(h, shot, &s));
   if (axis < 0 || axis >= s->dim) return fail(h, LOSS_E_ARG, "axis out of range");
   if (!g || !out || (mem != LOSS_MEM_HOST && mem != LOSS_MEM_DEVICE)) return fail(h, LOSS_E_ARG, "bad buffers");
-  return run_derivative_adjoint(h, *s, axis_slot(*s, axis), g, out, mem);
+  const int k = axis_slot(*s, axis);
+  // (the result is formed while g is read; an axis with knots takes its own kernels)
+  if (mem == LOSS_MEM_DEVICE && !s->nu_tab[k] && overlaps(*s, g, out)) return fail(h, LOSS_E_ARG, "out overlaps g");
+  return run_derivative_adjoint(h, *s, k, g, out, mem);
 }
 
 loss_status_t loss_gradient(loss_handle_t h, int32_t shot, const double* d_obs, int32_t checkpoint_every,

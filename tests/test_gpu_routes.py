@@ -159,3 +159,31 @@ def test_autotune_reports_what_runs(pkg, physics, prec):
     g.close()
     ref, _ = _steps(pkg, w, 5, shapes=[(k, r["threads_per_block"], r["chunk_log2"]) for k, r in res.items()])
     assert _same(got, ref)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("axis", [0, 1])
+def test_transpose_over_its_input(pkg, prec, axis):
+    """Device arrays that share memory are refused, the same host array twice is not."""
+    import ctypes
+
+    import torch
+
+    w = dataclasses.replace(_shot((64, 128), (1, 2), 12, prec, 5), receivers={})
+    g = pkg.Grid.from_workloads([w])
+    a = random_field(w.shape, 3, 4.0).astype(g.dtype)
+    ref = g.derivative_adjoint(0, axis, a)
+    f = pkg.lib().loss_derivative_adjoint
+    buf = torch.zeros(3 * a.size, dtype=torch.from_numpy(a).dtype, device="cuda")
+    buf[:a.size] = torch.from_numpy(a).reshape(-1).cuda()
+    torch.cuda.synchronize()
+    p, nb = buf.data_ptr(), a.nbytes
+    for out in (p, p + nb - a.itemsize):
+        assert f(g.h, 0, axis, ctypes.c_void_p(p), ctypes.c_void_p(out), pkg.LOSS_MEM_DEVICE) == pkg.LOSS_E_ARG
+    assert f(g.h, 0, axis, ctypes.c_void_p(p), ctypes.c_void_p(p + nb), pkg.LOSS_MEM_DEVICE) == pkg.LOSS_OK
+    g.sync()
+    assert np.array_equal(buf[a.size:2 * a.size].cpu().numpy().reshape(a.shape), ref)
+    b = a.copy()
+    assert f(g.h, 0, axis, b.ctypes.data, b.ctypes.data, pkg.LOSS_MEM_HOST) == pkg.LOSS_OK
+    assert np.array_equal(b, ref)
+    g.close()
