@@ -453,7 +453,7 @@ static loss_status_t derivative_adjoint_t(loss_ctx* h, Shot& s, int k, const T* 
       else cm = col_map(h->num_sms, s, k, sy, sz);
       LaunchScope ls(h, kid);
       const double sc = fir_const(ca.M).a * 3.0 / s.h[k];
-      return cuda_check(h, launch_trans_stream<T>(ca, cm, rm, k == 2, false, g, out, (T)sc, lo_part<T>(sc), h->stream),
+      return cuda_check(h, launch_trans_stream<T>(ca, cm, rm, k == 2, g, out, (T)sc, lo_part<T>(sc), h->stream),
                         "adjoint kernel");
     }
   }

@@ -326,8 +326,8 @@ template <typename T>
 cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, const T* f, T* d1, T* d2,
                                 T s1, T s2, cudaStream_t st);
 template <typename T>
-cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, bool acc, const T* in,
-                                T* out, T scale, T scale_lo, cudaStream_t st);
+cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, const T* in, T* out,
+                                T scale, T scale_lo, cudaStream_t st);
 // Whether the operators of axis slot k run on the engines: the derivative's tables fit the static array of
 // loss_derivative_noalloc (which launches the same kernels), and the dense array fits the engines' 32-bit offsets.
 constexpr size_t kNoAllocScratchBytes = 64 * 1024;
@@ -342,8 +342,7 @@ loss_status_t deriv_stream(loss_ctx* h, const Shot& s, int k, const ConvAxis& g,
 // loss_kernels_acstream.cu: 2-D acoustic step on the barrier-free engines
 template <typename T, bool KAHAN>
 cudaError_t launch_ac_rows(const AcXArgs<T>& a, const ConvAxis& g, const RowMap& rm, cudaStream_t st);
-template <typename T, bool K>
-cudaError_t launch_ac_cols(const AcZArgs<T>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st);
+cudaError_t launch_ac_cols(const AcZArgs<double>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st);
 template <typename T, bool K>
 void ac_batch_tables(const std::vector<AcStreamShot<T>>& shots, std::vector<unsigned char>& bytes, AcBatchKind (&k)[8]);
 template <typename T, bool K>

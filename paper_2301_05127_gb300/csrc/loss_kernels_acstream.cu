@@ -188,8 +188,10 @@ struct AcRowOp {
   }
 };
 
-template <typename T, bool KAHAN, int MODE, bool REC>
+// Columns, FP64 (the FP32 z part runs on the tiles).
+template <int MODE, bool REC>
 struct AcColOp {
+  using T = double;
   static constexpr int NF = 1;
   static constexpr bool SECOND = false;
   static constexpr int kBlocks = 4;
@@ -197,25 +199,14 @@ struct AcColOp {
   AcZArgs<T> a;
   int b_on, pad;
   struct Regs {
-    T v, b, m, c;
+    T v, b, m;
   };
   __device__ __forceinline__ const T* src(int) const { return MODE == 1 ? a.sigma : a.v3; }
   __device__ __forceinline__ void load(Regs& r, int pos, uint32_t o) const {
     if constexpr (MODE == 1) {
       r.v = at_off(a.v3, o);
-      if constexpr (KAHAN) r.c = at_off(a.cv3, o);
       if (b_on) r.b = at_off(a.b, o);
       if (a.pml && a.zA.in(pos)) r.m = at_off(a.psiz, o);
-    }
-  }
-  __device__ __forceinline__ void add(const Regs& r, uint32_t o, T delta) const {
-    if constexpr (KAHAN) {
-      float v = r.v, c = r.c;
-      kahan_add(v, c, delta);
-      at_off(a.v3, o) = v;
-      at_off(a.cv3, o) = c;
-    } else {
-      at_off(a.v3, o) = r.v + delta;
     }
   }
   __device__ __forceinline__ void apply(Regs& r, const T (&e)[1], int pos, uint32_t o, int, int) const {
@@ -235,13 +226,9 @@ struct AcColOp {
         at_off(a.dlt, o) = bb * (ih - T(0.5) * inc);
       }
       at_off(a.psiz, o) = m1;
-      add(r, o, b_on || sizeof(T) == 8 ? bb * inc : mulc(inc, a.b0, a.b0_lo));
-    } else if constexpr (sizeof(T) == 8) {
-      at_off(a.v3, o) = b_on ? fma(r.b * -(a.s3h * a.acoef), e[0], r.v) : fma(e[0], a.sc, r.v);
-    } else if (b_on) {
-      add(r, o, r.b * mulc(e[0], -(a.s3h * a.acoef), -(a.s3h * a.acoef_lo + a.s3h_lo * a.acoef)));
+      at_off(a.v3, o) = r.v + bb * inc;
     } else {
-      add(r, o, mulc(e[0], a.sc, a.sc_lo));
+      at_off(a.v3, o) = b_on ? fma(r.b * -(a.s3h * a.acoef), e[0], r.v) : fma(e[0], a.sc, r.v);
     }
   }
 };
@@ -306,19 +293,14 @@ cudaError_t launch_ac_rows(const AcXArgs<T>& a, const ConvAxis& g, const RowMap&
   return go_row<T>(g, rm, AcRowOp<T, KAHAN, false, false, true, false>{f, b_on, 0}, st);
 }
 // mode 1: Z1, mode 2: Z2.
-template <typename T, bool K>
-cudaError_t launch_ac_cols(const AcZArgs<T>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st) {
+cudaError_t launch_ac_cols(const AcZArgs<double>& a, const ConvAxis& g, const ColMap& cm, int mode, cudaStream_t st) {
   const int b_on = a.b ? 1 : 0;
-  AcZArgs<T> f = a;
+  AcZArgs<double> f = a;
   fill_unused(f);
-  if (mode == 2) return go_col<T>(g, cm, AcColOp<T, K, 2, false>{f, b_on, 0}, st);
-  if (a.pml && a.dlt) return go_col<T>(g, cm, AcColOp<T, K, 1, true>{f, b_on, 0}, st);
-  return go_col<T>(g, cm, AcColOp<T, K, 1, false>{f, b_on, 0}, st);
+  if (mode == 2) return go_col<double>(g, cm, AcColOp<2, false>{f, b_on, 0}, st);
+  if (a.pml && a.dlt) return go_col<double>(g, cm, AcColOp<1, true>{f, b_on, 0}, st);
+  return go_col<double>(g, cm, AcColOp<1, false>{f, b_on, 0}, st);
 }
-template cudaError_t launch_ac_cols<float, false>(const AcZArgs<float>&, const ConvAxis&, const ColMap&, int, cudaStream_t);
-template cudaError_t launch_ac_cols<float, true>(const AcZArgs<float>&, const ConvAxis&, const ColMap&, int, cudaStream_t);
-template cudaError_t launch_ac_cols<double, false>(const AcZArgs<double>&, const ConvAxis&, const ColMap&, int,
-                                                   cudaStream_t);
 template cudaError_t launch_ac_rows<float, false>(const AcXArgs<float>&, const ConvAxis&, const RowMap&, cudaStream_t);
 template cudaError_t launch_ac_rows<float, true>(const AcXArgs<float>&, const ConvAxis&, const RowMap&, cudaStream_t);
 template cudaError_t launch_ac_rows<double, false>(const AcXArgs<double>&, const ConvAxis&, const RowMap&,
@@ -340,9 +322,9 @@ static void with_kind(int kind, F&& f) {
     switch (kind) {
       case 0: return f(RowJob<D, AcRowOp<D, K, false, true, true, true>>{});
       case 1: return f(RowJob<D, AcRowOp<D, K, true, true, true, true>>{});
-      case 5: return f(ColJob<D, AcColOp<D, false, 1, false>>{});
-      case 6: return f(ColJob<D, AcColOp<D, false, 1, true>>{});
-      default: return f(ColJob<D, AcColOp<D, false, 2, false>>{});
+      case 5: return f(ColJob<D, AcColOp<1, false>>{});
+      case 6: return f(ColJob<D, AcColOp<1, true>>{});
+      default: return f(ColJob<D, AcColOp<2, false>>{});
     }
   }
 }

@@ -1,5 +1,5 @@
 // sm_103a kernels of the stand-alone derivative operators (first and second derivative, transpose) on the barrier-free
-// engines of loss_stream.cuh, dense arrays, and of the FP64 adjoint terms built from them.
+// engines of loss_stream.cuh, dense arrays.
 //
 // The transpose of e = (R - L) + sum_j D_j r^|i - q_j| (D_j = sum_m w_jm f_{q_j + m}; times 3 a / h):
 //   out_i = L_i - R_i (zeros beyond the ends, odd reflection transposed) + sum_j w_j,i-q_j Dbar_j,
@@ -29,17 +29,16 @@ struct DerivRowOp {
   T* d1;
   T* d2;
   T s1, s2;
-  int vec, pad;
   __device__ __forceinline__ const T* src(int) const { return f; }
   __device__ __forceinline__ void chunk(T (&e)[1][9], int, int len, int64_t gi, int) const {
 #pragma unroll
     for (int j = 0; j < 9; ++j) e[0][j] *= s1;
-    st9(d1 + gi, vec, len, e[0]);
+    st9(d1 + gi, false, len, e[0]);
   }
   __device__ __forceinline__ void chunk2nd(T (&v)[9], int, int len, int64_t gi) const {
 #pragma unroll
     for (int j = 0; j < 9; ++j) v[j] *= s2;
-    st9(d2 + gi, vec, len, v);
+    st9(d2 + gi, false, len, v);
   }
 };
 template <typename T, bool D2>
@@ -100,9 +99,9 @@ __device__ __forceinline__ TransD<T> trans_junction(const ConvAxis& g, int j, co
   return trans_sum(at_off(f, o + (uint32_t)q * sb), r * (a + b));
 }
 
-// out (+)= scale * transpose along rows.  ACC: add to out.
-template <typename T, bool ACC>
-__global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, const T* __restrict__ in, T* out,
+// out = scale * transpose along rows.
+template <typename T>
+__global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, const T* __restrict__ in, T* __restrict__ out,
                                                       T scale, T scale_lo) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ T rs[kReach];
@@ -135,7 +134,7 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
     T e[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) e[j] = T(0);
-    if (len > 0) ld9(in + gi, rm.vec, len, e);
+    if (len > 0) ld9(in + gi, false, len, e);
     int j0 = 0, nj = 0;
     if (g.ntaps) {
       const int lo = 8 * o0, hi = o1 == rm.nch ? g.n : 8 * o1 - 1;
@@ -184,20 +183,14 @@ __global__ void __launch_bounds__(128, 4) k_row_trans(ConvAxis g, RowMap rm, con
       }
 #pragma unroll
       for (int j = 0; j < 9; ++j) e[j] = mulc(e[j], scale, scale_lo);
-      if constexpr (ACC) {
-        T u[9];
-        ld9(out + gi, rm.vec, len, u);
-#pragma unroll
-        for (int j = 0; j < 9; ++j) e[j] += u[j];
-      }
-      st9(out + gi, rm.vec, len, e);
+      st9(out + gi, false, len, e);
     }
   }
 }
 
-// out (+)= scale * transpose along strided lines, marched as k_col.
-template <typename T, bool ACC>
-__global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, const T* __restrict__ in, T* out,
+// out = scale * transpose along strided lines, marched as k_col.
+template <typename T>
+__global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, const T* __restrict__ in, T* __restrict__ out,
                                                       T scale, T scale_lo) {
   constexpr int W = Conv<T>::W, NR = W + 2, NJ = 4;
   constexpr T r = (T)kConvR, r8 = (T)conv_pow(8), r16 = (T)conv_pow(16);
@@ -323,20 +316,15 @@ __global__ void __launch_bounds__(128, 4) k_col_trans(ConvAxis g, ColMap cm, con
       }
     }
     const int len = min(8, s1 - p0);
-    T u[8];
-    if constexpr (ACC) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) u[j] = at_off(out, base + (uint32_t)min(p0 + j, n) * sb);
-    }
     if (valid)
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (j < len) at_off(out, base + (uint32_t)(p0 + j) * sb) = (ACC ? u[j] : T(0)) + mulc(e[j], scale, scale_lo);
+        if (j < len) at_off(out, base + (uint32_t)(p0 + j) * sb) = mulc(e[j], scale, scale_lo);
   }
   cp_async_wait<0>();
 }
 
-// Derivatives of a dense or pitched array (rm.vec: rows are 16-byte aligned and padded).  x: rows, else lines.
+// Derivatives of a dense array.  x: rows (no alignment is known), else lines.
 template <typename T>
 cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, const T* f, T* d1, T* d2,
                                 T s1, T s2, cudaStream_t st) {
@@ -350,8 +338,8 @@ cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMa
       kern<<<row_blocks(rm, decltype(op)::kBlocks, rm.warps), 32 * rm.warps, smem, st>>>(g, rm, op);
       return cudaGetLastError();
     };
-    if (d2) return go(DerivRowOp<T, true>{f, d1, d2, s1, s2, rm.vec, 0}, k_row<T, DerivRowOp<T, true>>);
-    return go(DerivRowOp<T, false>{f, d1, d1, s1, s2, rm.vec, 0}, k_row<T, DerivRowOp<T, false>>);
+    if (d2) return go(DerivRowOp<T, true>{f, d1, d2, s1, s2}, k_row<T, DerivRowOp<T, true>>);
+    return go(DerivRowOp<T, false>{f, d1, d1, s1, s2}, k_row<T, DerivRowOp<T, false>>);
   }
   auto go = [&](auto op, auto kern, size_t smem) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -369,11 +357,11 @@ cudaError_t launch_deriv_stream(const ConvAxis& g, const ColMap& cm, const RowMa
 }
 
 template <typename T>
-cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, bool acc, const T* in,
-                                T* out, T scale, T scale_lo, cudaStream_t st) {
+cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMap& rm, bool x, const T* in, T* out, T scale,
+                                T scale_lo, cudaStream_t st) {
   if (x) {
     const size_t smem = (size_t)rm.warps * rm.wbytes;
-    auto kern = acc ? k_row_trans<T, true> : k_row_trans<T, false>;
+    auto kern = k_row_trans<T>;
     if (smem > 32 * 1024) {
       const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
       if (e != cudaSuccess) return e;
@@ -382,7 +370,7 @@ cudaError_t launch_trans_stream(const ConvAxis& g, const ColMap& cm, const RowMa
     return cudaGetLastError();
   }
   const size_t smem = col_smem<T>(1, cm.warps);
-  auto kern = acc ? k_col_trans<T, true> : k_col_trans<T, false>;
+  auto kern = k_col_trans<T>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)col_smem<T>(1, 4, true));
   if (e != cudaSuccess) return e;
@@ -394,9 +382,9 @@ template cudaError_t launch_deriv_stream<float>(const ConvAxis&, const ColMap&, 
                                                 float*, float, float, cudaStream_t);
 template cudaError_t launch_deriv_stream<double>(const ConvAxis&, const ColMap&, const RowMap&, bool, const double*,
                                                  double*, double*, double, double, cudaStream_t);
-template cudaError_t launch_trans_stream<float>(const ConvAxis&, const ColMap&, const RowMap&, bool, bool, const float*,
-                                                float*, float, float, cudaStream_t);
-template cudaError_t launch_trans_stream<double>(const ConvAxis&, const ColMap&, const RowMap&, bool, bool,
-                                                 const double*, double*, double, double, cudaStream_t);
+template cudaError_t launch_trans_stream<float>(const ConvAxis&, const ColMap&, const RowMap&, bool, const float*, float*,
+                                                float, float, cudaStream_t);
+template cudaError_t launch_trans_stream<double>(const ConvAxis&, const ColMap&, const RowMap&, bool, const double*, double*,
+                                                 double, double, cudaStream_t);
 
 }  // namespace lossk

@@ -271,16 +271,19 @@ static loss_status_t acs_rows(loss_ctx* h, Shot& s, int do_B, double acoef, doub
   LaunchScope ls(h, LOSS_KERNEL_ACOUSTIC_X);
   return cuda_check(h, launch_ac_rows<T, K>(a, g, row_map(h->num_sms, s, 1, g, s.sy, s.sz, true), h->stream), "acoustic x kernel");
 }
-// Z1 (mode 1) or Z2 (mode 2) of the FP64 step on the engines.
-template <typename T, bool K>
+// Z1 (mode 1) or Z2 (mode 2) of the FP64 step on the engines (acs_ok: FP64 only).
+template <typename T>
 static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
-  ConvAxis g;
-  bool ok;
-  LOSS_TRY(conv_axis(h, s, 0, &g, &ok));
-  AcZArgs<T> a = ac_z_args<T>(h, s, LineGeom{}, acoef, 0);
-  conv_scale(a, s, 0, acoef);
-  LaunchScope ls(h, mode == 1 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2);
-  return cuda_check(h, launch_ac_cols<T, K>(a, g, col_map(h->num_sms, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
+  if constexpr (sizeof(T) == 8) {
+    ConvAxis g;
+    bool ok;
+    LOSS_TRY(conv_axis(h, s, 0, &g, &ok));
+    AcZArgs<T> a = ac_z_args<T>(h, s, LineGeom{}, acoef, 0);
+    conv_scale(a, s, 0, acoef);
+    LaunchScope ls(h, mode == 1 ? LOSS_KERNEL_ACOUSTIC_Z : LOSS_KERNEL_ACOUSTIC_Z2);
+    return cuda_check(h, launch_ac_cols(a, g, col_map(h->num_sms, s, 0, s.sy, s.sz), mode, h->stream), "acoustic z kernel");
+  }
+  return LOSS_E_UNSUPPORTED;
 }
 
 // Whether the FP32 rows of this shot that the pipelined kernel would take run on the row engine: rows of at least 513
@@ -391,8 +394,8 @@ static loss_status_t acoustic2d_start(loss_ctx* h, Shot& s) {
   LOSS_TRY(acs_ok(h, s, &stream));
   if (stream) {
     LOSS_TRY((acs_rows<T, K>(h, s, 0, 0.5 * dt, 0.0)));
-    LOSS_TRY((acs_cols<T, K>(h, s, 1, 0.5 * dt)));
-    return acs_cols<T, K>(h, s, 2, 0.0);
+    LOSS_TRY((acs_cols<T>(h, s, 1, 0.5 * dt)));
+    return acs_cols<T>(h, s, 2, 0.0);
   }
   LOSS_TRY((ac_x<T, K>(h, s, 0, 0.5 * dt, 0.0)));
   return ac_z<T, K>(h, s, 0.5 * dt, 1);
@@ -438,8 +441,8 @@ static loss_status_t acoustic2d_step(loss_ctx* h, Shot& s) {
     LOSS_TRY(tz<K>(h, s, 1, dt));
     LOSS_TRY(tz<K>(h, s, 2, 0.0));
   } else if (stream) {
-    LOSS_TRY((acs_cols<T, K>(h, s, 1, dt)));
-    LOSS_TRY((acs_cols<T, K>(h, s, 2, 0.0)));
+    LOSS_TRY((acs_cols<T>(h, s, 1, dt)));
+    LOSS_TRY((acs_cols<T>(h, s, 2, 0.0)));
   } else {
     LOSS_TRY((ac_z<T, K>(h, s, dt, 1)));
   }
@@ -463,7 +466,7 @@ static loss_status_t acoustic2d_unstagger(loss_ctx* h, Shot& s) {
   LOSS_TRY(acs_ok(h, s, &stream));
   if (stream) {
     LOSS_TRY((acs_rows<T, K>(h, s, 0, -0.5 * dt, 0.0)));
-    LOSS_TRY((acs_cols<T, K>(h, s, 1, -0.5 * dt)));
+    LOSS_TRY((acs_cols<T>(h, s, 1, -0.5 * dt)));
     s.staggered = false;
     return LOSS_OK;
   }
