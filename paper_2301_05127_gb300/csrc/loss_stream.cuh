@@ -20,8 +20,9 @@
 // below the working precision (host rule conv_axis in loss_step.cu); longer patches make the second term of the
 // patch-end correction, r^M D, vanish by the same rule.
 //
-// Every address formed here is a readable one, whatever the predicate it stands under: offsets are clamped to their line
-// or row, and pointers that a launch lacks are replaced on the host or excluded by a template parameter.
+// Accesses: loads outside a predicate have their offsets clamped to their line or row; the ring's copies and the stores
+// stand under the predicate that their position lies on the line (their offsets may lie past it, and are not used
+// then).  Pointers that a launch lacks are replaced on the host or excluded by a template parameter.
 #pragma once
 
 #include <cstdint>
