@@ -865,6 +865,7 @@ __global__ void __launch_bounds__(256, 2) k_xp_batch(const XpShot* __restrict__ 
   const PlainLayout lay{};
   float* base = reinterpret_cast<float*>(sm);
   xp_init_barriers(bar);
+  __syncthreads();  // no thread waits on a barrier that is not one yet (what an earlier kernel left in its place)
   float* TAB = base + L.TAB;
   float* dlf = base + L.DL;  // junction corrections, 65 per group
   auto desc = [&](int s) -> const XpShot& { return *reinterpret_cast<const XpShot*>(slot[s & 1]); };

@@ -187,3 +187,18 @@ def test_transpose_over_its_input(pkg, prec, axis):
     assert f(g.h, 0, axis, b.ctypes.data, b.ctypes.data, pkg.LOSS_MEM_HOST) == pkg.LOSS_OK
     assert np.array_equal(b, ref)
     g.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_kahan"])
+def test_short_rows_after_the_row_engine(pkg, prec):
+    """A batch whose pipelined x kernel has blocks of several warps (rows of 257 to 512 points, two groups of rows in a
+    block, blocks that go from one shot to the next) and follows the row kernel's launches of the long shots."""
+    sizes = [(12, 64), (4, 64), (5, 64), (7, 64), (4, 96), (9, 96), (4, 64)]
+    ws = [_shot((512, k * m), (4, k), 12, prec, 80 + i) for i, (k, m) in enumerate(sizes)]
+    ref, _ = _run(pkg, ws, batched=False)
+    for graph in (0, 3):
+        got, counts = _run(pkg, ws, graph=graph, chunks=(3, 9))
+        again, _ = _run(pkg, ws, graph=graph)
+        assert counts["acoustic_x"] == 27
+        assert all(_same(a, b) for a, b in zip(again, ref)), graph
+        assert np.isfinite(got[0][0]).all()
