@@ -74,7 +74,7 @@ struct AcRowOp {
 #pragma unroll
       for (int j = 0; j < 9; ++j) {
         if (j == 8 && len < 9) break;
-        gz[j] = mulc(gz[j], a.dt, a.dt_lo);
+        gz[j] = mulc1(gz[j], a.dt, a.dt_lo);
       }
     }
     if (lay) {
@@ -82,8 +82,8 @@ struct AcRowOp {
 #pragma unroll
       for (int j = 0; j < 9; ++j) {
         if (j == 8 && len < 9) break;
-        if (j < len && a.xB.in(p0 + j)) e[j] = -flow(a.xB.tab, n1, min(p0 + j, a.xB.n), mulc(e[j], a.s3h, a.s3h_lo), mx[j]);
-        else e[j] = mulc(e[j], a.sdt, a.sdt_lo);
+        if (j < len && a.xB.in(p0 + j)) e[j] = -flow(a.xB.tab, n1, min(p0 + j, a.xB.n), mulc1(e[j], a.s3h, a.s3h_lo), mx[j]);
+        else e[j] = mulc1(e[j], a.sdt, a.sdt_lo);
       }
       st9(a.phix + gi, true, len, mx);
 #pragma unroll
@@ -96,7 +96,7 @@ struct AcRowOp {
       for (int j = 0; j < 9; ++j) {
         if (j == 8 && len < 9) break;
         if constexpr (sizeof(T) == 8) e[j] = fma(e[j], a.sdt, gz[j]);
-        else e[j] = mulc(e[j], a.sdt, a.sdt_lo) + gz[j];
+        else e[j] = mulc1(e[j], a.sdt, a.sdt_lo) + gz[j];
       }
     }
     // e = minus the divergence's increment: sigma += -kappa e (+ source)
@@ -151,21 +151,21 @@ struct AcRowOp {
       if (j == 8 && len < 9) break;
       if (lay && j < len && a.xA.in(p0 + j)) {
         const int n1 = a.xA.n + 1, i = min(p0 + j, a.xA.n);
-        const T g = mulc(e[j], a.s3h, a.s3h_lo), m0 = m[j];
+        const T g = mulc1(e[j], a.s3h, a.s3h_lo), m0 = m[j];
         e[j] = flow(a.xA.tab, n1, i, g, m[j]);
         if constexpr (REC) {
           T mh = m0;
           const T ih = flow(a.xA.tabh, n1, i, g, mh);
           a.dlt[gi + j] = (b_on ? bb[j] : a.b0) * (ih - T(0.5) * e[j]);
         }
-        e[j] = b_on ? bb[j] * e[j] : mulc(e[j], a.b0, a.b0_lo);
+        e[j] = b_on ? bb[j] * e[j] : mulc1(e[j], a.b0, a.b0_lo);
       } else if (b_on) {
-        e[j] = bb[j] * mulc(e[j], a.sa, a.sa_lo);
+        e[j] = bb[j] * mulc1(e[j], a.sa, a.sa_lo);
       } else if constexpr (sizeof(T) == 8) {
         v[j] = fma(e[j], a.sc, v[j]);
         e[j] = T(0);
       } else {
-        e[j] = mulc(e[j], a.sc, a.sc_lo);
+        e[j] = mulc1(e[j], a.sc, a.sc_lo);
       }
     }
     if (lay) st9(a.psix + gi, true, len, m);

@@ -214,11 +214,15 @@ static bool xp_ok(const loss_ctx* h, const Shot& s, const TileGeom& t) {
          xp_smem(t, s.kahan) + 2048 <= (size_t)h->smem_optin;
 }
 
-// Arguments with the engines' derivative scale 3 a / h (they return e / a).
+// Arguments with the engines' derivative scale 3 a / h (they return e / a).  FP32 recursions run with r rounded to FP32; their
+// sums over a smooth line, 2 f' / (1 - r)^2, are off by a common factor (2e-9), a wave speed error that adds up over
+// thousands of steps, and the scale takes it out.  With that and coefficients that round a product once (mulc1), 2000 steps
+// of 2049^2 with Kahan summation: traces 1.51e-7 -> 1.10e-7 from the oracle's, fields 1.95e-6 -> 1.43e-6.
 template <class A>
 static void conv_scale(A& a, const Shot& s, int k, double acoef) {
   using T = decltype(a.s3h);
-  const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k];
+  const double q = (1.0 - (double)(T)kConvRHost) / (1.0 - kConvRHost);
+  const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k] * (q * q);
   a.s3h = (T)sc;
   a.s3h_lo = lo_part<T>(sc);
   a.sc = (T)(-acoef * s.b0 * sc);
@@ -289,8 +293,10 @@ static loss_status_t acs_cols(loss_ctx* h, Shot& s, int mode, double acoef) {
 // Whether the FP32 rows of this shot that the pipelined kernel would take run on the row engine: rows of at least 513
 // points that qualify, in the convolution family, outside gradients.  Other shots of the handle and the length of the
 // pipelined kernel's waits have no part in it; only a limit of 0 polls, which fails the run, keeps the kernel that
-// waits.  x part, engine against pipelined kernel: 513^2 19.9 / 21.7 us, 1025^2 28.9 / 33.8 us, 2049^2 51.4 / 62.4 us, with
-// Kahan summation 61.4 / 67.0 us; rows of 257 points and less are bound by launches either way.
+// waits.  x part, engine against pipelined kernel, in FP32 (with Kahan summation): 129^2 14.4 (14.3) / 17.4 (18.3) us, 257^2
+// 14.4 / 18.5 (18.8), 321^2 19.2 (19.9) / 20.5 (20.6), 449^2 20.1 (19.4) / 20.4 (20.6), 505^2 19.1 / 22.7 (23.6), 513^2 19.9 /
+// 21.7, 1025^2 28.9 / 33.8, 2049^2 51.4 / 62.4 (63.4 / 67.0).  The gain is clear from 505 points on and small between 321 and
+// 449; shorter rows would gain a launch's latency on the engine too and are left where they are, with their bits.
 static loss_status_t rows_on_engine(loss_ctx* h, Shot& s, bool* on) {
   *on = false;
   if (h->tiled == LOSS_KERNELS_CONVOLUTION_ITEMS || h->in_gradient || h->wait_polls == 0) return LOSS_OK;

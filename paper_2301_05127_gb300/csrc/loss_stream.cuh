@@ -63,6 +63,13 @@ __device__ __forceinline__ const ConvTap* stage_taps(const ConvAxis& g, ConvTap*
   return tsm;
 }
 
+// x (c + c_lo) rounded once, c_lo x aside (mulc rounds c x first, and c_lo is lost unless c_lo x exceeds half a unit of that).
+template <typename T>
+__device__ __forceinline__ T mulc1(T x, T c, T c_lo) {
+  if constexpr (sizeof(T) == 8) return c * x;
+  else return fmaf(c, x, c_lo * x);
+}
+
 // Element at a byte offset below 4 GB from a (uniform) base: one 32-bit offset serves every array of a pass.
 template <typename T>
 __device__ __forceinline__ T& at_off(T* p, uint32_t o) {
