@@ -282,13 +282,14 @@ loss_status_t loss_set_schedule(loss_handle_t handle, int32_t batched, int32_t g
  * LOSS_KERNELS_CONVOLUTION (the default) = the truncated-convolution form: the same patch systems solved through
  * the closed-form inverse of the (1, 4, 1) operator, truncated where |sqrt(3) - 2|^k < 1e-9, with exact patch-end
  * corrections from the PMBC junction values (x rows pipelined through TMA bulk copies, z lines on independent
- * 32-column x one-patch tiles; rows the pipelined kernel does not take, longer than 2049 points or with patches
- * whose length is not a multiple of 8, go to independent (row, patch) items in two launches);
- * LOSS_KERNELS_CONVOLUTION_ITEMS = the same with every row on (row, patch) items.  In the convolution family FP32 3-D
- * elastic steps, FP32 rows of 513 points and more and rows that the pipelined kernel does not take, and in both families
+ * 32-column x one-patch tiles);
+ * LOSS_KERNELS_CONVOLUTION_ITEMS = the same with every FP32 row on independent (row, patch) items, two launches.
+ * In the convolution family FP32 3-D elastic steps, FP32 rows of 513 points and more and rows that the pipelined kernel
+ * does not take (longer than 4097 points, or with patches whose length is not a multiple of 8), and in both families
  * FP64 2-D and 3-D elastic steps, run on column and row kernels that march lines and rows without block barriers, where
- * patches are long enough for them (at least 8 points more than a junction's correction reaches, 40 points per axis)
- * and arrays hold at most 4 GB.  All agree with the FP64 oracle
+ * patches are long enough for them (at least 8 points more than a junction's correction reaches, 40 points per axis),
+ * arrays hold at most 4 GB and no launch shape is asked for (loss_set_launch).  FP32 rows that neither those nor the
+ * pipelined kernel take go to items.  All agree with the FP64 oracle
  * at the FP32 tolerance; they differ in rounding.  LOSS_E_ARG for another value. */
 enum { LOSS_KERNELS_LINE = 0, LOSS_KERNELS_CONVOLUTION = 1, LOSS_KERNELS_CONVOLUTION_ITEMS = 2 };
 loss_status_t loss_set_kernels(loss_handle_t handle, int32_t family);

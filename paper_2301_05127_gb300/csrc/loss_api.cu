@@ -1400,8 +1400,9 @@ static loss_status_t run_derivative_t(loss_ctx* h, Shot& s, int k, const T* f, T
   LOSS_TRY(line_geom(h, s, k, sz, sy, &g, &logc, &threads, d2 ? 3 : 2, 0, h->lines_per_block[LOSS_KERNEL_DERIVATIVE],
                      h->chunk_log2[LOSS_KERNEL_DERIVATIVE], h->tile_threads[LOSS_KERNEL_DERIVATIVE]));
   // A launch shape asked for (loss_set_launch, loss_set_tile) is one of the line kernel's, and only that kernel reads
-  // a whole line before it writes one.  FP64 second derivatives along columns stay there too: the second recurrence
-  // costs more arithmetic than the line kernel's elimination shares (257^3: 837 us on the engine, 801 us there).
+  // a whole line before it writes one.  FP64 second derivatives along columns stay there too, engine against line kernel:
+  // 129^2 51 / 33 us, 513^2 52 / 34, 65^3 64 / 38, 257^3 847 / 807 (the second recurrence lengthens a column's serial chain and
+  // its arithmetic); 1025^2 63 / 68, 2049^2 215 / 276 and 129^3 114 / 136 would be faster on the engine.
   const int kid = LOSS_KERNEL_DERIVATIVE;
   if (d1 && !phi && !(d2 && s.esize == 8 && k != 2) && !overlaps(s, f, d1) && !overlaps(s, f, d2) && h->lines_per_block[kid] <= 0 && h->tile_threads[kid] <= 0 && h->chunk_log2[kid] <= 0) {
     ConvAxis ca;

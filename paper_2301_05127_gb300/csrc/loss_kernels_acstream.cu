@@ -9,8 +9,8 @@
 // The FP64 line kernels held whole lines of one block behind seven barriers per derivative and spent 11 FP64 operations
 // per point and derivative; FP64 runs at 2 FMA per SM and clock here, so operations are what the step costs.  These spend
 // about 5 (two warm-up sums, two recursions, one difference) plus the pointwise update: 1025^2 step 251 us -> 175 us.
-// 129^2 (154 us -> 90 us) waits for the serial FP64 chain of a line's chunks.  FP32 rows are bound by issue slots and
-// latency (2049^2 x part with Kahan summation 67 us on the pipelined kernel, 61 us here, 44 bytes a point).
+// 129^2 (154 us -> 92 us) waits for the serial FP64 chain of a line's chunks.  FP32 rows are bound by issue slots and
+// latency (2049^2 x part with Kahan summation 67 us on the pipelined kernel, 63 us here, 44 bytes a point).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -8,8 +8,8 @@
 //
 // Memory bound: one read and one write of the array per output (257^3 FP32: 136 MB).  The line kernel they replace
 // (k_deriv, k_adj: whole lines staged in shared memory between barriers, a block's loads, elimination and stores in
-// turn) took 1.75 ms for first and second derivatives and transposes along the axes of a 257^3 FP32 array that these do in 0.60 ms (with the host between); 129^2 FP64 operators,
-// which launches bound, 95 us -> 88 us.  The line kernel stays for PMBC values, short patches, arrays beyond 32-bit
+// turn) took 1.75 ms for first and second derivatives and transposes along the axes of a 257^3 FP32 array that these do in
+// 0.57 ms (with the host between); 129^2 FP64 operators, which launches bound, 95 us -> 80 us.  The line kernel stays for PMBC values, short patches, arrays beyond 32-bit
 // offsets, arrays written over their input, and launch shapes that the caller asked for.
 #include <cuda_runtime.h>
 
