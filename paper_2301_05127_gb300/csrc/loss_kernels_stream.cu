@@ -74,7 +74,7 @@ struct ElColOp {
     T g[3];
     if (a.pml && a.pB.in(pos)) {
 #pragma unroll
-      for (int f = 0; f < 3; ++f) g[f] = mulc(e[f], a.s3h, a.s3h_lo);
+      for (int f = 0; f < 3; ++f) g[f] = mulc1(e[f], a.s3h, a.s3h_lo);
       // the exact sub-flow (PmlAxis::step) on the memory values loaded ahead
       const PmlAxis<T>& pa = kStress ? a.pB : a.pA;
       const int n1 = pa.n + 1;
@@ -101,7 +101,7 @@ struct ElColOp {
       }
     } else {
 #pragma unroll
-      for (int f = 0; f < 3; ++f) g[f] = mulc(e[f], a.st, a.st_lo);
+      for (int f = 0; f < 3; ++f) g[f] = mulc1(e[f], a.st, a.st_lo);
     }
     if constexpr (PASS == ES_BY) {
       at_off(t[1], o) = r.t[0] + g[0];
@@ -113,8 +113,8 @@ struct ElColOp {
     } else if constexpr (PASS == ES_BZ) {
       const T xa = r.t[0], tb = r.t[1], tc = r.t[2], xd = r.t[3], te = r.t[4];
       // constant moduli enter through mulc (their rounding errors would bias every update the same way)
-      auto mlam = [&](T v) { return lam_on ? r.m0 * v : mulc(v, a.lam0, a.lam0_lo); };
-      auto mmu = [&](T v) { return mu_on ? r.m1 * v : mulc(v, a.mu0, a.mu0_lo); };
+      auto mlam = [&](T v) { return lam_on ? r.m0 * v : mulc1(v, a.lam0, a.lam0_lo); };
+      auto mmu = [&](T v) { return mu_on ? r.m1 * v : mulc1(v, a.mu0, a.mu0_lo); };
       const T ltr = mlam(xa + xd + g[2]);
       T s11 = ltr + T(2) * mmu(xa), s22 = ltr + T(2) * mmu(xd), s33 = ltr + T(2) * mmu(g[2]);
       T s13 = mmu(tc + g[0]);
@@ -140,7 +140,7 @@ struct ElColOp {
         if ((unsigned)dz < 25u && (unsigned)dy < 25u && (unsigned)dx < 25u)
           force = source_at(dz, dy, dx);
       }
-      auto mb = [&](T v) { return b_on ? r.m0 * v : mulc(v, a.b0, a.b0_lo); };
+      auto mb = [&](T v) { return b_on ? r.m0 * v : mulc1(v, a.b0, a.b0_lo); };
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
         const T ff = (a.force_mask & (1 << f)) ? force : T(0);
@@ -187,7 +187,7 @@ struct ElRowOp {
           T x[3];
 #pragma unroll
           for (int f = 0; f < 3; ++f) {
-            const T g = mulc(e[f][j], a.s3h, a.s3h_lo);
+            const T g = mulc1(e[f][j], a.s3h, a.s3h_lo);
             const T m1 = T0 * m[f][j] - T1 * g;
             x[f] = -(T2 * (m1 - m[f][j]) - T3 * g);
             if constexpr (REC) {
@@ -200,7 +200,7 @@ struct ElRowOp {
           }
         } else {
 #pragma unroll
-          for (int f = 0; f < 3; ++f) e[f][j] = mulc(e[f][j], a.st, a.st_lo);
+          for (int f = 0; f < 3; ++f) e[f][j] = mulc1(e[f][j], a.st, a.st_lo);
         }
       }
 #pragma unroll
@@ -211,7 +211,7 @@ struct ElRowOp {
 #pragma unroll
         for (int j = 0; j < 9; ++j) {
           if (j == 8 && len < 9) break;
-          e[f][j] = mulc(e[f][j], a.st, a.st_lo);
+          e[f][j] = mulc1(e[f][j], a.st, a.st_lo);
         }
     }
 #pragma unroll

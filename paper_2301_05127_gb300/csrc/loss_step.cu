@@ -214,15 +214,22 @@ static bool xp_ok(const loss_ctx* h, const Shot& s, const TileGeom& t) {
          xp_smem(t, s.kahan) + 2048 <= (size_t)h->smem_optin;
 }
 
-// Arguments with the engines' derivative scale 3 a / h (they return e / a).  FP32 recursions run with r rounded to FP32; their
+// Derivative scale of the engines' steps, 3 a / h (they return e / a).  FP32 recursions run with r rounded to FP32; their
 // sums over a smooth line, 2 f' / (1 - r)^2, are off by a common factor (2e-9), a wave speed error that adds up over
 // thousands of steps, and the scale takes it out.  With that and coefficients that round a product once (mulc1), 2000 steps
-// of 2049^2 with Kahan summation: traces 1.51e-7 -> 1.10e-7 from the oracle's, fields 1.95e-6 -> 1.43e-6.
+// of 2049^2 with Kahan summation: traces 1.51e-7 -> 1.10e-7 from the oracle's, fields 1.95e-6 -> 1.43e-6; 1000 elastic ones
+// of 257^3: 2.38e-6 -> 1.13e-6, 2.08e-6 -> 6.0e-7.
+template <typename T>
+static double engine_scale(const Shot& s, int k) {
+  const double q = (1.0 - (double)(T)kConvRHost) / (1.0 - kConvRHost);
+  return fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k] * (q * q);
+}
+
+// Arguments with that scale.
 template <class A>
 static void conv_scale(A& a, const Shot& s, int k, double acoef) {
   using T = decltype(a.s3h);
-  const double q = (1.0 - (double)(T)kConvRHost) / (1.0 - kConvRHost);
-  const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k] * (q * q);
+  const double sc = engine_scale<T>(s, k);
   a.s3h = (T)sc;
   a.s3h_lo = lo_part<T>(sc);
   a.sc = (T)(-acoef * s.b0 * sc);
@@ -789,7 +796,7 @@ static loss_status_t els_pass(loss_ctx* h, Shot& s, int pass, double acoef, doub
   const bool B = pass == ES_BX || pass == ES_BY || pass == ES_BZ;
   const int src = B ? 0 : (pass == ES_AZ ? 1 : (pass == ES_AX ? 2 : 3));
   ElArgs<T> a = el_args<T>(h, s, k, src, B ? 1 : 0, B ? 0 : 1, acoef, amp);
-  const double sc = fir_const((int)(s.n[k] / s.p[k])).a * 3.0 / s.h[k];  // the engines return e / a
+  const double sc = engine_scale<T>(s, k);
   a.s3h = (T)sc;
   a.s3h_lo = lo_part<T>(sc);
   const double tau = B ? s.d.dt : acoef;
