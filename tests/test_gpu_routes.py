@@ -202,3 +202,26 @@ def test_short_rows_after_the_row_engine(pkg, prec):
         assert counts["acoustic_x"] == 27
         assert all(_same(a, b) for a, b in zip(again, ref)), graph
         assert np.isfinite(got[0][0]).all()
+
+
+@pytest.mark.parametrize("physics,kernel", [("acoustic", "acoustic_z"), ("elastic", "elastic_x")])
+@pytest.mark.parametrize("graph", [0, 2])
+def test_shape_set_between_steps(pkg, physics, kernel, graph):
+    """A launch shape set and taken back between steps moves the run to the other kernels and back: the fields stay those
+    of the run without it, to the tolerance of the FP64 form."""
+    w = _engine_workload(physics, "fp64")
+    out = []
+    for shapes in ([None] * 3, [None, (128, 4), (0, 0)]):
+        g = pkg.Grid.from_workloads([w])
+        g.set_schedule(True, graph)
+        for s in shapes:
+            if s is not None:
+                g.set_tile(kernel, *s)
+            g.step(4)
+        out.append([g.get_field(0, f) for f in (FIELDS if physics == "acoustic" else ELASTIC)])
+        g.close()
+    assert not _same(*out)
+    names = FIELDS if physics == "acoustic" else ELASTIC
+    for f, a, b in zip(names, *out):  # against the largest field of its kind (velocities, stresses)
+        scale = max(np.linalg.norm(x) for k, x in zip(names, out[0]) if k[0] == f[0])
+        assert np.linalg.norm(a - b) <= 1e-12 * scale, f
